@@ -463,9 +463,10 @@ hicops_status hicops_index_copy_csr(const hicops_index* index, uint64_t* off, ui
 /* Launch shape of the search kernel (the paper's R/I/K balancing of
  * superstep 3 becomes the choice of how spectra and peptide ranges map onto
  * persistent CTAs).  Zero fields take the default.  threads: CTA size, 256,
- * 384 or 512 (default 384 for top_k <= 16, else 256).  chunk_entries: index entries a CTA aims to accumulate per pass
- * over a range of peptide ids, in units of 1024, 1..16 (default 12); the range
- * is sized from the spectrum's entry density.  ctas_per_sm: resident CTAs per
+ * 384 or 512 (default 256 for up to 160 query bins a spectrum, else 384).
+ * chunk_entries: index entries a CTA aims to read per pass over a range of
+ * peptide ids, in units of 1024, 1..16 (default 16, which sets no such limit);
+ * the range is sized from the spectrum's entry density.  ctas_per_sm: resident CTAs per
  * SM (0 = as many as fit).  seg_pids: a spectrum's precursor window is split
  * into work units of at least this many peptide ids (0 = split only when the
  * batch is too small to fill the GPU).  Results do not depend on the shape. */

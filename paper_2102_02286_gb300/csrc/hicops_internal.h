@@ -36,6 +36,14 @@ constexpr uint32_t kSMask = (1u << 20) - 1;
 // Query bins per spectrum: every retained peak widened to 2 t + 1 bins.
 inline uint32_t query_bins_cap(const hicops_params& p) { return (2 * p.tol_bins + 1) * p.top_n_peaks; }
 
+// What the search needs of a bin's bucket, in one 16-byte load.
+struct BinInfo {
+    uint32_t group;   // the bucket's first 4-entry group
+    int32_t row;      // its skip-table row (-1: empty bucket)
+    int32_t hot;      // its bitmaps' row (-1: not hot)
+    uint32_t flags;   // hot: bit 0 has b entries, bit 1 has y entries
+};
+
 // Thread-local error message (host.cpp).
 void set_error(const char* fmt, ...);
 
@@ -52,15 +60,20 @@ struct DeviceIndex {
     int64_t* ls = nullptr;         // [s_max + 1]   LS[s] = round(2^32 log10 s)
     // chunk skip table of every non-empty bucket: row[bin] (-1 empty) and
     // skip[row * skip_stride + j] = entries with pid < j << kChunkShift
-    int32_t* skip_row = nullptr;   // [n_bins]
+    int32_t* skip_row = nullptr;   // [n_bins] (only while the index is built)
     uint32_t* skip = nullptr;      // [rows * skip_stride]
     uint32_t skip_stride = 0;      // chunks + 1
+    BinInfo* bins = nullptr;       // [n_bins] the above and the bitmap rows, by bin
+    // forward index: the ion bins of each peptide, fwd[4 fwd_off[pid] .. 4 fwd_off[pid + 1])
+    uint64_t* fwd_off = nullptr;   // [P + 1] in groups of 4 (16 bytes)
+    uint32_t* fwd = nullptr;       // bin << 1 | isY, ascending; each list padded to whole groups with 0xffffffff
+    uint64_t n_fwd = 0;            // groups
     // hot buckets (at least P >> kHotShift entries) as pid bitmaps
-    int32_t* hot_id = nullptr;     // [n_bins] (-1 not hot)
+    int32_t* hot_id = nullptr;     // [n_bins] (-1 not hot; only while the index is built)
     uint32_t* pid_map = nullptr;   // [P] global pids of a subset (else NULL)
     uint32_t* hot_b = nullptr;     // [n_hot * hot_words] b-ion bits
     uint32_t* hot_y = nullptr;     // [n_hot * hot_words] y-ion bits
-    uint32_t* hot_flags = nullptr; // [n_hot] bit 0: has b entries, bit 1: has y entries
+    uint32_t* hot_flags = nullptr; // [n_hot] bit 0: has b entries, bit 1: has y entries (while built)
     uint32_t n_hot = 0;
     uint64_t hot_words = 0;
     uint64_t bytes = 0;

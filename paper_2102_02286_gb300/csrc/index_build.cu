@@ -101,16 +101,27 @@ __global__ void ion_count_kernel(IonArgs a, uint32_t* __restrict__ count) {
     count[pid] = n;
 }
 
-__global__ void ion_emit_kernel(IonArgs a, const uint64_t* __restrict__ off, uint64_t* __restrict__ keys) {
+// list lengths in groups of 4 ion bins
+__global__ void ion_groups_kernel(uint32_t* __restrict__ count, uint64_t P) {
+    const uint64_t pid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (pid < P) count[pid] = (count[pid] + 3u) >> 2;
+}
+
+// keys for the sort by bin, and the forward list
+__global__ void ion_emit_kernel(IonArgs a, const uint64_t* __restrict__ off, uint64_t* __restrict__ keys,
+                                const uint64_t* __restrict__ fwd_off, uint32_t* __restrict__ fwd) {
     __shared__ double smres[128], smmod[128];
     for (int i = threadIdx.x; i < 128; i += blockDim.x) { smres[i] = a.mres[i]; smmod[i] = a.mmod[i]; }
     __syncthreads();
     const uint64_t pid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (pid >= a.P) return;
-    uint64_t o = off[pid];
+    uint64_t o = off[pid], f = 4 * fwd_off[pid];
     for_each_ion_bin(a, smres, smmod, pid, [&](uint32_t bin, uint32_t isy) {
-        keys[o++] = ((uint64_t)bin << 32) | (uint64_t)((uint32_t)(pid << 1) | isy);
+        keys[o] = ((uint64_t)bin << 32) | (uint64_t)((uint32_t)(pid << 1) | isy);
+        ++o;
+        fwd[f++] = (bin << 1) | isy;   // n_bins < 2^31 (parameter check)
     });
+    for (; f & 3; ++f) fwd[f] = 0xffffffffu;
 }
 
 // ---- stable LSD radix sort on the bin field (bits 32..) of 64-bit keys
@@ -272,6 +283,16 @@ __global__ void hot_fill_kernel(const uint64_t* __restrict__ keys, uint64_t n, c
     atomicOr(&hflags[h], (e & 1u) ? 2u : 1u);
 }
 
+// the search's record of every bin
+__global__ void bin_info_kernel(const uint64_t* __restrict__ off, const int32_t* __restrict__ row,
+                                const int32_t* __restrict__ hot_id, const uint32_t* __restrict__ hflags,
+                                uint32_t nbins, BinInfo* __restrict__ out) {
+    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= nbins) return;
+    const int32_t h = hot_id[b];
+    out[b] = BinInfo{(uint32_t)(off[b] >> 2), row[b], h, h >= 0 ? hflags[h] : 0u};
+}
+
 template <class T>
 cudaError_t dalloc(T** p, uint64_t n, std::vector<void*>& tmp) {
     cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (n ? n : 1));
@@ -281,6 +302,10 @@ cudaError_t dalloc(T** p, uint64_t n, std::vector<void*>& tmp) {
 
 struct TmpFree {
     std::vector<void*> ptrs;
+    void release(void* p) {
+        ptrs.erase(std::find(ptrs.begin(), ptrs.end(), p));
+        cudaFree(p);
+    }
     ~TmpFree() { for (void* p : ptrs) cudaFree(p); }
 };
 
@@ -303,6 +328,9 @@ void free_device_index(hicops_index* idx) {
         cudaFree(d.hot_b);
         cudaFree(d.hot_y);
         cudaFree(d.hot_flags);
+        cudaFree(d.bins);
+        cudaFree(d.fwd_off);
+        cudaFree(d.fwd);
         cudaFree(d.pid_map);
         for (void* e : d.ev) if (e) cudaEventDestroy((cudaEvent_t)e);
         if (cur >= 0 && cur != d.device) cudaSetDevice(cur);
@@ -370,6 +398,7 @@ hicops_status upload_index(hicops_index* idx) {
     uint64_t* d_total;
     HC_CUDA(dalloc(&d_cnt, P, tf.ptrs));
     HC_CUDA(dalloc(&d_ionoff, P, tf.ptrs));
+    HC_CUDA(cudaMalloc(&d.fwd_off, sizeof(uint64_t) * (P + 1)));
     HC_CUDA(dalloc(&d_total, 1, tf.ptrs));
     uint64_t* d_scan_tmp;
     HC_CUDA(dalloc(&d_scan_tmp, scan_tmp_words(P), tf.ptrs));
@@ -377,14 +406,19 @@ hicops_status upload_index(hicops_index* idx) {
     if (P) ion_count_kernel<<<pgrid, kIonThreads, 0, s>>>(a, d_cnt);
     HC_CUDA(cudaGetLastError());
     HC_CUDA(exclusive_scan<uint32_t>(d_cnt, P, d_ionoff, d_total, d_scan_tmp, s));
+    if (P) ion_groups_kernel<<<pgrid, kIonThreads, 0, s>>>(d_cnt, P);
+    HC_CUDA(cudaGetLastError());
+    HC_CUDA(exclusive_scan<uint32_t>(d_cnt, P, d.fwd_off, d.fwd_off + P, d_scan_tmp, s));
     uint64_t E = 0;
+    HC_CUDA(cudaMemcpyAsync(&d.n_fwd, d.fwd_off + P, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     HC_CUDA(cudaMemcpyAsync(&E, d_total, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     HC_CUDA(cudaStreamSynchronize(s));
 
     uint64_t *keys, *keys2;
     HC_CUDA(dalloc(&keys, E, tf.ptrs));
     HC_CUDA(dalloc(&keys2, E, tf.ptrs));
-    if (P) ion_emit_kernel<<<pgrid, kIonThreads, 0, s>>>(a, d_ionoff, keys);
+    HC_CUDA(cudaMalloc(&d.fwd, 16 * (d.n_fwd ? d.n_fwd : 1)));
+    if (P) ion_emit_kernel<<<pgrid, kIonThreads, 0, s>>>(a, d_ionoff, keys, d.fwd_off, d.fwd);
     HC_CUDA(cudaGetLastError());
 
     // stable radix sort on the bin bits
@@ -424,6 +458,9 @@ hicops_status upload_index(hicops_index* idx) {
     uint64_t mx = 0;
     HC_CUDA(cudaMemcpyAsync(&mx, d_mx, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
     HC_CUDA(cudaStreamSynchronize(s));
+    // the sort's other buffer goes before the stored entries come, so that the
+    // build's peak stays at 20 bytes an entry (two key buffers and the forward lists)
+    tf.release(keys2);
     if (mx >= (1ull << 32) - 3) {
         set_error("a bucket holds %llu entries (limit 2^32 - 4)", (unsigned long long)mx);
         return HICOPS_EOVERFLOW;
@@ -486,12 +523,21 @@ hicops_status upload_index(hicops_index* idx) {
     HC_CUDA(cudaMemsetAsync(d.hot_flags, 0, sizeof(uint32_t) * (nhot ? nhot : 1), s));
     if (E && nhot) hot_fill_kernel<<<egrid, 256, 0, s>>>(keys, E, d.hot_id, d.hot_words, d.hot_b, d.hot_y, d.hot_flags);
     HC_CUDA(cudaGetLastError());
+    HC_CUDA(cudaMalloc(&d.bins, sizeof(BinInfo) * nb));
+    bin_info_kernel<<<bgrid, 256, 0, s>>>(d.off, d.skip_row, d.hot_id, d.hot_flags, nb, d.bins);
+    HC_CUDA(cudaGetLastError());
     HC_CUDA(cudaStreamSynchronize(s));
+    cudaFree(d.skip_row);
+    cudaFree(d.hot_id);
+    cudaFree(d.hot_flags);
+    d.skip_row = d.hot_id = nullptr;
+    d.hot_flags = nullptr;
 
     d.n_stored = Ep;
     d.bytes = sizeof(double) * P + sizeof(uint64_t) * (idx->n_bins + 1) + sizeof(uint32_t) * (Ep + 4) +
-              sizeof(int64_t) * (lf.size() + ls.size()) + sizeof(int32_t) * 2 * nb +
-              sizeof(uint32_t) * rows * d.skip_stride + 2 * hbytes;
+              sizeof(int64_t) * (lf.size() + ls.size()) + sizeof(BinInfo) * nb +
+              sizeof(uint32_t) * rows * d.skip_stride + 2 * hbytes + sizeof(uint64_t) * (P + 1) +
+              16 * (d.n_fwd ? d.n_fwd : 1);
     idx->stats.n_entries = E;
     idx->stats.max_bucket = mx;
     idx->stats.device_bytes = d.bytes;

@@ -13,6 +13,7 @@
 // hicops_search allocates its scratch stream-ordered per call; a plan
 // (hicops_plan_*) allocates it once and can replay the sequence as a CUDA
 // graph.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 #include <cfloat>
@@ -71,8 +72,7 @@ struct Workspace {
     uint64_t *seg_off = nullptr, *stmp = nullptr;
     UnitTop* utop = nullptr;
     unsigned long long* work = nullptr;
-    uint32_t* order = nullptr;   // [cap_n * max_seg] units, longest first
-    uint32_t* order_q = nullptr; // [cap_n * max_seg] their spectra
+    uint4* unit = nullptr;       // [cap_n * max_seg] units in the order they are taken
     uint32_t* ocnt = nullptr;    // [2 * kOrderBuckets] bucket counts and starts
     hicops_psm* psm = nullptr;   // used when the caller gives no device output
     uint32_t* hist = nullptr;
@@ -94,8 +94,7 @@ hicops_status alloc_workspace(A& al, const hicops_params& p, uint32_t cap_n, uin
     HC_CUDA(al.get(&w.stmp, scan_tmp_words(cap_n)));
     HC_CUDA(al.get(&w.utop, (uint64_t)cap_n * max_seg * p.top_k));
     HC_CUDA(al.get(&w.work, 1));
-    HC_CUDA(al.get(&w.order, (uint64_t)cap_n * max_seg));
-    HC_CUDA(al.get(&w.order_q, (uint64_t)cap_n * max_seg));
+    HC_CUDA(al.get(&w.unit, (uint64_t)cap_n * max_seg));
     HC_CUDA(al.get(&w.ocnt, 2 * kOrderBuckets));
     if (outputs) {
         HC_CUDA(al.get(&w.psm, (uint64_t)cap_n * p.top_k));
@@ -127,13 +126,16 @@ hicops_status check_config(const hicops_search_config& c) {
     return HICOPS_OK;
 }
 
-// Default shape: 384-thread CTAs (two fit an SM while the top-k lists are
-// at most 16 long), else 256; super-chunks of up to about 12 k entries (the
-// planes and the log's room cap sparse spectra's super-chunks earlier).
-hicops_search_config resolved(const hicops_search_config& c, uint32_t k) {
+// Default shape: 256-thread CTAs, three an SM, where their planes hold 2^18
+// peptides (up to 160 query bins a spectrum), else 384-thread CTAs, two an SM,
+// whose planes hold twice that; super-chunks of any number of entries.
+// Measured both ways (search kernel): 30k spectra of 100 peaks at +-500 Da 8.3
+// against 8.5 ms, 2,500 at +-10 Da 0.11 against 0.16 ms; 5,000 spectra of 300
+// bins 3.9 against 3.2 ms, 12k of 50-500 peaks 3.6 against 3.4 ms.
+hicops_search_config resolved(const hicops_search_config& c, uint32_t query_bins) {
     hicops_search_config r = c;
-    if (!r.threads) r.threads = k <= 16 ? 384 : 256;
-    if (!r.chunk_entries) r.chunk_entries = 12;
+    if (!r.threads) r.threads = query_bins <= 160 ? 256 : 384;
+    if (!r.chunk_entries) r.chunk_entries = 16;
     return r;
 }
 
@@ -147,49 +149,80 @@ uint32_t max_segments(const hicops_search_config& c, uint32_t n) {
     return m;
 }
 
-template <int KMAX, int THREADS, int MAXP>
-hicops_status launch_search_t(const SearchArgs& sa, uint32_t ctas_per_sm, uint64_t max_units, cudaStream_t s) {
-    static std::atomic<int> occ{-1};   // CTAs per SM; concurrent first calls compute the same value
-    const size_t smem = sizeof(uint32_t) * Layout<KMAX, THREADS, MAXP>::kDynWords;   // planes, log, slots / counters
-    if (occ.load(std::memory_order_acquire) < 0) {
-        HC_CUDA(cudaFuncSetAttribute(search_kernel<KMAX, THREADS, MAXP>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        int b = 0;
-        HC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, search_kernel<KMAX, THREADS, MAXP>, THREADS,
-                                                              smem));
-        occ.store(b < 1 ? 1 : b, std::memory_order_release);
+// The parts of a CTA's shared memory when ctas CTAs share an SM.
+SearchLayout make_layout(uint32_t stride, uint32_t k, uint32_t threads, uint32_t ctas) {
+    const uint32_t maxp = (stride + 31) & ~31u, nwarps = threads / 32;
+    const uint32_t words = (kSmemPerSm / ctas - 1024) / 4;
+    SearchLayout l{};
+    uint32_t at = 0;
+    auto take = [&at](uint32_t n) { const uint32_t o = at; at += (n + 3) & ~3u; return o; };   // 16-byte aligned
+    take((sizeof(SearchShared) + 3) / 4);
+    l.runs = take(4 * maxp + 8);      // (fetching looks one run past the last)
+    l.subs = take(2 * threads / kSub);
+    l.head = take(kHeads / 2);
+    l.qpeak = take(2 * maxp);
+    l.next = take(maxp / 2);
+    l.tkey = take(2 * nwarps * k);
+    l.tab = take(kSlots);
+    l.wq = take(nwarps * kWarpQueue);
+    l.plane2 = take(kPlane2Words);
+    l.hotc = take(maxp);
+    l.pbase = take(maxp);
+    l.prow = take(maxp);
+    l.qpid = take(kQueue);
+    l.tpid = take(nwarps * k);
+    l.tpk = take(nwarps * k);
+    l.qneed = take(kQueue / 4);
+    // at most 2^kOffBits bits
+    l.plane_words = 1;       // (0 would not be a power of two; too small is for the caller to see)
+    while (at + 2 * l.plane_words <= words && l.plane_words < (1u << (kOffBits - 5))) l.plane_words *= 2;
+    for (uint32_t* o : {&l.runs, &l.subs, &l.head, &l.qpeak, &l.next, &l.tkey, &l.tab, &l.wq, &l.plane2, &l.hotc, &l.pbase,
+                        &l.prow, &l.qpid, &l.tpid, &l.tpk, &l.qneed})
+        *o += l.plane_words;
+    l.end = at + l.plane_words;
+    return l;
+}
+
+template <int THREADS, int PPT>
+hicops_status launch_search_t(const SearchArgs& sa, uint32_t ctas, uint64_t max_units, cudaStream_t s) {
+    static std::atomic<bool> ready{false};   // concurrent first calls set the same values
+    const size_t smem = sizeof(uint32_t) * sa.lay.end;
+    if (!ready.load(std::memory_order_acquire)) {
+        HC_CUDA(cudaFuncSetAttribute(search_kernel<THREADS, PPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(kSmemPerSm - 1024)));
+        HC_CUDA(cudaFuncSetAttribute(search_kernel<THREADS, PPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     cudaSharedmemCarveoutMaxShared));
+        ready.store(true, std::memory_order_release);
     }
-    int per_sm = occ.load(std::memory_order_acquire);
-    if (ctas_per_sm && (int)ctas_per_sm < per_sm) per_sm = (int)ctas_per_sm;
     // no more CTAs than work units can exist
-    uint64_t grid = (uint64_t)g_sm_count.load(std::memory_order_relaxed) * per_sm;
+    uint64_t grid = (uint64_t)g_sm_count.load(std::memory_order_relaxed) * ctas;
     if (max_units < grid) grid = max_units ? max_units : 1;
-    search_kernel<KMAX, THREADS, MAXP><<<(unsigned)grid, THREADS, smem, s>>>(sa);
+    search_kernel<THREADS, PPT><<<(unsigned)grid, THREADS, smem, s>>>(sa);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
     return HICOPS_OK;
 }
 
-// The kernel for at most 512 query bins a spectrum (no fragment tolerance, or
-// a narrow one) has the smaller static shared memory and the larger planes.
-template <int THREADS, int MAXP>
-hicops_status launch_search_p(const SearchArgs& sa, uint32_t ctas_per_sm, uint64_t max_units, cudaStream_t s) {
-    if (sa.k <= 8) return launch_search_t<8, THREADS, MAXP>(sa, ctas_per_sm, max_units, s);
-    if (sa.k <= 16) return launch_search_t<16, THREADS, MAXP>(sa, ctas_per_sm, max_units, s);
-    return launch_search_t<32, THREADS, MAXP>(sa, ctas_per_sm, max_units, s);
-}
-
+// PPT: ordinary peaks a thread owns at most
 template <int THREADS>
-hicops_status launch_search_k(const SearchArgs& sa, uint32_t ctas_per_sm, uint64_t max_units, cudaStream_t s) {
-    if (sa.topn <= 512) return launch_search_p<THREADS, 512>(sa, ctas_per_sm, max_units, s);
-    return launch_search_p<THREADS, kMaxTopN>(sa, ctas_per_sm, max_units, s);
+hicops_status launch_search_p(const SearchArgs& sa, uint32_t ctas, uint64_t max_units, cudaStream_t s) {
+    if (sa.stride <= THREADS) return launch_search_t<THREADS, 1>(sa, ctas, max_units, s);
+    if (sa.stride <= 2 * THREADS) return launch_search_t<THREADS, 2>(sa, ctas, max_units, s);
+    return launch_search_t<THREADS, 4>(sa, ctas, max_units, s);
 }
 
-hicops_status launch_search(const SearchArgs& sa, const hicops_search_config& c, uint64_t max_units,
-                            cudaStream_t s) {
-    if (c.threads == 512) return launch_search_k<512>(sa, c.ctas_per_sm, max_units, s);
-    if (c.threads == 384) return launch_search_k<384>(sa, c.ctas_per_sm, max_units, s);
-    return launch_search_k<256>(sa, c.ctas_per_sm, max_units, s);
+hicops_status launch_search(SearchArgs& sa, const hicops_search_config& c, uint64_t max_units, cudaStream_t s) {
+    uint32_t ctas = (uint32_t)search_min_ctas((int)c.threads);
+    if (c.ctas_per_sm && c.ctas_per_sm < ctas) ctas = c.ctas_per_sm;
+    // many query bins or long top-k lists leave little for the plane: fewer
+    // CTAs then, down to one an SM, where 16 columns fit beside the largest
+    for (;; --ctas) {
+        sa.lay = make_layout(sa.stride, sa.k, c.threads, ctas);
+        if (ctas == 1 || sa.lay.plane_words >= kMinPlaneWords) break;
+    }
+    if (c.threads == 512) return launch_search_p<512>(sa, ctas, max_units, s);
+    if (c.threads == 384) return launch_search_p<384>(sa, ctas, max_units, s);
+    return launch_search_p<256>(sa, ctas, max_units, s);
 }
 
 inline void mark(hicops_index* idx, int i, cudaStream_t s, bool on) {
@@ -226,7 +259,7 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
                              cudaStream_t s, bool timing_marks) {
     const hicops_params& p = idx->p;
     const DeviceIndex& di = idx->dev;
-    const hicops_search_config cfg = resolved(cfg_in, idx->p.top_k);
+    const hicops_search_config cfg = resolved(cfg_in, query_bins_cap(idx->p));
     const uint32_t k = p.top_k;
     mark(idx, 0, s, timing_marks);
     hicops_status st = prepare_queries(idx, d, n, w.qbin, w.qiq, w.qn, w.lo, w.hi, s);
@@ -234,29 +267,30 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     mark(idx, 1, s, timing_marks);
     const uint32_t max_seg = w.max_seg;
     const uint32_t seg_pids = cfg.seg_pids ? cfg.seg_pids : (uint32_t)kMinSegPids;
-    plan_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, n, max_seg, seg_pids, w.nseg);
-    count_launches(1);
-    HC_CUDA(cudaGetLastError());
-    HC_CUDA(exclusive_scan<uint32_t>(w.nseg, n, w.seg_off, w.seg_off + n, w.stmp, s));
     // longest units first; a small batch has too few units per CTA for the
-    // order to matter, and its three kernels would be most of its launch cost
-    const bool ordered = n >= kOrderMinSpectra;
-    if (ordered) {
+    // order to matter, and is planned by one kernel
+    if (n >= kOrderMinSpectra) {
+        plan_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, n, max_seg, seg_pids, w.nseg, w.work);
+        count_launches(1);
+        HC_CUDA(cudaGetLastError());
+        HC_CUDA(exclusive_scan<uint32_t>(w.nseg, n, w.seg_off, w.seg_off + n, w.stmp, s));
         HC_CUDA(cudaMemsetAsync(w.ocnt, 0, sizeof(uint32_t) * kOrderBuckets, s));
         order_count_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, w.seg_off, n, w.ocnt);
         order_scan_kernel<<<1, 32, 0, s>>>(w.ocnt);
         order_scatter_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, w.seg_off, n, w.ocnt + kOrderBuckets,
-                                                             w.order, w.order_q);
+                                                             w.unit);
         count_launches(3);
-        HC_CUDA(cudaGetLastError());
+    } else {
+        plan_small_kernel<<<1, kPlanThreads, 0, s>>>(w.qn, w.lo, w.hi, n, max_seg, seg_pids, w.seg_off, w.unit, w.work);
+        count_launches(1);
     }
+    HC_CUDA(cudaGetLastError());
     HC_CUDA(cudaMemsetAsync(d_hist, 0, sizeof(uint32_t) * n * kHistBins, s));
     HC_CUDA(cudaMemsetAsync(d_ns, 0, sizeof(uint32_t) * n, s));
-    HC_CUDA(cudaMemsetAsync(w.work, 0, sizeof(unsigned long long), s));
-    SearchArgs sa{w.qbin, w.qiq, w.qn, w.lo, w.hi, w.seg_off, n, query_bins_cap(p), di.off, di.entry,
-                  di.skip_row, di.skip, di.skip_stride, di.hot_id, di.hot_b, di.hot_y, di.hot_flags,
-                  di.hot_words, di.lf, di.ls, (uint32_t)idx->s_max, p.min_shared, k, cfg.chunk_entries * 1024u, w.utop, d_hist, d_ns,
-                  w.work, ordered ? w.order : nullptr, w.order_q};
+    SearchArgs sa{w.qbin, w.qiq, w.qn, n, query_bins_cap(p), w.unit, w.seg_off + n, di.bins, di.entry, di.skip,
+                  di.skip_stride, di.hot_b, di.hot_y, di.hot_words, di.fwd_off, reinterpret_cast<const uint4*>(di.fwd), di.lf, di.ls,
+                  (uint32_t)idx->s_max, p.min_shared, k, cfg.chunk_entries < 16 ? cfg.chunk_entries * 1024u : 0xffffffffu, w.utop, d_hist, d_ns, w.work,
+                  SearchLayout{}};
     mark(idx, 2, s, timing_marks);
     st = launch_search(sa, cfg, (uint64_t)n * max_seg, s);
     if (st != HICOPS_OK) return st;
@@ -696,7 +730,7 @@ constexpr uint64_t noalloc_bytes(uint64_t cap) {
            + 4096                                                // scan temporaries
            + align256(sizeof(UnitTop) * cap * kNoAllocSegs * kMaxTopK)
            + 256                                                 // work counter
-           + 2 * align256(4 * cap * kNoAllocSegs)                // unit order and its spectra
+           + align256(sizeof(uint4) * cap * kNoAllocSegs)        // units
            + align256(4 * 2 * kOrderBuckets)                     // its bucket counts
            + align256(sizeof(hicops_psm) * cap * kMaxTopK)       // psm (unused here)
            + align256(4 * cap * kHistBins) + align256(4 * cap);  // hist, n_scored

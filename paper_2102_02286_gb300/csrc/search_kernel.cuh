@@ -2,77 +2,76 @@
 // Supplementary Algorithm 3), included by search_kernels.cuh.
 //
 // One persistent CTA pulls work units (spectrum q, peptide-id segment) from a
-// device counter.  The segment is cut into super-chunks of whole skip-table
-// columns (kChunk peptide ids each, at most kMaxCols); the columns per
-// super-chunk are chosen per unit from the skip tables so that a super-chunk
-// holds about target_entries index entries of the spectrum's ordinary peaks.
+// device counter.  The segment is walked in super-chunks of whole skip-table
+// columns (kChunk peptide ids each).  Of the tens of thousands of index
+// entries a unit reads, a few dozen peptides reach min_shared, so the pass
+// over the entries only finds which peptides can, and those are scored
+// afterwards from the forward index (each peptide's own list of ion bins):
+//   pass A  every index entry of the ordinary peaks' runs sets its peptide's
+//           bit in a bit-plane in shared memory; an entry whose bit was set
+//           is a repeat and goes to its warp's queue, which is emptied with
+//           every lane busy into an open-addressing table of (peptide,
+//           repeats).  In a wide window (deep) a super-chunk spans more
+//           peptides than the plane has bits, and a repeat has to find its
+//           bit in a second plane set before it counts;
+//   scan    only in a unit whose hot slices can qualify a peptide of one
+//           ordinary hit (or none): the plane together with the bitmaps;
+//   select  peptides of the table that can reach min_shared with their hot
+//           bits go to the unit's queue (their ordinary hits are known, or
+//           bounded from above when deep);
+//   drain   at the unit's end, or when the queue runs full: the hot bits are
+//           checked, then eight lanes read each remaining peptide's ion bins
+//           (16-byte loads) and look them up in a table of the spectrum's
+//           retained bins: nb, ny and S are exact, the key K = LF[nb] + LF[ny]
+//           + LS[S] enters the histogram and the warp's top-k list.
+// Should the repeats not fit their table, the super-chunk is halved, down to
+// one column, which is then searched with one counter a peptide.
 //
-// Almost every peptide in a precursor window is hit by at most one ordinary
-// peak, and with fewer than min_shared - 1 hot slices such a peptide cannot
-// reach min_shared.  So a super-chunk is searched as:
-//   pass A  every index entry (all ordinary peaks' runs, rounded out to
-//           16-byte groups, laid end to end by a prefix sum; lane l of a warp
-//           takes the 4-entry groups 4 l, 4 l + 128, ..., one 16-byte load
-//           each) sets the peptide's bit in a "seen" bit-plane and, when it
-//           was set, in a "twice" plane (shared-memory atomicOr), and is
-//           logged in shared memory as (peptide offset << 1 | isY | peak <<
-//           19); first bits set in the twice plane are counted;
-//   mark    only when nslices >= min_shared - 1 (peptides seen once with
-//           enough hot bits are candidates too) or when there are more than
-//           kRound candidates: the planes are scanned with the bitmaps,
-//           candidates counted and split into rounds of at most kRound
-//           candidates by runs of whole plane words; when the hot peaks alone
-//           can reach min_shared, the peptides of the segment no ordinary
-//           peak hit but with enough hot bits are scored here; otherwise
-//           there is one round of the twice plane;
-//   replay  per round, the log is walked; a candidate's record goes to its
-//           warp's queue, and full queues add (1 << 26 | iq) for a b ion or
-//           (1 << 20 | iq) for a y ion to the peptide's 32-bit counter (nb |
-//           ny | S) in an open-addressing table of kSlots 64-bit slots
-//           (offset << 32 | counter); a round has fewer than kSlots keys, so
-//           probing always ends;
-//   epilogue the occupied slots get the hot peaks' contributions from the
-//           bucket bitmaps; peptides with nb + ny >= min_shared are ranked
-//           with the exact key K = LF[nb] + LF[ny] + LS[S] and counted in the
-//           shared histogram; those better than their warp's k-th enter the
-//           warp's top-k list in shared memory (lanes take turns at points
-//           where the warp is converged), and the warps' lists are merged at
-//           the end of the unit.  Keeping the lists out of registers leaves
-//           80 registers a thread, so CTAs of 384 threads run two per SM.
-// The planes take 2 x 512 words per column of the super-chunk and the log
-// the words after them, so sparse spectra get wide super-chunks and dense
-// ones long logs.  A super-chunk whose planes and log do not fit is searched
-// column by column with 16384 directly indexed counters.
+// What bounds it: the latencies and the issue slots of pass A (one shared
+// atomic and about 16 instructions an entry; DRAM moves 470 KB a spectrum, a
+// third of the time at full rate) and, in spectra with thousands of scored
+// peptides, the drain.  Against the form that logged every entry and replayed
+// the log (one bit a peptide in two planes, super-chunks of 13 columns): 30k
+// spectra of 100 peaks at +-500 Da on 13.0 M peptides 15.7 -> 8.3 ms, 6k of 150
+// peaks on 11.7 M peptides 5.2 -> 3.5 ms, 12k of 50-500 peaks at mixed
+// tolerances 4.9 -> 3.1 ms.
 
 constexpr int kMaxHot = 6;                 // bitmap slices (b or y bitmap of a hot bucket) per spectrum
 constexpr int kMaxWarps = 16;              // CTAs of up to 512 threads
-constexpr int kTouchCap = 3584;            // touched list of a direct-counter column (more: full scan)
-constexpr uint32_t kSlots = 1024;          // candidate counters per round
-constexpr uint32_t kRound = 768;           // candidates per round (+31 at most)
-constexpr uint32_t kListWords = 1152;      // compaction lists: up to 3 groups of 32 slots per warp
-constexpr uint32_t kRoundsCap = 32;        // candidate rounds of a super-chunk at most
-constexpr uint32_t kSmemPerCta = 233472 / 2 - 1024;   // shared memory of one of two CTAs on an SM
-
+constexpr uint32_t kSub = 8;               // lanes that walk a run together (8 groups of 4 entries: 128 bytes)
+constexpr uint32_t kSlotBits = 11;
+constexpr uint32_t kSlots = 1u << kSlotBits;   // repeat counters of a super-chunk
+constexpr uint32_t kProbes = 64;           // slots tried before the table counts as full
+constexpr uint32_t kHeads = 2048;          // chains of the retained bins' table
+constexpr uint32_t kKeysAim = 700;         // peptides of the repeat table aimed at
+constexpr uint32_t kQueue = 1152;          // a unit's queue of peptides to score
+constexpr uint32_t kWarpQueue = 144;       // a warp's repeats waiting for the table
+constexpr uint32_t kPlane2Bits = 11;       // words of the second plane (2^16 bits)
+constexpr uint32_t kPlane2Words = 1u << kPlane2Bits;
+constexpr float kPlane2Aim = 6500.0f;      // repeats it takes (they collide n n / 2^17 times)
+constexpr uint32_t kNoEnd = 0x7fffffffu;    // length of the run that closes the list
+constexpr uint32_t kOffBits = 24;          // peptide offset inside a super-chunk (repeat table key)
+constexpr uint32_t kDirectNeed = 0x80u;    // queue flag: found by a scan of every peptide
+constexpr uint32_t kMinPlaneWords = 4096;  // smallest plane worth another CTA on the SM (8 columns)
+constexpr uint32_t kSmemPerSm = 233472;    // shared memory of an SM; each CTA also takes 1 KB of it
 
 struct SearchArgs {
     const uint32_t* qbin;
     const uint32_t* qiq;
     const uint32_t* qn;
-    const uint32_t* lo;
-    const uint32_t* hi;
-    const uint64_t* seg_off;    // [n + 1] first unit of each spectrum
     uint32_t n;
-    uint32_t topn;
-    const uint64_t* off;        // bucket offsets
+    uint32_t stride;            // qbin / qiq words per spectrum
+    const uint4* unit;          // [units] the units in the order they are taken
+    const uint64_t* n_units;    // their number
+    const BinInfo* bins;        // [n_bins] bucket of every bin
     const uint32_t* entry;      // pid << 1 | isY
-    const int32_t* skip_row;
     const uint32_t* skip;
     uint32_t skip_stride;
-    const int32_t* hot_id;
     const uint32_t* hot_b;
     const uint32_t* hot_y;
-    const uint32_t* hot_flags;
     uint64_t hot_words;
+    const uint64_t* fwd_off;    // [P + 1] forward lists, in groups of 4
+    const uint4* fwd;           // bin << 1 | isY
     const int64_t* lf;
     const int64_t* ls;
     uint32_t s_max;             // last valid index of ls
@@ -83,908 +82,1026 @@ struct SearchArgs {
     uint32_t* hist;             // [n * 256]
     uint32_t* nscored;          // [n]
     unsigned long long* work;   // unit counter
-    const uint32_t* order;      // [units] the units in the order they are taken (longest first), or NULL
-    const uint32_t* order_q;    // [units] the spectrum of each of them
+    SearchLayout lay;
 };
 
 __device__ __forceinline__ bool better(int64_t ka, uint32_t pa, int64_t kb, uint32_t pb) {
     return ka > kb || (ka == kb && pa < pb);
 }
 
-// A warp's best k candidates of the current unit, sorted by (key desc, pid
-// asc), in shared memory; one lane at a time inserts (warp-synchronous).
-template <int KMAX>
-struct WarpTop {
-    int64_t key[KMAX];
-    uint32_t pid[KMAX];
-    uint32_t pk[KMAX];
-    int n;
-    __device__ __forceinline__ bool passes(int64_t kk, uint32_t p, int k) const {
-        return n < k || better(kk, p, key[k - 1], pid[k - 1]);
-    }
-    __device__ __forceinline__ void insert(int64_t kk, uint32_t p, uint32_t packed, int k) {
-        if (!passes(kk, p, k)) return;
-        int pos = n < k ? n : k - 1;
-        while (pos > 0 && better(kk, p, key[pos - 1], pid[pos - 1])) {
-            key[pos] = key[pos - 1];
-            pid[pos] = pid[pos - 1];
-            pk[pos] = pk[pos - 1];
-            --pos;
-        }
-        key[pos] = kk;
-        pid[pos] = p;
-        pk[pos] = packed;
-        if (n < k) ++n;
-    }
+// Where a CTA is in its unit (the same in every thread).
+struct UnitState {
+    uint32_t c, e;                    // the super-chunk's columns
+    uint32_t m;                       // columns of a super-chunk
+    uint32_t deep;                    // repeats pass the second plane before the table
+    uint32_t taken;                   // the next unit is taken
+    uint32_t slot;                    // of the current unit
 };
 
-template <int MAXP>
 struct SearchShared {
-    uint32_t pbase[MAXP];             // bucket start of each ordinary peak, in 4-entry groups
-    uint32_t prow[MAXP];              // its skip-table row
-    uint32_t pinc[MAXP];              // its quantised intensity
-    uint32_t pre[2][MAXP + 1];        // exclusive prefix of the run lengths (parity)
-    uint32_t rs[2][MAXP];             // run starts relative to the bucket (parity)
-    union {
-        uint16_t touched[MAXP <= 512 ? 1 : kTouchCap];   // counters that became non-zero (else dynamic)
-        uint16_t hotc[MAXP];          // (classification) hot peaks: index into qbin
-    };
-    uint16_t wli[2][kMaxWarps];       // peak holding each warp's first entry (parity)
-    uint16_t wb[kRoundsCap + 1];      // first plane word of each candidate round
-    int ntouched;                     // > kTouchCap means the list overflowed
-    int nrounds;
-    uint32_t ncand[2];                // candidates counted by pass A (alternating super-chunks)
     const uint32_t* slice[kMaxHot];   // bitmap rows of the spectrum's hot slices
-    uint32_t slice_inc[kMaxHot];      // counter increment of a set bit
     uint32_t hist[kHistBins];
     int64_t lf[kMaxLen + 1];
-    uint32_t wsum[kMaxWarps];
-    uint32_t wcand[kMaxWarps];
+    uint32_t wsum[kMaxWarps], wruns[kMaxWarps];
+    int wn[kMaxWarps];                // length of each warp's top-k list
+    uint32_t nkeys;                   // peptides in the repeat table
+    int over;                         // it was full (or holds more than the queue takes)
+    int no_room;                      // the queue may not take what the repeat table holds (-1: it is empty)
+    uint32_t nq, npass;               // peptides in the queue, and of them past the hot-bit check
     int nnorm, nhotc, nslices, nhotpeaks;
-    uint64_t unit;
-    uint32_t q, np;
-    uint32_t seg_lo, seg_hi;
+    uint4 unit[2];                    // the current unit and the one taken next (alternating): spectrum, segment,
+                                      // unit number
+    uint64_t t_next;                  // its place in the order
+    int have;                         // there is one
+    uint32_t per, total;              // pieces of an octet's share, and of all
+    UnitState st;                     // the current unit's, across the calls that need every register
 };
 
-// Dynamic shared memory of the kernel for top-k lists of KMAX, CTAs of
-// THREADS and at most MAXP query bins, in 32-bit words: what two CTAs on an
-// SM leave beside their static part.  A super-chunk of m columns (W = 512 m
-// words per plane):
-//   [0, W) seen plane | [W, 2W) twice plane | [2W, 2W + R) log |
-//   [kListWord, kSlotWord) slot compaction lists | [kSlotWord, kDynWords) kSlots 64-bit slots;
-// or [0, 16384) direct counters (lists and slots are zero then), with the
-// direct columns' touched list right above them for MAXP = 512, where the
-// smaller static part leaves the planes and log about 21 k words (about
-// 15.5 k for MAXP = 1024).
-template <int KMAX, int THREADS, int MAXP>
-struct Layout {
-    static constexpr uint32_t kStatic = sizeof(SearchShared<MAXP>) + (THREADS / 32) * sizeof(WarpTop<KMAX>) + 64;
-    static constexpr uint32_t kDynWords = ((kSmemPerCta - kStatic) / 4) & ~31u;
-    static constexpr uint32_t kSlotWord = kDynWords - 2 * kSlots;
-    static constexpr uint32_t kListWord = kSlotWord - kListWords;
-    static constexpr uint32_t kMaxRounds = kListWord / kRound + 2;
-    // widest super-chunk (columns of kChunk ids): planes within the counters'
-    // 16384 words (below the touched list) and 19-bit record offsets, and
-    // room for a log of 2048 words beside the widest planes
-    static constexpr uint32_t kMaxCols = (kListWord - 2048) / 1024 < 16 ? (kListWord - 2048) / 1024 : 16;
-    static constexpr bool kTouchDyn = MAXP <= 512;
-    static_assert(kMaxRounds <= kRoundsCap, "round starts fit");
-    static_assert(kMaxCols >= 1 && 2 * kMaxCols * kChunk / 32 < kListWord, "planes leave room for a log");
-    static_assert(2 * kMaxCols * kChunk / 32 <= kChunk, "planes never reach the touched list");
-    static_assert(2 * kMaxCols * kChunk <= 0x80000u, "record offsets fit 19 bits below the peak index");
-    static_assert(!kTouchDyn || kChunk + kTouchCap / 2 <= kListWord, "the touched list lies below the lists");
-    static_assert(kDynWords >= kChunk, "the direct counters fit");
+// All shared memory is dynamic: the plane first (its address is then a
+// constant of the atomics), SearchShared behind it and the parts of the
+// layout.  Functions that are not inlined reach it through these, so that
+// their accesses are shared-memory instructions too.
+__device__ __forceinline__ uint32_t* search_smem() {
+    extern __shared__ __align__(16) uint32_t smem32[];
+    return smem32;
+}
+__device__ __forceinline__ SearchShared& search_shared(const SearchArgs& a) {
+    return *reinterpret_cast<SearchShared*>(search_smem() + a.lay.plane_words);
+}
+
+// The parts of dynamic shared memory, and what the scoring of a unit needs.
+struct SearchParts {
+    uint4* runs;          // [maxp + 1] the super-chunk's non-empty runs: first group, groups, the first piece's
+                          // start from the first group (its line's: 0 or below); then one without end
+    uint2* subs;          // [nsub] where each octet's share starts: its run, and its first piece there
+    uint32_t* head;       // [kHeads / 2] pairs of 16-bit chain heads of the retained bins' table: peak + 1, or 0
+    uint2* qpeak;         // [maxp] the retained peaks: bin, quantised intensity
+    uint16_t* next;       // [maxp] the next peak of the chain + 1, or 0
+    int64_t* tkey;        // [nwarps * k] the warps' best candidates, sorted by (key desc, pid asc)
+    uint32_t* tab;        // [kSlots] (offset << (32 - kOffBits)) | repeats
+    uint32_t* wq;         // [nwarps * kWarpQueue] repeats on their way to it
+    uint32_t* plane2;     // [kPlane2Words]
+    uint32_t* hotc;       // [maxp] the bins of the hot peaks
+    uint32_t* pbase;      // [maxp] first group of each ordinary peak's bucket
+    uint32_t* prow;       // [maxp] its skip-table row
+    uint32_t* qpid;       // [kQueue]
+    uint32_t* tpid;       // [nwarps * k]
+    uint32_t* tpk;        // [nwarps * k]
+    uint8_t* qneed;       // [kQueue] hot bits needed, and kDirectNeed
+    uint32_t* plane;      // [plane_words] (a power of two)
 };
 
-__device__ __forceinline__ uint32_t counter_inc_y(uint32_t isy, uint32_t iq) {
-    return iq + (isy ? (1u << kNyShift) : (1u << kNbShift));
+__device__ __forceinline__ SearchParts search_parts(const SearchLayout& l) {
+    uint32_t* const base = search_smem();
+    SearchParts p;
+    p.runs = reinterpret_cast<uint4*>(base + l.runs);
+    p.subs = reinterpret_cast<uint2*>(base + l.subs);
+    p.head = base + l.head;
+    p.qpeak = reinterpret_cast<uint2*>(base + l.qpeak);
+    p.next = reinterpret_cast<uint16_t*>(base + l.next);
+    p.tkey = reinterpret_cast<int64_t*>(base + l.tkey);
+    p.tab = base + l.tab;
+    p.wq = base + l.wq;
+    p.plane2 = base + l.plane2;
+    p.hotc = base + l.hotc;
+    p.pbase = base + l.pbase;
+    p.prow = base + l.prow;
+    p.qpid = base + l.qpid;
+    p.tpid = base + l.tpid;
+    p.tpk = base + l.tpk;
+    p.qneed = reinterpret_cast<uint8_t*>(base + l.qneed);
+    p.plane = base;
+    return p;
 }
 
-__device__ __forceinline__ uint32_t slot_of(uint32_t off) { return (off * 2654435761u) >> 22; }   // 10 bits
+__device__ __forceinline__ uint32_t hash_u32(uint32_t x) { return x * 2654435761u; }
 
-// A run [ra, rb) of a bucket (positions relative to its 16-byte aligned
-// start) is read as whole groups of 4 entries: from ra rounded down to a
-// multiple of 4 to rb rounded up.  The extra entries at either end lie in the
-// same bucket outside the run's columns, or are the bucket's pad slots; both
-// fall outside every peptide range the run is searched for.
-__device__ __forceinline__ uint32_t group_start(uint32_t ra) { return ra & ~3u; }
-__device__ __forceinline__ uint32_t group_len(uint32_t ra, uint32_t rb) {
-    return ra == rb ? 0u : ((rb + 3u) & ~3u) - (ra & ~3u);
-}
-
-// Exclusive scan of the ordinary peaks' run lengths (in whole groups), in two
-// halves around a barrier the caller provides.  Thread tid owns peaks
-// tid*ppt .. +ppt-1.
-template <int PPT, class SH>
-__device__ __forceinline__ uint32_t scan_runs_1(SH& sh, int nnorm, int ppt, const uint32_t (&ra)[PPT],
-                                                const uint32_t (&rb)[PPT]) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t sum = 0;
-#pragma unroll
-    for (int i = 0; i < PPT; ++i) {
-        const int t = tid * ppt + i;
-        if (i < ppt && t < nnorm) sum += group_len(ra[i], rb[i]);
+// The match of one ion bin, as nb | ny | S: a chained table by the bin modulo
+// kHeads, where most bins find an empty head and few more than one peak.
+__device__ __forceinline__ uint32_t match_ion(const SearchParts& sp, uint32_t ion) {
+    const uint32_t bin = ion >> 1;   // pads are 0xffffffff: bin 2^31 - 1, in no spectrum
+    uint32_t c = 0;
+    uint32_t i = reinterpret_cast<const uint16_t*>(sp.head)[bin & (kHeads - 1u)];
+    while (i) {
+        const uint2 pk = sp.qpeak[i - 1u];
+        if (pk.x == bin) {
+            c = pk.y + ((ion & 1u) ? (1u << kNyShift) : (1u << kNbShift));
+            break;
+        }
+        i = sp.next[i - 1u];
     }
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += x;
-    }
-    if (lane == 31) sh.wsum[warp] = incl;
-    return incl - sum;
+    return c;
+}
+__device__ __forceinline__ uint32_t match_group(const SearchParts& sp, const uint4& x) {
+    return match_ion(sp, x.x) + match_ion(sp, x.y) + match_ion(sp, x.z) + match_ion(sp, x.w);
 }
 
-// Warp shares are multiples of 4 entries so that a lane's 4 consecutive
-// entries never cross into the next warp's share.
-template <int THREADS>
-__device__ __forceinline__ uint32_t warp_share(uint32_t total) {
-    constexpr int nwarps = THREADS / 32;
-    return ((total + nwarps - 1) / nwarps + 3) & ~3u;
+// The lanes' scored peptides (nb | ny | S in c): key, histogram, the warp's
+// top-k list (lanes in turn).  Every lane of the warp calls it.
+__device__ __forceinline__ void score_lanes(const SearchArgs& a, SearchShared& sh, const SearchParts& sp, bool ok,
+                                            uint32_t pid, uint32_t c) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = (int)a.k;
+    int64_t* const tkey = sp.tkey + warp * k;
+    uint32_t* const tpid = sp.tpid + warp * k;
+    uint32_t* const tpk = sp.tpk + warp * k;
+    const uint32_t nb = c >> kNbShift, ny = (c >> kNyShift) & 63u;
+    int64_t K = INT64_MIN;
+    bool pend = false;
+    if (ok && nb + ny >= a.min_shared) {
+        uint32_t S = c & kSMask;
+        if (S > a.s_max) S = a.s_max;   // unreachable for a consistent index
+        K = sh.lf[nb] + sh.lf[ny] + __ldg(a.ls + S);
+        const int64_t hb = K >> 31;
+        atomicAdd(&sh.hist[hb > 255 ? 255 : (hb < 0 ? 0 : hb)], 1u);
+        const int n = sh.wn[warp];
+        pend = n < k || better(K, pid, tkey[k - 1], tpid[k - 1]);
+    }
+    unsigned pm = __ballot_sync(0xffffffffu, pend);
+    while (pm) {
+        const int l = __ffs(pm) - 1;
+        pm &= pm - 1;
+        if (lane == l) {
+            const int n = sh.wn[warp];
+            if (n < k || better(K, pid, tkey[k - 1], tpid[k - 1])) {
+                int pos = n < k ? n : k - 1;
+                while (pos > 0 && better(K, pid, tkey[pos - 1], tpid[pos - 1])) {
+                    tkey[pos] = tkey[pos - 1];
+                    tpid[pos] = tpid[pos - 1];
+                    tpk[pos] = tpk[pos - 1];
+                    --pos;
+                }
+                tkey[pos] = K;
+                tpid[pos] = pid;
+                tpk[pos] = c;
+                if (n < k) sh.wn[warp] = n + 1;
+            }
+        }
+        __syncwarp();
+    }
 }
 
-template <int THREADS, int PPT, class SH>
-__device__ __forceinline__ void scan_runs_2(SH& sh, int buf, int nnorm, int ppt, uint32_t excl,
-                                            const uint32_t (&ra)[PPT], const uint32_t (&rb)[PPT]) {
-    const int tid = threadIdx.x, warp = tid >> 5;
-    constexpr int nwarps = THREADS / 32;
-    uint32_t wbase = 0, total = 0;
+// A peptide is taken when its hot bits reach what its ordinary hits leave to
+// min_shared (need); in a unit whose plane was scanned (once) a peptide of
+// min_shared - 1 hot bits or more came from the scan (kDirectNeed), so the
+// repeat table's entry for it is dropped.
+__device__ __forceinline__ bool hot_check(const SearchArgs& a, const SearchShared& sh, uint32_t pid, uint32_t nd,
+                                          bool once) {
+    const bool scanned = (nd & kDirectNeed) != 0u;
+    const uint32_t need = nd & ~kDirectNeed;
+    if (!need && (scanned || !once)) return true;
+    const int nslices = sh.nslices;
+    uint32_t hw[kMaxHot], h = 0;   // every slice's word in flight at once
 #pragma unroll
-    for (int w = 0; w < nwarps; ++w) {
-        const uint32_t s = sh.wsum[w];
-        if (w < warp) wbase += s;
-        total += s;
+    for (int s = 0; s < kMaxHot; ++s) hw[s] = s < nslices ? __ldg(sh.slice[s] + (pid >> 5)) : 0u;
+#pragma unroll
+    for (int s = 0; s < kMaxHot; ++s) h += (hw[s] >> (pid & 31)) & 1u;
+    return h >= need && (scanned || !once || h + 1u < a.min_shared);
+}
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// Scores cnt peptides pid[0..cnt) with the octets of the calling warp and of
+// the nocts octets in all: octet o takes pid[o], pid[o + nocts], ...  Two
+// peptides' first 64 ion bins (two 16-byte groups a lane) are in flight an
+// octet; after eight peptides a lane's worth of results is scored.  oct0 is
+// the lowest of the warp's octets, so that trips are warp-uniform.
+__device__ __forceinline__ void score_list(const SearchArgs& a, SearchShared& sh, const SearchParts& sp,
+                                           const uint32_t* pids, uint32_t cnt, uint32_t oct, uint32_t oct0,
+                                           uint32_t nocts) {
+    const uint32_t lane = threadIdx.x & 31, sl = lane & 7u;
+    const uint4 none = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+    for (uint32_t i0 = 0; i0 + oct0 < cnt; i0 += 8 * nocts) {
+        // lane sl of the octet looks up item i0 + sl * nocts + oct
+        const uint32_t it = i0 + sl * nocts + oct;
+        uint32_t ng = 0;
+        uint64_t g0 = 0;
+        if (it < cnt) {
+            const uint32_t pid = pids[it];
+            g0 = __ldg(a.fwd_off + pid);
+            ng = (uint32_t)(__ldg(a.fwd_off + pid + 1) - g0);
+            // (the lists' lines on their way while the first two are matched)
+            if (ng) prefetch_l2(a.fwd + g0);
+            if (ng > 8u) prefetch_l2(a.fwd + g0 + 8u);
+            if (ng > 16u) prefetch_l2(a.fwd + g0 + 16u);
+        }
+        uint32_t c = 0;
+#pragma unroll 1
+        for (uint32_t h = 0; h < 8 && i0 + h * nocts + oct0 < cnt; h += 2) {   // warp-uniform
+            uint4 x[2], y[2];
+            uint32_t nn[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int src = (int)((lane & 24u) + h) + j;
+                const uint64_t gg = __shfl_sync(0xffffffffu, g0, src);
+                nn[j] = __shfl_sync(0xffffffffu, ng, src);
+                x[j] = sl < nn[j] ? __ldg(a.fwd + gg + sl) : none;
+                y[j] = sl + 8u < nn[j] ? __ldg(a.fwd + gg + sl + 8u) : none;
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                uint32_t r = match_group(sp, x[j]);
+                if (__any_sync(0xffffffffu, nn[j] > 8u)) r += match_group(sp, y[j]);
+                if (__any_sync(0xffffffffu, nn[j] > 16u)) {   // more than 64 ion bins
+                    const uint64_t gg = __shfl_sync(0xffffffffu, g0, (int)((lane & 24u) + h) + j);
+#pragma unroll 1
+                    for (uint32_t g = sl + 16u; __any_sync(0xffffffffu, g < nn[j]); g += 8u)
+                        r += match_group(sp, g < nn[j] ? __ldg(a.fwd + gg + g) : none);
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);   // fields cannot overflow
+                if (sl == h + (uint32_t)j) c = r;
+            }
+        }
+        score_lanes(a, sh, sp, it < cnt, it < cnt ? pids[it] : 0u, c);
     }
-    const uint32_t per = warp_share<THREADS>(total);
-    uint32_t run = wbase + excl;
+}
+
+// Scores the unit's queue with the whole block and empties it (every thread
+// calls it, behind a barrier after the last append; it ends with one).  The
+// peptides past the hot-bit check are gathered in the warps' queues, which
+// are empty between two passes.
+__device__ __noinline__ void drain_queue(const SearchArgs& a) {
+    SearchShared& sh = search_shared(a);
+    const bool once = (uint32_t)sh.nslices + 1u >= a.min_shared;   // the plane was scanned
+    const SearchParts sp = search_parts(a.lay);
+    uint32_t* const pass = sp.wq;
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t cnt = min(sh.nq, kQueue);
+    for (uint32_t i0 = tid & ~31u; i0 < cnt; i0 += blockDim.x) {   // warp-uniform trips
+        const uint32_t i = i0 + lane;
+        bool ok = i < cnt;
+        uint32_t pid = 0;
+        if (ok) {
+            pid = sp.qpid[i];
+            ok = hot_check(a, sh, pid, sp.qneed[i], once);
+        }
+        if (ok) pass[atomicAdd(&sh.npass, 1u)] = pid;
+    }
+    __syncthreads();
+    // consecutive peptides go to different warps
+    const uint32_t nwarps = blockDim.x >> 5;
+    score_list(a, sh, sp, pass, sh.npass, (lane >> 3) * nwarps + (tid >> 5), tid >> 5, 4u * nwarps);
+    __syncthreads();
+    if (tid == 0) sh.nq = sh.npass = 0u;
+    __syncthreads();
+}
+
+// Appends the lane's peptide to the unit's queue; false when it is full.
+__device__ __forceinline__ bool push(const SearchArgs& a, SearchShared& sh, const SearchParts& sp, uint32_t pid,
+                                     uint32_t need) {
+    const uint32_t at = atomicAdd(&sh.nq, 1u);
+    if (!(need & ~kDirectNeed)) prefetch_l2(a.fwd_off + pid);   // (it is sure to be scored)
+    if (at >= kQueue) return false;   // (the counter stays past the end)
+    sp.qpid[at] = pid;
+    sp.qneed[at] = (uint8_t)need;
+    return true;
+}
+
+// One more repeat of the peptide at offset off.
+__device__ __forceinline__ void add_repeat(SearchShared& sh, const SearchParts& sp, uint32_t off) {
+    uint32_t s = hash_u32(off) >> (32 - kSlotBits);
+    for (uint32_t probe = 0; probe < kProbes; ++probe) {
+        const uint32_t old = atomicCAS(&sp.tab[s], 0u, (off << (32 - kOffBits)) | 1u);
+        if (old == 0u) {
+            atomicAdd(&sh.nkeys, 1u);
+            return;
+        }
+        if ((old >> (32 - kOffBits)) == off) {   // (a peptide has at most 126 ions: 8 bits hold its repeats)
+            atomicAdd(&sp.tab[s], 1u);
+            return;
+        }
+        s = (s + 1u) & (kSlots - 1u);
+    }
+    sh.over = 1;
+}
+
+// The plane of a super-chunk (first peptide pb, words in use, peptides [x0,
+// x1)) together with the hot bitmaps: queues the peptides seen once or more
+// with at least min_shared - 1 hot bits, and, when the hot peaks alone can
+// reach min_shared, unseen ones with that many, and clears the plane.  Lane l
+// of a warp takes 4 words at a time (16-byte reads).  When the queue is full
+// every warp stops where it is, the block scores the queue, and they go on.
+// Every thread calls it.
+__device__ __noinline__ void scan_plane(const SearchArgs& a, uint32_t pb, uint32_t x0, uint32_t x1, uint32_t words) {
+    SearchShared& sh = search_shared(a);
+    const SearchParts sp = search_parts(a.lay);
+    uint32_t* const plane = sp.plane;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const uint32_t min_shared = a.min_shared;
+    const int nslices = sh.nslices;
+    const bool hot_alone = sh.nhotpeaks >= (int)min_shared;
+    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+    const bool all = !hot_alone && (uint32_t)nslices + 1u == min_shared;   // the intersection of the plane and every slice
+    // below 5 the counts here are exact: nothing is left to check
+    const uint32_t need = kDirectNeed | (min_shared <= 4u ? 0u : min_shared - 1u);
+    const uint32_t step = 128u * nwarps;
+    uint32_t w = warp * 128u + 4u * lane;   // the lane's next words
+    uint32_t cand[4];
+    bool held = false;      // candidates of the last step are left (the queue was full)
+    // (entries outside the super-chunk may have set bits past its words)
+    for (uint32_t i = words + threadIdx.x; i < a.lay.plane_words; i += blockDim.x)
+        plane[((pb >> 5) + i) & (a.lay.plane_words - 1u)] = 0u;
+    for (;;) {
+        bool full = false;
+        while (held || w - 4u * lane < words) {   // warp-uniform
+            if (!held) {
+                uint4 v = zero4;
+                if (w < words) {
+                    uint4* const at = reinterpret_cast<uint4*>(plane + (((pb >> 5) + w) & (a.lay.plane_words - 1u)));
+                    v = *at;
+                    v = make_uint4(__brev(v.x), __brev(v.y), __brev(v.z), __brev(v.w));   // the plane's bits run from the top
+                    *at = zero4;
+                }
+                const bool look = w < words && (hot_alone || (v.x | v.y | v.z | v.w) != 0u);
+                if (all) {
+                    // (three slices' words in flight: min_shared is 4 in most searches)
+#pragma unroll 1
+                    for (int s = 0; s < nslices; s += 3) {
+                        const uint4 h0 = look ? __ldg(reinterpret_cast<const uint4*>(sh.slice[s] + (pb >> 5) + w)) : zero4;
+                        uint4 h1 = h0, h2 = h0;
+                        if (look && s + 1 < nslices) h1 = __ldg(reinterpret_cast<const uint4*>(sh.slice[s + 1] + (pb >> 5) + w));
+                        if (look && s + 2 < nslices) h2 = __ldg(reinterpret_cast<const uint4*>(sh.slice[s + 2] + (pb >> 5) + w));
+                        v.x &= h0.x & h1.x & h2.x, v.y &= h0.y & h1.y & h2.y;
+                        v.z &= h0.z & h1.z & h2.z, v.w &= h0.w & h1.w & h2.w;
+                    }
+                    cand[0] = v.x, cand[1] = v.y, cand[2] = v.z, cand[3] = v.w;
+                } else {
+                    // per peptide its hot bits' number: two low bits b1, b2, and b3 = 4 or more
+                    uint32_t b1[4] = {0u, 0u, 0u, 0u}, b2[4] = {0u, 0u, 0u, 0u}, b3[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 2
+                    for (int s = 0; s < nslices; ++s) {
+                        const uint4 h = look ? __ldg(reinterpret_cast<const uint4*>(sh.slice[s] + (pb >> 5) + w)) : zero4;
+                        const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
 #pragma unroll
-    for (int i = 0; i < PPT; ++i) {
-        const int t = tid * ppt + i;
-        if (i < ppt && t < nnorm) {
-            const uint32_t len = group_len(ra[i], rb[i]);
-            sh.pre[buf][t] = run;
-            sh.rs[buf][t] = group_start(ra[i]);
-            if (len)   // warps whose share starts inside this run
-                for (uint32_t w = (run + per - 1) / per; w * per < run + len && w < (uint32_t)nwarps; ++w)
-                    sh.wli[buf][w] = (uint16_t)t;
-            run += len;
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t k1 = b1[i] & hw[i];
+                            b1[i] ^= hw[i];
+                            b3[i] |= b2[i] & k1;
+                            b2[i] ^= k1;
+                        }
+                    }
+                    auto at_least = [](uint32_t c1, uint32_t c2, uint32_t c3, uint32_t t) {
+                        // (a superset for t above 4: the queue's check is exact)
+                        return t == 0 ? 0xffffffffu : t == 1 ? (c1 | c2 | c3) : t == 2 ? (c2 | c3)
+                               : t == 3 ? ((c2 & c1) | c3) : c3;
+                    };
+                    const uint32_t seen[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        cand[i] = seen[i] & at_least(b1[i], b2[i], b3[i], min_shared - 1u);
+                        if (hot_alone && look) cand[i] |= ~seen[i] & at_least(b1[i], b2[i], b3[i], min_shared);
+                    }
+                }
+            }
+            held = false;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t gp = pb + ((w + (uint32_t)i) << 5);
+                while (cand[i] && !held) {
+                    const uint32_t pid = gp + (uint32_t)__ffs(cand[i]) - 1u;
+                    if (pid - x0 < x1 - x0 && !push(a, sh, sp, pid, need)) held = true;   // (peptides [x0, x1) only)
+                    else cand[i] &= cand[i] - 1u;
+                }
+            }
+            held = __any_sync(0xffffffffu, held);
+            if (held) {
+                full = true;
+                break;
+            }
+            w += step;
+        }
+        if (!__syncthreads_or(full)) break;
+        drain_queue(a);
+    }
+}
+
+// A column [x0, x1) whose repeats overflow their list, with one 32-bit counter
+// a peptide, in parts of the plane's size (the plane is all zero before and
+// after).  The column's runs are in place.  Every thread calls it.
+__device__ __noinline__ void direct_column(const SearchArgs& a, uint32_t x0, uint32_t x1) {
+    SearchShared& sh = search_shared(a);
+    const SearchParts sp = search_parts(a.lay);
+    uint32_t* const plane = sp.plane;
+    const uint32_t tid = threadIdx.x, part = a.lay.plane_words;
+    const uint32_t min_shared = a.min_shared, nslices = (uint32_t)sh.nslices;
+    const bool hot_alone = sh.nhotpeaks >= (int)min_shared;
+    for (uint32_t pb = x0; pb < x1; pb += part) {
+        const uint32_t span = min(part, x1 - pb);
+        for (int t = 0; sp.runs[t].y != kNoEnd; ++t) {   // (the run without end closes the list)
+            const uint4 r = sp.runs[t];
+            for (uint32_t g = tid; g < r.y; g += blockDim.x) {
+                const uint4 e = __ldg(reinterpret_cast<const uint4*>(a.entry) + r.x + g);
+                const uint32_t e4[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t o = (e4[i] >> 1) - pb;   // (a pad is past every span)
+                    if (o < span) atomicAdd(&plane[o], 1u);
+                }
+            }
+        }
+        __syncthreads();
+        uint32_t i = tid;
+        for (;;) {
+            bool full = false;
+            for (; i < span; i += blockDim.x) {
+                const uint32_t ord = plane[i];
+                if (((ord && ord + nslices >= min_shared) || hot_alone) &&
+                    !push(a, sh, sp, pb + i, kDirectNeed | (ord < min_shared ? min_shared - ord : 0u))) {
+                    full = true;
+                    break;
+                }
+                plane[i] = 0u;
+            }
+            if (!__syncthreads_or(full)) break;
+            drain_queue(a);
         }
     }
-    if (tid == 0) sh.pre[buf][nnorm] = total;
 }
 
-template <int KMAX, int THREADS, int MAXP>
-__global__ void __launch_bounds__(THREADS, THREADS <= 384 ? 2 : 1) search_kernel(SearchArgs a) {
-    using L = Layout<KMAX, THREADS, MAXP>;
-    constexpr uint32_t kDynWords = L::kDynWords, kSlotWord = L::kSlotWord, kListWord = L::kListWord;
-    constexpr uint32_t kMaxRounds = L::kMaxRounds, kMaxCols = L::kMaxCols;
-    extern __shared__ __align__(16) uint32_t smem32[];   // kDynWords words (layout above)
-    uint32_t* const cnt = smem32;
-    uint32_t* const seen = smem32;
-    uint32_t* const lists = smem32 + kListWord;
-    unsigned long long* const tab = reinterpret_cast<unsigned long long*>(smem32 + kSlotWord);
-    __shared__ SearchShared<MAXP> sh;
-    uint16_t* const touched = L::kTouchDyn ? reinterpret_cast<uint16_t*>(smem32 + kChunk) : sh.touched;
+// A run [ra, rb) of a bucket (positions relative to its 16-byte aligned start
+// at group base) is read as whole groups of 4 entries.  The extra entries at
+// either end lie in the same bucket outside the run's columns, or are the
+// bucket's pad slots; both fall outside every peptide range the run is
+// searched for.  Its pieces are the 128-byte lines it touches: octets that
+// read whole lines take 61 cycles a step of two pieces from DRAM, octets
+// that straddle them 83 to 116 (measured on the reads and atomics alone).
+struct Run {
+    uint32_t start, len;   // first group, groups
+    __device__ __forceinline__ Run(uint32_t base, uint32_t ra, uint32_t rb)
+        : start(base + (ra >> 2)), len(ra == rb ? 0u : ((rb + 3u) >> 2) - (ra >> 2)) {}
+    __device__ __forceinline__ uint32_t pieces() const {
+        return len ? (start + len + kSub - 1u) / kSub - start / kSub : 0u;
+    }
+};
+
+// Predicated accesses of the pass over the entries, without branches.
+// 16-byte group g of the index when ok; the first word is all ones otherwise.
+__device__ __forceinline__ uint4 load_group(const uint32_t* entry, uint32_t g, bool ok) {
+    uint4 v;
+    v.x = 0xffffffffu;   // (the others stay what they are then)
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t@p ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(reinterpret_cast<const uint4*>(entry) + g), "r"((uint32_t)ok));
+    return v;
+}
+// stores v at shared address at when ok is not 0; the address behind it then
+__device__ __forceinline__ uint32_t put_shared(uint32_t at, uint32_t v, uint32_t ok) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.u32 [%0], %1;\n\t@p add.u32 %0, %0, 4;\n\t}"
+                 : "+r"(at) : "r"(v), "r"(ok) : "memory");
+    return at;
+}
+
+constexpr int search_min_ctas(int threads) { return threads <= 256 ? 3 : threads <= 384 ? 2 : 1; }
+
+template <int THREADS, int PPT>
+__global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kernel(const __grid_constant__ SearchArgs a) {
+    SearchShared& sh = search_shared(a);
     constexpr int nwarps = THREADS / 32;
-    constexpr int PPT = (MAXP + THREADS - 1) / THREADS;   // ordinary peaks per thread (at most)
-    constexpr int kListStride = (32 / nwarps + (32 % nwarps ? 1 : 0)) * 32;   // list words per warp
-    static_assert(kListStride * nwarps <= (int)kListWords, "compaction lists fit");
-    __shared__ WarpTop<KMAX> wtop[nwarps];
+    constexpr uint32_t nsub = THREADS / kSub;
+    constexpr int kG = 2;               // pieces in flight a thread
+    const SearchParts sp = search_parts(a.lay);
+    uint32_t* const plane = sp.plane;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    const uint32_t last_col = a.skip_stride - 1;
-    for (int i = tid; i < (int)kDynWords; i += THREADS) smem32[i] = 0u;
+    for (uint32_t i = tid; i < a.lay.plane_words; i += THREADS) plane[i] = 0u;
+    for (uint32_t i = tid; i < kSlots; i += THREADS) sp.tab[i] = 0u;
+    for (uint32_t i = tid; i < kPlane2Words; i += THREADS) sp.plane2[i] = 0u;
+    for (uint32_t i = tid; i < kHeads / 2; i += THREADS) sp.head[i] = 0u;
     for (int i = tid; i < (int)kHistBins; i += THREADS) sh.hist[i] = 0;
     for (int i = tid; i <= (int)kMaxLen; i += THREADS) sh.lf[i] = a.lf[i];
-    if (tid == 0) { sh.ncand[0] = 0u; sh.ncand[1] = 0u; }
-    if (tid < nwarps) wtop[tid].n = 0;
-    const uint64_t total_units = a.seg_off[a.n];
-    const int k = (int)a.k;
-    const uint32_t min_shared = a.min_shared;
-    int par = 0;                  // alternates per super-chunk: which ncand counts
-    uint32_t log_lo = kListWord, log_dirty = 0;   // words [log_lo, log_dirty) may hold log records
-    __syncthreads();
+    UnitState st;
+    st.slot = 0;
+    // (thread 0) the unit at place t of the order becomes the CTA's next one
+    auto set_unit = [&](uint64_t t) {
+        sh.have = t < *a.n_units;
+        if (sh.have) sh.unit[st.slot ^ 1u] = __ldg(a.unit + t);
+    };
+    if (tid == 0) {
+        set_unit(blockIdx.x);   // the first by block index, then the counter's
+        sh.nkeys = 0u;
+        sh.over = 0;
+    }
+    // The calls below take what registers they like: the unit's state waits in
+    // shared memory (every one of them has a barrier).
+    auto save = [&]() {
+        if (tid == 0) sh.st = st;
+    };
+    auto restore = [&]() { st = sh.st; };
     for (;;) {
         if (tid == 0) {
-            const uint64_t t = atomicAdd(a.work, 1ull);
-            const bool listed = t < total_units && a.order;
-            const uint64_t u = listed ? (uint64_t)a.order[t] : t;
-            sh.unit = u;
             sh.nnorm = 0;
             sh.nhotc = 0;
             sh.nslices = 0;
             sh.nhotpeaks = 0;
-            sh.ntouched = 0;
-            if (u < total_units) {
-                // spectrum owning unit u (without an order list: the last q
-                // with seg_off[q] <= u)
-                uint32_t lo_q = 0, hi_q = a.n;
-                if (listed) lo_q = a.order_q[t];
-                else
-                    while (hi_q - lo_q > 1) {
-                        const uint32_t m = (lo_q + hi_q) >> 1;
-                        if (a.seg_off[m] <= u) lo_q = m; else hi_q = m;
-                    }
-                const uint32_t q = lo_q;
-                const uint32_t s = (uint32_t)(u - a.seg_off[q]);
-                const uint32_t ns = (uint32_t)(a.seg_off[q + 1] - a.seg_off[q]);
-                const uint32_t W = a.hi[q] - a.lo[q];
-                const uint32_t len = (W + ns - 1) / ns;
-                sh.q = q;
-                sh.np = a.qn[q];
-                sh.seg_lo = a.lo[q] + s * len;
-                sh.seg_hi = min(a.hi[q], sh.seg_lo + len);
-            }
         }
         __syncthreads();
-        const uint64_t u = sh.unit;
-        if (u >= total_units) break;
-        const uint32_t q = sh.q, np = sh.np, seg_lo = sh.seg_lo, seg_hi = sh.seg_hi;
-        // classify the retained peaks: hot (bitmap) candidates or ordinary (skip table)
-        for (uint32_t t = tid; t < np; t += THREADS) {
-            const uint32_t bin = a.qbin[(uint64_t)q * a.topn + t];
-            if (a.hot_id[bin] >= 0) {
-                sh.hotc[atomicAdd(&sh.nhotc, 1)] = (uint16_t)t;
-                continue;
-            }
-            const int32_t row = a.skip_row[bin];
-            if (row < 0) continue;   // empty bucket
-            const int s = atomicAdd(&sh.nnorm, 1);
-            sh.pbase[s] = (uint32_t)(a.off[bin] >> 2);
-            sh.prow[s] = (uint32_t)row;
-            sh.pinc[s] = a.qiq[(uint64_t)q * a.topn + t];
-        }
-        __syncthreads();
-        if (warp == 0) {
-            // bitmap slices for the hot peaks while they last (warp 0, 32
-            // hot peaks at a time: lanes load their peaks' tables together,
-            // a prefix of slices needed picks the takers); the rest are
-            // streamed like ordinary peaks.  Which hot peaks get slices does
-            // not change any result.
-            int ns = 0, nh = 0;   // warp-uniform
-            const int nhc = sh.nhotc;
-            for (int c0 = 0; c0 < nhc; c0 += 32) {
-                const int c = c0 + lane;
-                const bool act = c < nhc;
-                uint32_t bin = 0, iq = 0, fl = 0;
-                int32_t hid = 0;
-                if (act) {
-                    const uint32_t t = sh.hotc[c];
-                    bin = a.qbin[(uint64_t)q * a.topn + t];
-                    iq = a.qiq[(uint64_t)q * a.topn + t];
-                    hid = a.hot_id[bin];
-                    fl = a.hot_flags[hid];
-                }
-                const int need = (fl & 1u ? 1 : 0) + (fl & 2u ? 1 : 0);
-                int incl = need;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int x = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += x;
-                }
-                const bool take = act && ns + incl <= kMaxHot;   // a prefix of the lanes
-                if (take) {
-                    int p = ns + incl - need;
-                    if (fl & 1u) { sh.slice[p] = a.hot_b + (uint64_t)hid * a.hot_words; sh.slice_inc[p++] = (1u << kNbShift) + iq; }
-                    if (fl & 2u) { sh.slice[p] = a.hot_y + (uint64_t)hid * a.hot_words; sh.slice_inc[p] = (1u << kNyShift) + iq; }
-                } else if (act) {
+        if (!sh.have) break;
+        st.slot ^= 1u;
+        if (tid < nwarps) sh.wn[tid] = 0;      // (nothing is appended or scored before the next barriers)
+        if (tid == 0) sh.nq = sh.npass = 0u;
+        st.taken = 0;
+        // the retained peaks: hot (bitmap) or ordinary (skip table), and all
+        // of them into the hash of the spectrum's bins
+        {
+            const uint32_t q = sh.unit[st.slot].x, np = a.qn[q];
+            const uint32_t* qb = a.qbin + (uint64_t)q * a.stride;
+            const uint32_t* qi = a.qiq + (uint64_t)q * a.stride;
+            for (uint32_t t = tid; t < np; t += THREADS) {
+                const uint32_t bin = qb[t], iq = qi[t];
+                const BinInfo bi = a.bins[bin];
+                // (the peak becomes its chain's head: half a word, so by compare and swap)
+                const uint32_t h = bin & (kHeads - 1u), half = 16u * (h & 1u);
+                uint32_t seen = sp.head[h >> 1], was;
+                do {
+                    was = seen;
+                    seen = atomicCAS(&sp.head[h >> 1], was, (was & ~(0xffffu << half)) | ((t + 1u) << half));
+                } while (seen != was);
+                sp.qpeak[t] = make_uint2(bin, iq);
+                sp.next[t] = (uint16_t)(was >> half);
+                if (bi.hot >= 0) {
+                    sp.hotc[atomicAdd(&sh.nhotc, 1)] = bin;
+                } else if (bi.row >= 0) {
                     const int s = atomicAdd(&sh.nnorm, 1);
-                    sh.pbase[s] = (uint32_t)(a.off[bin] >> 2);
-                    sh.prow[s] = (uint32_t)a.skip_row[bin];
-                    sh.pinc[s] = iq;
+                    sp.pbase[s] = bi.group;
+                    sp.prow[s] = (uint32_t)bi.row;
                 }
-                const unsigned tm = __ballot_sync(0xffffffffu, take);
-                nh += __popc(tm);
-                if (tm) ns += __shfl_sync(0xffffffffu, incl, 31 - __clz(tm));   // the last taker's prefix
-            }
-            if (lane == 0) {
-                sh.nslices = ns;
-                sh.nhotpeaks = nh;
             }
         }
         __syncthreads();
-        const int nnorm = sh.nnorm, nslices = sh.nslices;
-        const bool hot_alone = sh.nhotpeaks >= (int)min_shared;
-        // peptides hit once are candidates too when the hot slices alone can
-        // supply the other min_shared - 1 shared peaks
-        const bool once_counts = (uint32_t)nslices + 1u >= min_shared;
-        const int ppt = (nnorm + THREADS - 1) / THREADS;
-        const uint32_t col_lo = seg_lo >> kChunkShift, col_end = ((seg_hi - 1) >> kChunkShift) + 1;
-        uint32_t ra[PPT], rb[PPT];
-        auto load_runs = [&](uint32_t c0l, uint32_t c1l) {
+        if (sh.nhotc) {   // uniform
+            if (warp == 0) {
+                // Bitmap slices for the hot peaks, the densest first (a lane
+                // a hot peak, in rounds of an arg-max over their entries in
+                // the segment's columns).  With min_shared - 1 slices or more
+                // the plane has to be scanned for peptides of one ordinary hit
+                // or none, which costs what streaming 1/8 of the segment's
+                // peptides does: when the rest hold fewer entries, only
+                // min_shared - 2 slices are taken and the rest are streamed
+                // like ordinary peaks, as are those that get no slice at all.
+                // Which hot peaks get slices does not change any result.
+                const int nhc = sh.nhotc;
+                const uint32_t lo = sh.unit[st.slot].y, hi = sh.unit[st.slot].z;
+                const uint32_t c0 = lo >> kChunkShift, c1 = min(((hi - 1u) >> kChunkShift) + 1u, a.skip_stride - 1u);
+                int ns = 0, nh = 0;   // warp-uniform
+                for (int p0 = 0; p0 < nhc; p0 += 32) {   // (32 at a time: of more, the later ones are hardly ever taken)
+                    BinInfo bi{0u, -1, -1, 0u};
+                    uint32_t n = 0;
+                    bool left = p0 + lane < nhc;
+                    if (left) {
+                        bi = a.bins[sp.hotc[p0 + lane]];
+                        const uint32_t* sk = a.skip + (uint64_t)bi.row * a.skip_stride;
+                        n = __ldg(sk + c1) - __ldg(sk + c0);
+                    }
+                    const int need = (int)(bi.flags & 1u) + (int)((bi.flags >> 1) & 1u);
+                    float rest = (float)__reduce_add_sync(0xffffffffu, n >> 4) * 16.0f;   // entries of the peaks left
+                    bool open = true;
+                    while (open) {
+                        const uint32_t most = __reduce_max_sync(0xffffffffu, left ? n + 1u : 0u);
+                        if (!most) break;
+                        const int w = __ffs(__ballot_sync(0xffffffffu, left && n + 1u == most)) - 1;
+                        const int nd = __shfl_sync(0xffffffffu, need, w);
+                        // the cap: min_shared - 2 while the rest are few (all of them, not only these 32)
+                        const bool few = nhc <= 32 && rest < (float)(hi - lo) * 0.125f;
+                        if (ns + nd > (few ? min(kMaxHot, max((int)a.min_shared - 2, 0)) : kMaxHot)) open = false;
+                        if (open) {
+                            if (lane == w) {
+                                int p = ns;
+                                if (bi.flags & 1u) sh.slice[p++] = a.hot_b + (uint64_t)bi.hot * a.hot_words;
+                                if (bi.flags & 2u) sh.slice[p] = a.hot_y + (uint64_t)bi.hot * a.hot_words;
+                                left = false;
+                            }
+                            ns += nd;
+                            ++nh;
+                            rest -= (float)(most - 1u);
+                        }
+                    }
+                    if (left) {
+                        const int s = atomicAdd(&sh.nnorm, 1);
+                        sp.pbase[s] = bi.group;
+                        sp.prow[s] = (uint32_t)bi.row;
+                    }
+                }
+                if (lane == 0) {
+                    sh.nslices = ns;
+                    sh.nhotpeaks = nh;
+                }
+            }
+            __syncthreads();
+        }
+        // a thread owns the ordinary peaks tid * ppt .. + ppt - 1
+        auto skip_at = [&](uint32_t (&r)[PPT], uint32_t col) {
+            const int nnorm = sh.nnorm, ppt = (nnorm + THREADS - 1) / THREADS;
 #pragma unroll
             for (int i = 0; i < PPT; ++i) {
                 const int t = tid * ppt + i;
-                ra[i] = rb[i] = 0;
-                if (i < ppt && t < nnorm) {
-                    const uint32_t* sk = a.skip + (uint64_t)sh.prow[t] * a.skip_stride;
-                    ra[i] = __ldg(sk + c0l);
-                    rb[i] = __ldg(sk + min(c1l, last_col));
-                }
+                r[i] = 0;
+                if (i < ppt && t < nnorm)
+                    r[i] = __ldg(a.skip + (uint64_t)sp.prow[t] * a.skip_stride + min(col, a.skip_stride - 1u));
             }
         };
-        // columns per super-chunk, from the segment's total entries
-        uint32_t m = 1;
-        {
-            load_runs(col_lo, col_end);
-            uint32_t s = 0;
+        // Prefix of the runs' pieces (kSub groups each) and of the non-empty
+        // runs over the block, in two halves around a barrier.  A super-
+        // chunk's runs are [ra, rb) of the peaks' buckets.  Octet s of the
+        // block takes pieces [s per, (s + 1) per) of all; per is returned.
+        auto scan_1 = [&](const uint32_t (&ra)[PPT], const uint32_t (&rb)[PPT]) {
+            const int nnorm = sh.nnorm, ppt = (nnorm + THREADS - 1) / THREADS;
+            uint32_t sum = 0, cnt = 0;
 #pragma unroll
-            for (int i = 0; i < PPT; ++i) s += rb[i] - ra[i];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) sh.wsum[warp] = s;
-            __syncthreads();
-            uint32_t total = 0;
-#pragma unroll
-            for (int w = 0; w < nwarps; ++w) total += sh.wsum[w];
-            const uint32_t ncols = col_end - col_lo;
-            {
-                // about target_entries entries, and planes (1024 words a
-                // column) plus 1.25 times the mean log within kListWord
-                // words, so that denser-than-mean super-chunks still fit
-                uint64_t want = total ? ((uint64_t)a.target_entries * ncols) / total : ncols;
-                const uint64_t fit = (uint64_t)kListWord * ncols / ((uint64_t)1024 * ncols + total + total / 4);
-                if (want > fit) want = fit;
-                if (want < 1) want = 1;
-                if (want > kMaxCols) want = kMaxCols;
-                m = min((uint32_t)want, ncols);
-            }
-            __syncthreads();   // wsum is reused by the scans
-        }
-        // a lane's scored candidate waiting for its warp's list (flush)
-        int64_t pK = 0;
-        uint32_t pP = 0u, pC = 0u;
-        bool pend = false;
-        uint32_t* twice = smem32;   // the current super-chunk's twice plane and log
-        uint32_t* logw = smem32;
-
-        // Calls fn(f, entry, peak) for every entry f of parity buffer buf.
-        // Warp w takes a contiguous share; lane l takes f0 + l + 32 j, kJ
-        // loads in flight before any is used.  Each lane walks the runs
-        // forward, keeping the current run's end and the entry-array base
-        // gb (entry f of the run is entry[gb + f]) in registers.
-        auto for_each_entry = [&](int buf, auto&& fn) {
-            constexpr int kJ = 8;
-            const uint32_t R = sh.pre[buf][nnorm];
-            const uint32_t per = warp_share<THREADS>(R);
-            const uint32_t f0 = (uint32_t)warp * per, f1 = min(R, f0 + per);
-            if (f0 >= f1) return;
-            int li = sh.wli[buf][warp];
-            uint32_t nxt = sh.pre[buf][li + 1];
-            uint64_t gb = ((uint64_t)sh.pbase[li] << 2) + sh.rs[buf][li] - sh.pre[buf][li];
-            for (uint32_t fb = f0 + lane; fb < f1; fb += 32 * kJ) {
-                uint32_t ev[kJ];
-                uint32_t lp[kJ];
-#pragma unroll
-                for (int j = 0; j < kJ; ++j) {
-                    const uint32_t f = fb + 32 * j;
-                    ev[j] = 0xffffffffu;
-                    lp[j] = 0;
-                    if (f < f1) {
-                        while (f >= nxt) {
-                            ++li;
-                            nxt = sh.pre[buf][li + 1];
-                            gb = ((uint64_t)sh.pbase[li] << 2) + sh.rs[buf][li] - sh.pre[buf][li];
-                        }
-                        lp[j] = (uint32_t)li;
-                        ev[j] = __ldg(a.entry + (gb + f));
-                    }
+            for (int i = 0; i < PPT; ++i) {
+                const int t = tid * ppt + i;
+                if (i < ppt && t < nnorm && ra[i] != rb[i]) {
+                    sum += Run(sp.pbase[t], ra[i], rb[i]).pieces();
+                    ++cnt;
                 }
-#pragma unroll
-                for (int j = 0; j < kJ; ++j)
-                    if (fb + 32 * j < f1) fn(fb + 32 * j, ev[j], (int)lp[j]);
             }
+            uint2 incl = make_uint2(sum, cnt);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t x = __shfl_up_sync(0xffffffffu, incl.x, o), y = __shfl_up_sync(0xffffffffu, incl.y, o);
+                if (lane >= o) {
+                    incl.x += x;
+                    incl.y += y;
+                }
+            }
+            if (lane == 31) {
+                sh.wsum[warp] = incl.x;
+                sh.wruns[warp] = incl.y;
+            }
+            return make_uint2(incl.x - sum, incl.y - cnt);
         };
-        auto score = [&](uint32_t c, uint32_t pid) {
-            const uint32_t nb = c >> kNbShift, ny = (c >> kNyShift) & 63u;
-            if (nb + ny >= min_shared) {
-                uint32_t S = c & kSMask;
-                if (S > a.s_max) S = a.s_max;   // unreachable for a consistent index
-                const int64_t K = sh.lf[nb] + sh.lf[ny] + __ldg(a.ls + S);
-                const int64_t hb = K >> 31;
-                atomicAdd(&sh.hist[hb > 255 ? 255 : (hb < 0 ? 0 : hb)], 1u);
-                if (wtop[warp].passes(K, pid, k)) { pK = K; pP = pid; pC = c; pend = true; }
-            }
-        };
-        // pending candidates into the warp's list, one lane at a time; every
-        // lane of the warp calls it (convergent points only)
-        auto flush = [&]() {
-            unsigned pm = __ballot_sync(0xffffffffu, pend);
-            while (pm) {
-                const int l = __ffs(pm) - 1;
-                pm &= pm - 1;
-                if (lane == l) wtop[warp].insert(pK, pP, pC, k);
-                __syncwarp();
-            }
-            pend = false;
-        };
-        // one counter (c, pid): filter, add the hot slices, score
-        auto visit = [&](uint32_t c, uint32_t pid) {
-            const uint32_t nn = (c >> kNbShift) + ((c >> kNyShift) & 63u);
-            if (nn + (uint32_t)nslices < min_shared) return;
-            uint32_t hw[kMaxHot];   // every slice's word in flight at once
-#pragma unroll
-            for (int s = 0; s < kMaxHot; ++s) hw[s] = s < nslices ? __ldg(sh.slice[s] + (pid >> 5)) : 0u;
-#pragma unroll
-            for (int s = 0; s < kMaxHot; ++s)
-                if ((hw[s] >> (pid & 31)) & 1u) c += sh.slice_inc[s];
-            score(c, pid);
-        };
-
-        // ---- one column with direct counters (the caller provides the
-        // barriers before and after)
-        auto column_pass = [&](int buf, uint32_t cb, uint32_t x0, uint32_t x1) {
-            for_each_entry(buf, [&](uint32_t, uint32_t e, int li) {
-                const uint32_t pid = e >> 1;
-                bool first = false;
-                uint32_t off = 0;
-                if (pid >= x0 && pid < x1) {
-                    off = pid - cb;
-                    first = atomicAdd(&cnt[off], counter_inc_y(e & 1u, sh.pinc[li])) == 0u;
-                }
-                if (first) {
-                    const int slot = atomicAdd(&sh.ntouched, 1);
-                    if (slot < kTouchCap) touched[slot] = (uint16_t)off;
-                }
-            });
-            __syncthreads();
-            const int nt = sh.ntouched;
-            if (nt <= kTouchCap && !hot_alone) {
-                for (int i0 = warp * 32; i0 < nt; i0 += THREADS) {   // warp-uniform trip count
-                    const int i = i0 + lane;
-                    if (i < nt) {
-                        const uint32_t w = touched[i];
-                        const uint32_t c = cnt[w];
-                        cnt[w] = 0u;
-                        visit(c, cb + w);
-                    }
-                    flush();
-                }
-            } else {
-                // every counter, 32 peptide ids per step; bitmaps alone can
-                // qualify a peptide when hot_alone
-                for (uint32_t gi = tid; gi < kChunk / 32; gi += THREADS) {   // warp-uniform trip count
-                    const uint32_t gp = cb + (gi << 5);
-                    const bool act = !(gp + 32 <= x0 || gp >= x1);
-                    const uint32_t lo_b = x0 > gp ? x0 - gp : 0u;
-                    const uint32_t hi_b = x1 - gp >= 32u ? 32u : x1 - gp;
-                    const uint32_t valid = (hi_b >= 32u ? 0xffffffffu : ((1u << hi_b) - 1u)) & ~((1u << lo_b) - 1u);
-                    uint32_t hw[kMaxHot];
-#pragma unroll
-                    for (int s = 0; s < kMaxHot; ++s) hw[s] = act && s < nslices ? __ldg(sh.slice[s] + (gp >> 5)) : 0u;
-                    uint32_t cand = 0;
-                    for (int j = 0; act && j < 32; ++j) {
-                        const int jb = (j + lane) & 31;   // rotated: lanes hit different banks
-                        const uint32_t c = cnt[(gi << 5) + jb];
-                        uint32_t hc = 0;
-#pragma unroll
-                        for (int s = 0; s < kMaxHot; ++s) hc += (hw[s] >> jb) & 1u;
-                        const uint32_t nn = (c >> kNbShift) + ((c >> kNyShift) & 63u);
-                        if ((c != 0u || hc > 0u) && nn + hc >= min_shared) cand |= 1u << jb;
-                    }
-                    cand &= act ? valid : 0u;
-                    while (__any_sync(0xffffffffu, cand != 0u)) {   // one candidate a lane per step
-                        if (cand) {
-                            const int jb = __ffs(cand) - 1;
-                            cand &= cand - 1;
-                            uint32_t c = cnt[(gi << 5) + jb];
-#pragma unroll
-                            for (int s = 0; s < kMaxHot; ++s)
-                                if ((hw[s] >> jb) & 1u) c += sh.slice_inc[s];
-                            score(c, gp + jb);
-                        }
-                        flush();
-                    }
-                    if (act) {
-#pragma unroll 4
-                        for (int j = 0; j < 32; ++j) cnt[(gi << 5) + ((j + lane) & 31)] = 0u;
-                    }
-                }
-            }
-            __syncthreads();
-            if (tid == 0) sh.ntouched = 0;
-        };
-
-        // ---- a super-chunk in passes (see the header); entries of parity
-        // buffer buf, peptide ids [x0, x1) of the span starting at cb
-        // Pass A over the entries of parity buffer buf (the walk of
-        // for_each_entry, specialised to groups): lane l of a warp takes the
-        // 4-entry groups starting at f0 + 4 l + 128 j, each one 16-byte load,
-        // kG groups in flight before any is used; then per entry the
-        // seen-plane atomic, one 16-byte store of the group's 4 log records,
-        // and the twice-plane atomics of second hits, so latencies overlap.
-        // A log record is (entry - 2 cb) | peak << 19, i.e. offset << 1 |
-        // isY in bits 0..18; entries outside [x0, x1) log 0xffffffff.
-        auto pass_a = [&](int buf, uint32_t cb, uint32_t x0, uint32_t x1, int par) {
-            constexpr int kG = 4;
-            const uint32_t R = sh.pre[buf][nnorm];                 // a multiple of 4
-            const uint32_t per = warp_share<THREADS>(R);           // a multiple of 4
-            const uint32_t f0 = (uint32_t)warp * per, f1 = min(R, f0 + per);
-            uint32_t fresh = 0;   // twice bits this lane set first
-            if (f0 < f1) {
-                int li = sh.wli[buf][warp];
-                uint32_t nxt = sh.pre[buf][li + 1];
-                const uint32_t* gp = a.entry + (((uint64_t)sh.pbase[li] << 2) + sh.rs[buf][li] - sh.pre[buf][li]);
-                uint32_t lsh = (uint32_t)li << 19;
-                // entries of pids in [x0, x1): e - e_lo < e_span (unsigned)
-                const uint32_t e_lo = x0 << 1, e_span = (x1 - x0) << 1, e_cb = cb << 1;
-                uint4* const log4 = reinterpret_cast<uint4*>(logw);
-                for (uint32_t fb = f0 + 4u * lane; fb < f1; fb += 128u * kG) {
-                    uint4 ev[kG];
-                    uint32_t lr[kG];
-#pragma unroll
-                    for (int g = 0; g < kG; ++g) {
-                        const uint32_t f = fb + 128u * g;
-                        ev[g] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
-                        lr[g] = 0u;
-                        if (f < f1) {
-                            while (f >= nxt) {
-                                ++li;
-                                nxt = sh.pre[buf][li + 1];
-                                gp = a.entry + (((uint64_t)sh.pbase[li] << 2) + sh.rs[buf][li] - sh.pre[buf][li]);
-                                lsh = (uint32_t)li << 19;
-                            }
-                            lr[g] = lsh;
-                            ev[g] = __ldg(reinterpret_cast<const uint4*>(gp + f));   // 16-byte aligned
-                        }
-                    }
-#pragma unroll
-                    for (int g = 0; g < kG; ++g) {
-                        const uint32_t f = fb + 128u * g;
-                        const uint32_t e4[4] = {ev[g].x, ev[g].y, ev[g].z, ev[g].w};
-                        uint32_t rec[4], old[4], bitv[4], wd[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const bool in = e4[i] - e_lo < e_span;
-                            const uint32_t o2 = e4[i] - e_cb;
-                            bitv[i] = in ? __funnelshift_l(0u, 1u, o2 >> 1) : 0u;   // 1 << (offset & 31)
-                            wd[i] = o2 >> 6;
-                            old[i] = in ? atomicOr(&seen[wd[i]], bitv[i]) : 0u;
-                            rec[i] = in ? (o2 | lr[g]) : 0xffffffffu;
-                        }
-                        if (f < f1) log4[f >> 2] = make_uint4(rec[0], rec[1], rec[2], rec[3]);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            if (old[i] & bitv[i]) fresh += (atomicOr(&twice[wd[i]], bitv[i]) & bitv[i]) ? 0u : 1u;
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) fresh += __shfl_xor_sync(0xffffffffu, fresh, o);
-            if (lane == 0 && fresh) atomicAdd(&sh.ncand[par], fresh);
-        };
-        // candidate plane (twice, plus peptides seen once with enough hot
-        // bits when once_counts), its count and the rounds; clears the seen
-        // plane.  Warp w owns words [w * wpw, (w + 1) * wpw), lane l every
-        // 32nd of them (barriers inside).
-        auto mark = [&](uint32_t cb, uint32_t words, uint32_t x0, uint32_t x1) {
-            const uint32_t G = words >> 5;          // groups of 32 plane words, split evenly over the warps
-            const uint32_t g0 = (uint32_t)warp * G / nwarps, g1 = (uint32_t)(warp + 1) * G / nwarps;
-            const uint32_t wbeg = g0 << 5, wpw = (g1 - g0) << 5;
-            uint32_t mine = 0;
-            // lane l takes the 4 words wbeg + i0 + 4 l (i0 = 0, 128, ...:
-            // warp-uniform trips): 16-byte plane reads, and one 16-byte
-            // bitmap read per hot slice, all slices' reads in flight together
-            const uint32_t need = min_shared - 1;   // <= nslices <= kMaxHot when once_counts
-            for (uint32_t i0 = 0; i0 < wpw; i0 += 128u) {
-                const uint32_t w = wbeg + i0 + 4u * lane;
-                const bool act = i0 + 4u * lane < wpw;
-                uint4 s4 = make_uint4(0u, 0u, 0u, 0u), c4 = s4;
-                if (act) {
-                    s4 = *reinterpret_cast<const uint4*>(seen + w);
-                    c4 = *reinterpret_cast<const uint4*>(twice + w);
-                }
-                const bool any_s = (s4.x | s4.y | s4.z | s4.w) != 0u;
-                if (any_s) *reinterpret_cast<uint4*>(seen + w) = make_uint4(0u, 0u, 0u, 0u);
-                uint32_t ho[4] = {0u, 0u, 0u, 0u};   // hot_alone: peptides of no ordinary hit that qualify
-                if (act && once_counts && (any_s || hot_alone)) {
-                    uint4 h[kMaxHot];
-#pragma unroll
-                    for (int sl = 0; sl < kMaxHot; ++sl)
-                        h[sl] = sl < nslices ? __ldg(reinterpret_cast<const uint4*>(sh.slice[sl] + (cb >> 5) + w))
-                                             : make_uint4(0u, 0u, 0u, 0u);
-                    // per peptide its hot-bit count (b1, b2: the two low bits,
-                    // b3: 4 or more): seen once with at least need hot bits
-                    // joins the candidates; seen never with at least
-                    // min_shared is scored here (supersets for need or
-                    // min_shared above 3: visit() is exact)
-                    auto at_least = [](uint32_t b1, uint32_t b2, uint32_t b3, uint32_t t) {
-                        if (t == 0) return 0xffffffffu;
-                        if (t == 1) return b1 | b2 | b3;
-                        if (t == 2) return b2 | b3;
-                        if (t == 3) return (b2 & b1) | b3;
-                        return b3;
-                    };
-                    auto word = [&](uint32_t s1, uint32_t& c2, uint32_t& hot_only, auto pick) {
-                        uint32_t b1 = 0, b2 = 0, b3 = 0;
-#pragma unroll
-                        for (int sl = 0; sl < kMaxHot; ++sl) {
-                            const uint32_t hh = pick(h[sl]);
-                            const uint32_t k1 = b1 & hh;
-                            b1 ^= hh;
-                            const uint32_t k2 = b2 & k1;
-                            b2 ^= k1;
-                            b3 |= k2;
-                        }
-                        c2 |= s1 & at_least(b1, b2, b3, need);
-                        if (hot_alone) hot_only = ~s1 & at_least(b1, b2, b3, min_shared);
-                    };
-                    word(s4.x, c4.x, ho[0], [](const uint4& v) { return v.x; });
-                    word(s4.y, c4.y, ho[1], [](const uint4& v) { return v.y; });
-                    word(s4.z, c4.z, ho[2], [](const uint4& v) { return v.z; });
-                    word(s4.w, c4.w, ho[3], [](const uint4& v) { return v.w; });
-                    if (any_s) *reinterpret_cast<uint4*>(twice + w) = c4;
-                }
-                mine += __popc(c4.x) + __popc(c4.y) + __popc(c4.z) + __popc(c4.w);
-                if (hot_alone) {
-                    // score them now (they are in no log), inside [x0, x1)
-#pragma unroll
-                    for (int kw = 0; kw < 4; ++kw) {
-                        const uint32_t gp = cb + ((w + (uint32_t)kw) << 5);
-                        const uint32_t lo_b = x0 > gp ? min(x0 - gp, 32u) : 0u;
-                        const uint32_t hi_b = x1 > gp ? min(x1 - gp, 32u) : 0u;
-                        const uint32_t valid = (hi_b >= 32u ? 0xffffffffu : ((1u << hi_b) - 1u)) &
-                                               ~(lo_b >= 32u ? 0xffffffffu : ((1u << lo_b) - 1u));
-                        uint32_t msk = ho[kw] & valid;
-                        while (__any_sync(0xffffffffu, msk != 0u)) {
-                            if (msk) {
-                                const int b = __ffs(msk) - 1;
-                                msk &= msk - 1;
-                                visit(0u, gp + (uint32_t)b);
-                            }
-                            flush();
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
-            if (lane == 0) sh.wcand[warp] = mine;
-            // a round whose first word is never found is empty: it starts at words
-            for (int r = tid; r <= (int)kMaxRounds; r += THREADS) sh.wb[r] = r == 0 ? 0 : (uint16_t)words;
-            __syncthreads();
-            uint32_t run = 0, total = 0;
+        auto scan_2 = [&](uint2 run, const uint32_t (&ra)[PPT], const uint32_t (&rb)[PPT]) {
+            const int nnorm = sh.nnorm, ppt = (nnorm + THREADS - 1) / THREADS;
+            uint32_t total = 0, nruns = 0;
 #pragma unroll
             for (int w = 0; w < nwarps; ++w) {
-                if (w < warp) run += sh.wcand[w];
-                total += sh.wcand[w];
+                const uint32_t p = sh.wsum[w], r = sh.wruns[w];
+                if (w < warp) {
+                    run.x += p;
+                    run.y += r;
+                }
+                total += p;
+                nruns += r;
             }
-            // round r holds the words with r * kRound <= candidates-before < (r + 1) * kRound;
-            // one round (the common case) starts at word 0 and needs no scan
-            for (uint32_t i0 = 0; total > kRound && i0 < wpw; i0 += 32) {
-                const uint32_t w = wbeg + i0 + lane;
-                const uint32_t cw = __popc(twice[w]);
-                uint32_t incl = cw;
+            const uint32_t per = (total + nsub - 1u) / nsub;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += x;
-                }
-                const uint32_t before = run + incl - cw;
-                const uint32_t r = before / kRound;
-                if (r > 0 && (before - __popc(twice[w - 1])) / kRound < r) sh.wb[r] = (uint16_t)w;
-                run += __shfl_sync(0xffffffffu, incl, 31);
-            }
-            if (tid == 0) sh.nrounds = (int)(total ? (total - 1) / kRound + 1 : 0);
-            __syncthreads();
-        };
-        // Replay of the log: 4 records per thread in flight, then their
-        // twice-plane words; a candidate's record goes to its warp's queue
-        // (the warp's compaction-list words, free until the epilogue), and a
-        // full queue is inserted into the table with every lane busy, so the
-        // insert loop never runs for one or two lanes.  The loop is
-        // warp-uniform (i0 - lane is the warp's first index).
-        auto replay = [&](uint32_t R, uint32_t wlo, uint32_t whi) {
-            constexpr int kU = 4;
-            uint32_t* const queue = lists + (uint32_t)warp * kListStride;
-            uint32_t qn = 0;
-            auto flush = [&]() {
-                __syncwarp();   // the other lanes' appends are visible
-                for (uint32_t j = lane; j < qn; j += 32) {
-                    const uint32_t r = queue[j];
-                    const uint32_t off = (r & 0x7ffffu) >> 1;
-                    const uint32_t v = counter_inc_y(r & 1u, sh.pinc[r >> 19]);
-                    const unsigned long long item = ((unsigned long long)off << 32) | v;
-                    uint32_t sl = slot_of(off);
-                    for (uint32_t probe = 0; probe < kSlots; ++probe) {
-                        const unsigned long long old = atomicCAS(&tab[sl], 0ull, item);
-                        if (old == 0ull) break;
-                        if ((uint32_t)(old >> 32) == off) { atomicAdd(&tab[sl], (unsigned long long)v); break; }
-                        sl = (sl + 1) & (kSlots - 1);
-                    }
-                }
-                __syncwarp();
-                qn = 0;
-            };
-            for (uint32_t i0 = tid; i0 - lane < R; i0 += kU * THREADS) {
-                uint32_t rec[kU], tw[kU];
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const uint32_t i = i0 + u * THREADS;
-                    rec[u] = i < R ? logw[i] : 0xffffffffu;
-                }
-#pragma unroll
-                for (int u = 0; u < kU; ++u)
-                    tw[u] = rec[u] != 0xffffffffu ? twice[(rec[u] & 0x7ffffu) >> 6] : 0u;
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    const uint32_t off = (rec[u] & 0x7ffffu) >> 1;
-                    const uint32_t w = off >> 5;
-                    const bool cand = rec[u] != 0xffffffffu && ((tw[u] >> (off & 31)) & 1u) && w >= wlo && w < whi;
-                    const unsigned msk = __ballot_sync(0xffffffffu, cand);
-                    if (qn + 32 > (uint32_t)kListStride) flush();
-                    if (cand) queue[qn + __popc(msk & lt)] = rec[u];
-                    qn += __popc(msk);
+            for (int i = 0; i < PPT; ++i) {
+                const int t = tid * ppt + i;
+                if (i < ppt && t < nnorm && ra[i] != rb[i]) {
+                    const Run r(sp.pbase[t], ra[i], rb[i]);
+                    const uint32_t len = r.pieces();
+                    sp.runs[run.y] = make_uint4(r.start, r.len, 0u - r.start % kSub, 0u);
+                    for (uint32_t s = (run.x + per - 1u) / per; s * per < run.x + len; ++s)   // the octets that start here
+                        sp.subs[s] = make_uint2(run.y, s * per - run.x);
+                    run.x += len;
+                    ++run.y;
                 }
             }
-            flush();
-        };
-        // Visits the occupied slots.  Warp w compacts the occupied slot
-        // indices of its share [w * spw, (w + 1) * spw) into its list words,
-        // visits them with all lanes, and zeroes the slots and the list.
-        auto slots_epilogue = [&](uint32_t cb) {
-            const uint32_t base = (uint32_t)warp * kListStride;
-            uint32_t cnt = 0;
-            for (uint32_t g = warp; g < kSlots / 32; g += nwarps) {   // groups of 32 slots
-                const uint32_t sl = (g << 5) + lane;
-                const bool occ = tab[sl] != 0ull;
-                const unsigned msk = __ballot_sync(0xffffffffu, occ);
-                if (occ) lists[base + cnt + __popc(msk & lt)] = sl;
-                cnt += __popc(msk);
+            if (tid == 0) {
+                sp.runs[nruns] = make_uint4(0u, kNoEnd, 0u, 0u);
+                sh.per = per;
+                sh.total = total;
             }
-            __syncwarp();
-            for (uint32_t i0 = 0; i0 < cnt; i0 += 32) {
-                const uint32_t i = i0 + lane;
-                if (i < cnt) {
-                    const uint32_t sl = lists[base + i];
-                    const unsigned long long v = tab[sl];
-                    tab[sl] = 0ull;
-                    visit((uint32_t)v, cb + (uint32_t)(v >> 32));
-                }
-                flush();
-            }
-            __syncwarp();
-            for (uint32_t i0 = 0; i0 < (uint32_t)kListStride; i0 += 32) lists[base + i0 + lane] = 0u;
         };
-        // zeroes plane words [w0, w1), both multiples of 4
-        auto clear_words = [&](uint32_t* plane, uint32_t w0, uint32_t w1) {
-            uint4* p4 = reinterpret_cast<uint4*>(plane);
-            for (uint32_t i = w0 / 4 + tid; i < w1 / 4; i += THREADS) p4[i] = make_uint4(0u, 0u, 0u, 0u);
-        };
-        // prologue: bounds of the first super-chunk
-        uint32_t c = col_lo;
-        uint32_t e = min(col_lo + m, col_end);
-        int buf = 0;
-        load_runs(c, e);
+        // Columns per super-chunk: what the plane holds (one bit a peptide),
+        // about target_entries entries, and about kKeysAim repeats.  The
+        // repeats of a window of W peptides and n entries are about n n / W
+        // (twice what independent hits would give: measured 1.9 to 2.4 on the
+        // workloads' databases).  When a peptide of one ordinary hit cannot
+        // qualify and the window needs several such super-chunks, they are
+        // made wider than the plane (deep): peptides that share a bit only
+        // add repeats, about n n / 2 bits.  A repeat whose peptide needs three
+        // ordinary hits or more then has to find its bit in the second plane
+        // set (by an earlier repeat of its own, or of one that shares that
+        // bit) before it counts, so the table only sees what is left of them,
+        // and a peptide's ordinary hits are at most its count + 2.  The hits
+        // that score are exact in any case.
+        const uint32_t col_end = ((sh.unit[st.slot].z - 1) >> kChunkShift) + 1;
+        st.c = sh.unit[st.slot].y >> kChunkShift;
+        st.deep = 0;
         {
-            const uint32_t excl = scan_runs_1<PPT>(sh, nnorm, ppt, ra, rb);
+            uint32_t r0[PPT], r1[PPT];
+            skip_at(r0, st.c);
+            skip_at(r1, col_end);
+            uint32_t s = 0;
+#pragma unroll
+            for (int i = 0; i < PPT; ++i) s += r1[i] - r0[i];
+            s = __reduce_add_sync(0xffffffffu, s);
+            if (lane == 0) sh.wsum[warp] = s;
             __syncthreads();
-            scan_runs_2<THREADS, PPT>(sh, buf, nnorm, ppt, excl, ra, rb);
-        }
-        __syncthreads();
-        while (c < col_end) {
-            const uint32_t R = sh.pre[buf][nnorm];
-            const uint32_t words = ((e - c) << kChunkShift) >> 5;
-            const bool direct = 2 * words + R > kListWord;
-            // words [log_lo, log_dirty) may hold old log records: clear them
-            // before they become counters or this super-chunk's planes
-            if (log_dirty > log_lo && (direct || 2 * words > log_lo)) {
-                for (uint32_t i = log_lo + tid; i < log_dirty; i += THREADS) smem32[i] = 0u;
-                log_lo = kListWord;
-                log_dirty = 0;
-                __syncthreads();
+            float total = 0.0f;
+#pragma unroll
+            for (int w = 0; w < nwarps; ++w) total += (float)sh.wsum[w];
+            const uint32_t ncols = max(col_end - st.c, 1u);
+            const float per = total / (float)ncols;                   // entries a column
+            const float rep = per * per / (float)kChunk;              // repeats a column
+            auto cols = [&](float aim, float bits, uint32_t most) {   // rep m + (per m)^2 / 2 bits = aim
+                const float q = bits > 0.0f ? per * per / (2.0f * bits) : 0.0f;
+                float w = q > 0.0f ? (sqrtf(rep * rep + 4.0f * q * aim) - rep) / (2.0f * q) : aim / fmaxf(rep, 1e-6f);
+                w = fminf(w, (float)a.target_entries / fmaxf(per, 1e-6f));
+                return (uint32_t)fmaxf(1.0f, fminf(w, (float)min(most, ncols)));
+            };
+            st.m = cols((float)kKeysAim, 0.0f, a.lay.plane_words / (kChunk / 32));
+            if ((uint32_t)sh.nslices + 2u <= a.min_shared && st.m < ncols) {
+                const uint32_t md = cols(kPlane2Aim, 32.0f * (float)a.lay.plane_words, (1u << kOffBits) / kChunk - 1u);
+                if (md > st.m) {
+                    st.m = md;
+                    st.deep = 1;
+                }
             }
-            if (direct) {
-                // column by column with direct counters
-                if (e - c == 1) {
-                    const uint32_t cb = c << kChunkShift;
-                    column_pass(buf, cb, max(seg_lo, cb), min(seg_hi, cb + kChunk));
-                    __syncthreads();
-                } else {
-                    for (uint32_t cc = c; cc < e; ++cc) {
-                        load_runs(cc, cc + 1);
-                        const uint32_t excl = scan_runs_1<PPT>(sh, nnorm, ppt, ra, rb);
-                        __syncthreads();
-                        scan_runs_2<THREADS, PPT>(sh, buf ^ 1, nnorm, ppt, excl, ra, rb);
-                        __syncthreads();
-                        const uint32_t cb = cc << kChunkShift;
-                        column_pass(buf ^ 1, cb, max(seg_lo, cb), min(seg_hi, cb + kChunk));
-                        __syncthreads();
+            const uint32_t nsc = (ncols + st.m - 1u) / st.m;          // even super-chunks
+            st.m = (ncols + nsc - 1u) / nsc;
+            __syncthreads();   // wsum is reused by the scans
+        }
+        // the unit taken next, once the last super-chunk comes up (and once a
+        // unit, though its end may be redone)
+        auto take_unit = [&]() {
+            if (st.e == col_end && !st.taken) {
+                st.taken = 1;
+                if (tid == 0) sh.t_next = (uint64_t)gridDim.x + atomicAdd(a.work, 1ull);
+            }
+        };
+        // the first super-chunk from column st.c on
+        auto start = [&]() {
+            uint32_t r0[PPT], r1[PPT];
+            st.e = min(st.c + st.m, col_end);
+            take_unit();
+            skip_at(r0, st.c);
+            skip_at(r1, st.e);
+            const uint2 excl = scan_1(r0, r1);
+            __syncthreads();
+            scan_2(excl, r0, r1);
+            __syncthreads();
+        };
+        if (st.c < col_end) start();
+        while (st.c < col_end) {
+            const uint32_t x0 = max(sh.unit[st.slot].y, st.c << kChunkShift);
+            const uint32_t x1 = (uint32_t)min((uint64_t)sh.unit[st.slot].z, (uint64_t)st.e << kChunkShift);
+            const uint32_t pb = x0 & ~127u;                       // the plane's first peptide
+            // plane words in use
+            const uint32_t words = min(((x1 - pb + 127u) >> 5) & ~3u, a.lay.plane_words);
+            // ---- pass A.  kSub lanes take a contiguous share of the runs'
+            // pieces, one 16-byte group of 4 entries a lane and piece, kG
+            // pieces in flight, two at a time through the plane.
+            const uint32_t per = sh.per;
+            const uint32_t oct = (uint32_t)tid / kSub, sl = (uint32_t)tid % kSub;
+            const uint32_t mine = oct * per < sh.total ? min(per, sh.total - oct * per) : 0u;   // the octet's pieces
+            const uint4* run = sp.runs;                  // the next piece's run
+            uint4 cur = make_uint4(0u, kNoEnd, 0u, 0u);  // cur.z: the piece's first group, from the run's
+            if (mine) {
+                const uint2 at = sp.subs[oct];
+                run += at.x;
+                cur = *run;
+                cur.z += at.y * kSub;
+            }
+            const bool more = st.e < col_end;
+            uint32_t r1[PPT], r2[PPT];                            // the next super-chunk's runs
+            if (more) {
+                skip_at(r1, st.e);                                // in flight during pass A
+                skip_at(r2, min(st.e + st.m, col_end));
+            }
+            // Peptide pid has bit 31 - pid % 32 of the plane's word pid / 32
+            // modulo its words, so that a left shift by pid brings it to the
+            // sign.  Entries past the super-chunk's end or before its start (a
+            // run's rounding, a bucket's pads) set bits like any other: they
+            // can only add repeats, and theirs are left out of the count.
+            const uint32_t mask = 4u * a.lay.plane_words - 4u;   // of byte addresses
+            uint32_t* const wq = sp.wq + warp * kWarpQueue;
+            uint32_t qn = 0;                                     // repeats in the warp's queue
+            for (uint32_t done = 0;; done += (uint32_t)kG) {     // (the same trips in every thread)
+                uint4 ev[kG];
+                uint32_t rep = 0;                                // bit 4 kG - 1 - i: entry i's bit was set before
+                const bool last = done >= per;
+                if (!last) {
+#pragma unroll
+                    for (int j = 0; j < kG; ++j) {
+                        const uint4 nx = run[1];
+                        if ((int)cur.z >= (int)cur.y) {
+                            ++run;
+                            cur = nx;
+                        }
+                        ev[j] = load_group(a.entry, cur.x + cur.z + sl, done + (uint32_t)j < mine && cur.z + sl < cur.y);
+                        cur.z += kSub;
+                    }
+#pragma unroll
+                    for (int j = 0; j < kG; ++j) {
+                        // (a group inside a run starts with a real entry)
+                        const uint32_t top = ev[j].x != 0xffffffffu ? 0x80000000u : 0u;
+                        const uint32_t en[4] = {ev[j].x, ev[j].y, ev[j].z, ev[j].w};
+                        uint32_t old[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            old[i] = atomicOr(reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(plane) + ((en[i] >> 4) & mask)),
+                                              __funnelshift_r(top, 0u, en[i] >> 1));
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            rep = __funnelshift_l(__funnelshift_l(0u, old[i], en[i] >> 1), rep, 1);
+                        if (!top) rep &= ~15u;
                     }
                 }
-                c = e;
-                if (c < col_end) {
-                    e = min(c + m, col_end);
-                    load_runs(c, e);
-                    const uint32_t excl = scan_runs_1<PPT>(sh, nnorm, ppt, ra, rb);
-                    __syncthreads();
-                    scan_runs_2<THREADS, PPT>(sh, buf, nnorm, ppt, excl, ra, rb);
-                    __syncthreads();
+                do {
+                    // places in the queue: a prefix over the lanes' counts, bit
+                    // by bit; more than it holds go one a lane at a time
+                    uint32_t take = rep, n1 = 0, total = 0;
+                    const uint32_t n = __popc(rep);
+                    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+                    for (int b = 0; b < 5; ++b) {
+                        const unsigned m = __ballot_sync(0xffffffffu, (n >> b) & 1u);
+                        n1 += (uint32_t)__popc(m & lt) << b;
+                        total += (uint32_t)__popc(m) << b;
+                    }
+                    if (total > kWarpQueue) {
+                        take = rep & (0u - rep);
+                        const unsigned m = __ballot_sync(0xffffffffu, take != 0u);
+                        n1 = (uint32_t)__popc(m & lt);
+                        total = (uint32_t)__popc(m);
+                    }
+                    // the warp's queue into the table, when these do not fit and at the end
+                    if (qn && (last || qn + total > kWarpQueue)) {
+                        __syncwarp();
+                        // kR repeats a lane, their hot words and second-plane
+                        // atomics in flight together
+                        constexpr int kR = (kWarpQueue + 31) / 32;
+                        uint32_t pid[kR], h = 0, in = 0;   // h: four bits of hot bits a repeat; in: those that count
+#pragma unroll
+                        for (int r = 0; r < kR; ++r) {
+                            pid[r] = lane + 32u * r < qn ? wq[lane + 32u * r] >> 1 : x1;
+                            if (pid[r] - x0 < x1 - x0) in |= 1u << r;      // inside the super-chunk
+                        }
+                        if (st.deep) {
+                            const uint32_t nslices = (uint32_t)sh.nslices;
+                            if (nslices + 2u == a.min_shared)              // else three hits are needed in any case
+                                for (uint32_t s = 0; s < nslices; ++s) {
+                                    uint32_t hw[kR];
+#pragma unroll
+                                    for (int r = 0; r < kR; ++r)
+                                        hw[r] = (in >> r) & 1u ? __ldg(sh.slice[s] + (pid[r] >> 5)) : 0u;
+#pragma unroll
+                                    for (int r = 0; r < kR; ++r) h += ((hw[r] >> (pid[r] & 31u)) & 1u) << (4 * r);
+                                }
+                            uint32_t old[kR];
+#pragma unroll
+                            for (int r = 0; r < kR; ++r) {
+                                const uint32_t x = hash_u32(pid[r]);
+                                old[r] = 0xffffffffu;
+                                if (((in >> r) & 1u) && ((h >> (4 * r)) & 15u) + 2u < a.min_shared)
+                                    old[r] = atomicOr(&sp.plane2[x >> (32 - kPlane2Bits)], 1u << ((x >> 15) & 31u));
+                            }
+#pragma unroll
+                            for (int r = 0; r < kR; ++r)
+                                if (!((old[r] >> ((hash_u32(pid[r]) >> 15) & 31u)) & 1u)) in &= ~(1u << r);
+                        }
+                        while (__any_sync(0xffffffffu, in != 0u)) {        // few are left: one a lane and step
+                            uint32_t p = 0;
+#pragma unroll
+                            for (int r = kR - 1; r >= 0; --r)
+                                if ((in >> r) & 1u) p = pid[r];
+                            if (in) add_repeat(sh, sp, p - pb);
+                            in &= in - 1u;
+                        }
+                        __syncwarp();
+                        qn = 0;
+                    }
+                    if (total) {
+                        uint32_t to = (uint32_t)__cvta_generic_to_shared(wq) + 4u * (qn + n1);
+#pragma unroll
+                        for (int i = 0; i < 4 * kG; ++i) {
+                            const uint4& v = ev[i / 4];
+                            to = put_shared(to, i % 4 == 0 ? v.x : i % 4 == 1 ? v.y : i % 4 == 2 ? v.z : v.w,
+                                            take & (1u << (4 * kG - 1 - i)));
+                        }
+                        qn += total;
+                    }
+                    rep &= ~take;
+                } while (__any_sync(0xffffffffu, rep != 0u));
+                if (last) break;
+            }
+            if (!more && tid == 0) set_unit(sh.t_next);
+            uint2 excl = make_uint2(0u, 0u);
+            if (more) excl = scan_1(r1, r2);
+            // (the or makes every warp's mark before the barrier count)
+            if (__syncthreads_or(sh.over || sh.nkeys > kQueue)) {
+                // too many repeats: nothing of this super-chunk was used yet.
+                // A single column is searched with one counter a peptide;
+                // else half as many columns from here on.
+                if (tid == 0) {
+                    sh.over = 0;
+                    sh.nkeys = 0u;
                 }
+                for (uint32_t i = tid; i < kSlots; i += THREADS) sp.tab[i] = 0u;
+                for (uint32_t i = tid; i < kPlane2Words; i += THREADS) sp.plane2[i] = 0u;
+                for (uint32_t i = tid; i < a.lay.plane_words; i += THREADS) plane[i] = 0u;
+                __syncthreads();
+                if (st.e - st.c == 1) {
+                    save();
+                    direct_column(a, x0, x1);
+                    restore();
+                    st.c = st.e;
+                } else {
+                    st.m = (st.e - st.c + 1) / 2;
+                }
+                if (st.c < col_end) start();
                 continue;
             }
-            const uint32_t cbase = c << kChunkShift;
-            const uint32_t x0 = max(seg_lo, cbase), x1 = min(seg_hi, e << kChunkShift);
-            twice = seen + words;
-            logw = seen + 2 * words;
-            const uint32_t nc = e, ne = min(e + m, col_end);
-            const bool more = nc < col_end;
-            if (more) load_runs(nc, ne);                 // next super-chunk's bounds: in flight during pass A
-            pass_a(buf, cbase, x0, x1, par);
-            uint32_t excl = 0;
-            if (more) excl = scan_runs_1<PPT>(sh, nnorm, ppt, ra, rb);
-            if (2 * words < log_lo) log_lo = 2 * words;
-            if (2 * words + R > log_dirty) log_dirty = 2 * words + R;
-            __syncthreads();
-            const uint32_t ncand = sh.ncand[par];
-            if (tid == 0) sh.ncand[par ^ 1] = 0u;         // the next super-chunk's count
-            if (once_counts || ncand > kRound) {
-                mark(cbase, words, x0, x1);               // two barriers inside
-                const int nr = sh.nrounds;
-                for (int r = 0; r < nr; ++r) {
-                    const uint32_t wlo = sh.wb[r];
-                    const uint32_t whi = r == nr - 1 ? words : sh.wb[r + 1];
-                    replay(R, wlo, whi);
-                    __syncthreads();
-                    slots_epilogue(cbase);
-                    __syncthreads();
-                }
-                clear_words(twice, 0u, words);
-            } else if (ncand) {
-                replay(R, 0u, words);
-                __syncthreads();
-                slots_epilogue(cbase);
-                clear_words(seen, 0u, words);
-                clear_words(twice, 0u, words);
+            if (more) scan_2(excl, r1, r2);    // (pass A is behind the barrier: the runs are free)
+            // ---- the plane: its peptides of enough hot bits, and cleared
+            if ((uint32_t)sh.nslices + 1u >= a.min_shared) {
+                // peptides hit once (or never) may qualify through their hot bits
+                save();
+                scan_plane(a, pb, x0, x1, words);
+                restore();
             } else {
-                clear_words(seen, 0u, words);             // the twice plane is empty
+                uint4* p4 = reinterpret_cast<uint4*>(plane);
+                for (uint32_t i = tid; i < a.lay.plane_words / 4; i += THREADS) p4[i] = make_uint4(0u, 0u, 0u, 0u);
+                if (st.deep) {
+                    p4 = reinterpret_cast<uint4*>(sp.plane2);
+                    for (uint32_t i = tid; i < kPlane2Words / 4; i += THREADS) p4[i] = make_uint4(0u, 0u, 0u, 0u);
+                }
             }
-            if (more) scan_runs_2<THREADS, PPT>(sh, buf ^ 1, nnorm, ppt, excl, ra, rb);
-            buf ^= 1;
-            par ^= 1;
-            c = nc;
-            e = ne;
+            if (tid == 0) {   // (nothing is appended between here and the barrier)
+                sh.no_room = sh.nkeys == 0u ? -1 : sh.nq + sh.nkeys > kQueue;
+                sh.nkeys = 0u;
+            }
             __syncthreads();
-        }
-        // the unit's top-k: thread 0 merges the warps' lists
-        __syncthreads();
-        if (tid == 0) {
-            int hd[nwarps];
+            // ---- select: the warp's share of the table (there is room for
+            // all of it in the queue; nothing is appended before the drain)
+            if (sh.no_room >= 0) {   // uniform: the table is not empty
+                if (sh.no_room) {
+                    save();
+                    drain_queue(a);
+                    restore();
+                }
+                const uint32_t nslices = (uint32_t)sh.nslices, pb2 = max(sh.unit[st.slot].y, st.c << kChunkShift) & ~127u;
+                for (uint32_t s0 = (uint32_t)warp * 128u; s0 < kSlots; s0 += 4 * THREADS) {
+                    uint4* const t4 = reinterpret_cast<uint4*>(sp.tab + s0) + lane;   // 4 slots a lane
+                    const uint4 v4 = *t4;
+                    if ((v4.x | v4.y | v4.z | v4.w) == 0u) continue;
+                    *t4 = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int w = 0; w < nwarps; ++w) hd[w] = 0;
-            for (int r = 0; r < k; ++r) {
-                int bw = -1;
-                int64_t bk = INT64_MIN;
-                uint32_t bp = 0xffffffffu, bpk = 0u;
-#pragma unroll
-                for (int w = 0; w < nwarps; ++w) {
-                    if (hd[w] < wtop[w].n) {
-                        const int64_t kk = wtop[w].key[hd[w]];
-                        const uint32_t pp = wtop[w].pid[hd[w]];
-                        if (bw < 0 || better(kk, pp, bk, bp)) { bw = w; bk = kk; bp = pp; bpk = wtop[w].pk[hd[w]]; }
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t v = i == 0 ? v4.x : i == 1 ? v4.y : i == 2 ? v4.z : v4.w;
+                        const uint32_t ord = (v & ((1u << (32 - kOffBits)) - 1u)) + 1u + st.deep;   // (at most)
+                        if (v && ord + nslices >= a.min_shared)
+                            push(a, sh, sp, pb2 + (v >> (32 - kOffBits)), ord < a.min_shared ? a.min_shared - ord : 0u);
                     }
                 }
-#pragma unroll
-                for (int w = 0; w < nwarps; ++w)
-                    if (w == bw) ++hd[w];
-                UnitTop o;
-                o.key = bw >= 0 ? bk : INT64_MIN;
-                o.pid = bw >= 0 ? bp : 0xffffffffu;
-                o.packed = bw >= 0 ? bpk : 0u;
-                a.utop[u * k + r] = o;
             }
+            st.c = st.e;
+            st.e = min(st.e + st.m, col_end);
+            take_unit();
+        }
+        if (tid == 0 && !st.taken)   // an empty segment (a window split into more units than it has peptides)
+            set_unit((uint64_t)gridDim.x + atomicAdd(a.work, 1ull));
+        __syncthreads();
+        if (sh.nq) {   // uniform: the appends are behind the barrier
+            save();
+            drain_queue(a);
+            restore();
+        }
+        // the unit's top-k: every item of the warps' sorted lists finds its
+        // rank among all of them
+        const int k = (int)a.k;
+        for (uint32_t i = tid; i < (uint32_t)(nwarps * k); i += THREADS) {
+            const uint32_t w = i / (uint32_t)k, r = i % (uint32_t)k;
+            if (r >= (uint32_t)sh.wn[w]) continue;
+            UnitTop row;
+            row.key = sp.tkey[i];
+            row.pid = sp.tpid[i];
+            row.packed = sp.tpk[i];
+            uint32_t rank = r;
+            for (uint32_t x = 0; x < (uint32_t)nwarps && rank < (uint32_t)k; ++x) {
+                if (x == w) continue;
+                const uint32_t n = (uint32_t)sh.wn[x];
+                for (uint32_t y = 0; y < n; ++y) {
+                    if (!better(sp.tkey[x * k + y], sp.tpid[x * k + y], row.key, row.pid)) break;
+                    ++rank;
+                }
+            }
+            if (rank < (uint32_t)k) a.utop[(uint64_t)sh.unit[st.slot].w * k + rank] = row;
+        }
+        if (tid < k) {
+            int total = 0;
 #pragma unroll
-            for (int w = 0; w < nwarps; ++w) wtop[w].n = 0;
+            for (int w = 0; w < nwarps; ++w) total += sh.wn[w];
+            if (tid >= total) {
+                UnitTop row;
+                row.key = INT64_MIN;
+                row.pid = 0xffffffffu;
+                row.packed = 0u;
+                a.utop[(uint64_t)sh.unit[st.slot].w * k + tid] = row;
+            }
         }
         // histogram of this unit into the spectrum's histogram
         uint32_t mine = 0;
         for (int jb = tid; jb < (int)kHistBins; jb += THREADS) {
             const uint32_t h = sh.hist[jb];
-            if (h) { atomicAdd(&a.hist[(uint64_t)q * kHistBins + jb], h); mine += h; sh.hist[jb] = 0; }
+            if (h) {
+                atomicAdd(&a.hist[(uint64_t)sh.unit[st.slot].x * kHistBins + jb], h);
+                mine += h;
+                sh.hist[jb] = 0;
+            }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
-        if (lane == 0 && mine) atomicAdd(&a.nscored[q], mine);
-        __syncthreads();
+        mine = __reduce_add_sync(0xffffffffu, mine);
+        if (lane == 0 && mine) atomicAdd(&a.nscored[sh.unit[st.slot].x], mine);
+        for (uint32_t i = tid; i < kHeads / 2; i += THREADS) sp.head[i] = 0u;
     }
 }

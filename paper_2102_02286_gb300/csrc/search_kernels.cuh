@@ -279,22 +279,22 @@ __global__ void __launch_bounds__(kPrepWarps * 32) prep_warp_kernel(PrepArgs a) 
     }
 }
 
-// work units per spectrum: its window split into pieces of >= seg_pids ids
-__global__ void plan_kernel(const uint32_t* __restrict__ qn, const uint32_t* __restrict__ lo,
-                            const uint32_t* __restrict__ hi, uint32_t n, uint32_t max_seg, uint32_t seg_pids,
-                            uint32_t* __restrict__ nseg) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    uint32_t s = 0;
-    if (qn[q] > 0 && hi[q] > lo[q]) {
-        const uint32_t W = hi[q] - lo[q];
-        s = (uint32_t)(((uint64_t)W + seg_pids - 1) / seg_pids);
-        if (s > max_seg) s = max_seg;
-    }
-    nseg[q] = s;
+// work units of a spectrum: its window split into pieces of >= seg_pids ids
+__device__ __forceinline__ uint32_t units_of(uint32_t qn, uint32_t lo, uint32_t hi, uint32_t max_seg, uint32_t seg_pids) {
+    if (qn == 0 || hi <= lo) return 0;
+    const uint64_t s = ((uint64_t)(hi - lo) + seg_pids - 1) / seg_pids;
+    return s > max_seg ? max_seg : (uint32_t)s;
 }
 
-// ---- unit order: longest first (the persistent CTAs take units in this
+__global__ void plan_kernel(const uint32_t* __restrict__ qn, const uint32_t* __restrict__ lo,
+                            const uint32_t* __restrict__ hi, uint32_t n, uint32_t max_seg, uint32_t seg_pids,
+                            uint32_t* __restrict__ nseg, unsigned long long* __restrict__ work) {
+    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q == 0) *work = 0ull;
+    if (q < n) nseg[q] = units_of(qn[q], lo[q], hi[q], max_seg, seg_pids);
+}
+
+// ---- units in the order they are taken: longest first (the persistent CTAs take units in this
 // order, so the short ones fill the end of the launch).  A unit's cost is
 // estimated as its peptide range times the spectrum's retained peaks; units
 // are bucketed by the cost's binary magnitude (a counting sort over 64
@@ -344,10 +344,18 @@ __global__ void order_scan_kernel(uint32_t* __restrict__ cnt) {
     cnt[kOrderBuckets + 32 + lane] = tot_a + ib - b;
 }
 
+// A work unit: {spectrum, segment [lo, hi), unit number}.  The window of
+// spectrum q is split evenly into its ns units.
+__device__ __forceinline__ uint4 unit_record(uint32_t q, uint32_t lo, uint32_t hi, uint32_t ns, uint32_t s,
+                                             uint64_t u0) {
+    const uint32_t len = (uint32_t)(((uint64_t)(hi - lo) + ns - 1) / ns);
+    const uint64_t a = (uint64_t)lo + (uint64_t)s * len;
+    return make_uint4(q, (uint32_t)min(a, (uint64_t)hi), (uint32_t)min(a + len, (uint64_t)hi), (uint32_t)(u0 + s));
+}
+
 __global__ void order_scatter_kernel(const uint32_t* __restrict__ qn, const uint32_t* __restrict__ lo,
                                      const uint32_t* __restrict__ hi, const uint64_t* __restrict__ seg_off,
-                                     uint32_t n, uint32_t* __restrict__ cursor, uint32_t* __restrict__ order,
-                                     uint32_t* __restrict__ order_q) {
+                                     uint32_t n, uint32_t* __restrict__ cursor, uint4* __restrict__ unit) {
     __shared__ uint32_t bc[kOrderBuckets], bb[kOrderBuckets];
     for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x) bc[i] = 0;
     __syncthreads();
@@ -365,12 +373,71 @@ __global__ void order_scatter_kernel(const uint32_t* __restrict__ qn, const uint
     if (ns) {
         const uint32_t pos = bb[b] + local;
         const uint64_t u0 = seg_off[q];
-        for (uint32_t s = 0; s < ns; ++s) {
-            order[pos + s] = (uint32_t)(u0 + s);
-            order_q[pos + s] = q;
-        }
+        for (uint32_t s = 0; s < ns; ++s) unit[pos + s] = unit_record(q, lo[q], hi[q], ns, s, u0);
     }
 }
+
+// The whole planning of a small batch (fewer than kOrderMinSpectra spectra) in
+// one block: the spectra's units, their prefix and the unit records in
+// spectrum order.  Three launches (counts, scan, records) would be more of a
+// small call's time than the work in them.
+constexpr int kPlanThreads = 1024;
+__global__ void __launch_bounds__(kPlanThreads) plan_small_kernel(const uint32_t* __restrict__ qn,
+                                                                  const uint32_t* __restrict__ lo,
+                                                                  const uint32_t* __restrict__ hi, uint32_t n,
+                                                                  uint32_t max_seg, uint32_t seg_pids,
+                                                                  uint64_t* __restrict__ seg_off,
+                                                                  uint4* __restrict__ unit,
+                                                                  unsigned long long* __restrict__ work) {
+    __shared__ uint32_t off[kOrderMinSpectra + 1];   // (64 units a spectrum at most: 32 bits hold them)
+    __shared__ uint32_t wt[kPlanThreads / 32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t base = 0;
+    for (uint32_t q0 = 0; q0 < n; q0 += kPlanThreads) {
+        const uint32_t q = q0 + tid;
+        const uint32_t ns = q < n ? units_of(qn[q], lo[q], hi[q], max_seg, seg_pids) : 0u;
+        uint32_t incl = ns;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= (uint32_t)o) incl += x;
+        }
+        if (lane == 31) wt[warp] = incl;
+        __syncthreads();
+        const uint32_t t = wt[lane];
+        uint32_t before = lane < warp ? t : 0u;
+        before = __reduce_add_sync(0xffffffffu, before);
+        const uint32_t total = __reduce_add_sync(0xffffffffu, t);
+        if (q < n) {
+            off[q] = base + before + incl - ns;
+            seg_off[q] = off[q];
+        }
+        base += total;
+        __syncthreads();   // wt is reused
+    }
+    if (tid == 0) {
+        off[n] = base;
+        seg_off[n] = base;
+        *work = 0ull;
+    }
+    __syncthreads();
+    for (uint32_t u = tid; u < base; u += kPlanThreads) {
+        uint32_t a = 0, b = n;   // the last spectrum with off <= u: it has units, the next one starts above u
+        while (b - a > 1) {
+            const uint32_t m = (a + b) >> 1;
+            if (off[m] <= u) a = m; else b = m;
+        }
+        unit[u] = unit_record(a, lo[a], hi[a], off[a + 1] - off[a], u - off[a], off[a]);
+    }
+}
+
+// Shared memory of the search kernel, in 32-bit words: the plane, as large as
+// the rest leaves room for, then search_kernel.cuh's SearchShared and the
+// parts of its SearchParts.
+struct SearchLayout {
+    uint32_t runs, subs, head, qpeak, next, tkey, tab, wq, plane2, hotc, pbase, prow, qpid, tpid, tpk, qneed, end;
+    uint32_t plane_words;       // a power of two
+};
 
 #include "search_kernel.cuh"
 
