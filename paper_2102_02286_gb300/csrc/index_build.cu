@@ -16,7 +16,8 @@
 namespace hicops {
 namespace {
 
-constexpr int kIonThreads = 256;
+constexpr int kIonThreads = 128;
+constexpr int kIonStage = 2048;      // ion bins a warp stages in shared memory (8 KB)
 
 struct IonArgs {
     const uint32_t* base;        // [P] base peptide id
@@ -27,101 +28,196 @@ struct IonArgs {
     const double* mmod;          // [128]
     double w, mz_lo, mz_hi;
     uint64_t P;
+    // the same masses and limits in bins, with 32 fraction bits (fixed_ions)
+    const int64_t* fix;          // [2][128]: unmodified, modified
+    int64_t b_add, y_add;        // proton; water + proton
+    int64_t lo, hi;
+    uint32_t tol;                // most that a fixed-point value can be off, in 2^-32 bins
+    int fixed;                   // the fixed-point values hold for this index
 };
 
 // Visits the distinct in-range ion bins of one peptide in ascending bin
 // order; a bin reached by both a b and a y ion is reported once, as b.
 // b_i = (m_1 + .. + m_i) + proton, summed left to right;
 // y_i = ((m_L + m_{L-1} + .. + m_{i+1}) + H2O) + proton, summed from the C terminus.
+// Collected and sorted, so a modification that takes a residue's mass below
+// zero (sums that do not ascend) is indexed alike.
 template <class F>
-__device__ __forceinline__ void for_each_ion_bin(const IonArgs& a, const double* mres, const double* mmod,
-                                                 uint64_t pid, F&& emit) {
+__device__ __noinline__ void each_ion_bin_fp64(const IonArgs& a, uint64_t pid, F emit) {
     const uint32_t b = a.base[pid];
     const uint64_t m = a.mask[pid];
     const char* s = a.residues + a.base_off[b];
     const int L = (int)(a.base_off[b + 1] - a.base_off[b]);
+    uint32_t list[2 * kMaxLen];      // bin << 1 | isY, ascending
+    int n = 0;
+    auto add = [&](double mz, uint32_t isy) {
+        if (mz < a.mz_lo || mz >= a.mz_hi) return;
+        const uint32_t v = ((uint32_t)floor(mz / a.w) << 1) | isy;   // n_bins < 2^31 (parameter check)
+        int i = n++;
+        for (; i > 0 && list[i - 1] > v; --i) list[i] = list[i - 1];
+        list[i] = v;
+    };
     auto rm = [&](int j) -> double {
         const unsigned char c = (unsigned char)s[j];
-        return ((m >> j) & 1ull) ? mmod[c] : mres[c];
+        return ((m >> j) & 1ull) ? a.mmod[c] : a.mres[c];
     };
-    // b stream state: next ion index ib (1..L-1), running prefix
-    int ib = 1;
-    double pre = 0.0;
-    // y stream state: next ion index iy (L-1 down to 1), running suffix
-    int iy = L - 1;
-    double suf = 0.0;
-    uint32_t bb = 0, by = 0;
-    bool hb = false, hy = false;
-    auto next_b = [&]() -> bool {
-        while (ib <= L - 1) {
-            pre = pre + rm(ib - 1);
-            const double mz = pre + kProtonDa;
-            ++ib;
-            if (mz < a.mz_lo) continue;
-            if (mz >= a.mz_hi) { ib = L; return false; }
-            bb = (uint32_t)floor(mz / a.w);
-            return true;
-        }
-        return false;
-    };
-    auto next_y = [&]() -> bool {
-        while (iy >= 1) {
-            suf = suf + rm(iy);
-            const double mz = (suf + kWaterDa) + kProtonDa;
-            --iy;
-            if (mz < a.mz_lo) continue;
-            if (mz >= a.mz_hi) { iy = 0; return false; }
-            by = (uint32_t)floor(mz / a.w);
-            return true;
-        }
-        return false;
-    };
-    hb = next_b();
-    hy = next_y();
-    uint32_t last = 0xffffffffu;
-    while (hb || hy) {
-        if (hb && (!hy || bb <= by)) {
-            if (bb != last) { emit(bb, 0u); last = bb; }
-            hb = next_b();
-        } else {
-            if (by != last) { emit(by, 1u); last = by; }
-            hy = next_y();
-        }
+    double pre = 0.0, suf = 0.0;
+    for (int i = 1; i < L; ++i) {
+        pre = pre + rm(i - 1);
+        add(pre + kProtonDa, 0u);
     }
+    for (int i = L - 1; i >= 1; --i) {
+        suf = suf + rm(i);
+        add((suf + kWaterDa) + kProtonDa, 1u);
+    }
+    for (int i = 0; i < n; ++i)
+        if (i == 0 || (list[i] >> 1) != (list[i - 1] >> 1)) emit(list[i] >> 1, list[i] & 1u);
 }
 
-__global__ void ion_count_kernel(IonArgs a, uint32_t* __restrict__ count) {
-    __shared__ double smres[128], smmod[128];
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) { smres[i] = a.mres[i]; smmod[i] = a.mmod[i]; }
+// The same visits from fixed-point sums in units of a bin (32 fraction bits):
+// the high word of a sum is the bin, so an ion costs integer additions where
+// the FP64 form costs a division on a unit of 2 lanes a clock.  a.tol bounds
+// the distance between the fixed-point value and the FP64 quotient, so a value
+// farther than that from every bin edge and from both limits of the m/z range
+// has the FP64 form's bin.  At a value nearer than that the visit ends and
+// returns false: everything visited up to there is a prefix of the FP64
+// form's visits, which the caller then takes from the start.
+// One ion per step, from the stream with the lower bin (b at equal bins).
+template <class F>
+__device__ __forceinline__ bool each_ion_bin_fixed(const IonArgs& a, const int64_t* fix, uint64_t pid, F&& emit) {
+    const uint32_t b = a.base[pid];
+    const uint64_t m = a.mask[pid];
+    const char* s = a.residues + a.base_off[b];
+    const int L = (int)(a.base_off[b + 1] - a.base_off[b]);
+    if (L < 2) return true;
+    constexpr int64_t kDone = 0x7fffffffffffffffll;
+    bool sure = true;
+    auto check = [&](int64_t v) -> int64_t {
+        sure = sure && (uint32_t)v + a.tol >= 2u * a.tol && llabs(v - a.lo) > (int64_t)a.tol &&
+               llabs(v - a.hi) > (int64_t)a.tol;
+        return v >= a.hi ? kDone : v;
+    };
+    auto rm = [&](int j) { return fix[((uint32_t)(m >> j) & 1u) << 7 | (unsigned char)s[j]]; };
+    int ib = 0, iy = L - 1;               // residues taken next
+    int64_t sb = a.b_add + rm(0), sy = a.y_add + rm(L - 1);
+    int64_t vb = check(sb), vy = check(sy);
+    uint32_t last = 0xffffffffu;
+    while (sure && (vb != kDone || vy != kDone)) {
+        const bool tb = (vb >> 32) <= (vy >> 32);
+        const int64_t v = tb ? vb : vy;
+        const uint32_t bin = (uint32_t)(v >> 32);
+        if (v >= a.lo && bin != last) { emit(bin, tb ? 0u : 1u); last = bin; }
+        const int j = tb ? ++ib : --iy;
+        const bool more = tb ? j < L - 1 : j >= 1;
+        int64_t nv = kDone;
+        if (more) {
+            const int64_t sum = (tb ? sb : sy) + rm(j);
+            nv = check(sum);
+            if (tb) sb = sum; else sy = sum;
+        }
+        if (tb) vb = nv; else vy = nv;
+    }
+    return sure;
+}
+
+// 2.73 -> 0.20 ms for 50 M ions of 1.6 M peptides: bound by the issue of some 30
+// integer instructions an ion.
+__global__ void __launch_bounds__(kIonThreads) ion_count_kernel(IonArgs a, uint32_t* __restrict__ count,
+                                                                uint32_t* __restrict__ groups) {
+    __shared__ int64_t fix[256];
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) fix[i] = a.fix[i];
     __syncthreads();
     const uint64_t pid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (pid >= a.P) return;
     uint32_t n = 0;
-    for_each_ion_bin(a, smres, smmod, pid, [&](uint32_t, uint32_t) { ++n; });
+    if (!a.fixed || !each_ion_bin_fixed(a, fix, pid, [&](uint32_t, uint32_t) { ++n; })) {
+        uint32_t m = 0;
+        each_ion_bin_fp64(a, pid, [&](uint32_t, uint32_t) { ++m; });
+        n = m;
+    }
     count[pid] = n;
+    groups[pid] = (n + 3u) >> 2;   // the forward list's length in groups of 4
 }
 
-// list lengths in groups of 4 ion bins
-__global__ void ion_groups_kernel(uint32_t* __restrict__ count, uint64_t P) {
-    const uint64_t pid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pid < P) count[pid] = (count[pid] + 3u) >> 2;
-}
-
-// keys for the sort by bin, and the forward list
-__global__ void ion_emit_kernel(IonArgs a, const uint64_t* __restrict__ off, uint64_t* __restrict__ keys,
-                                const uint64_t* __restrict__ fwd_off, uint32_t* __restrict__ fwd) {
-    __shared__ double smres[128], smmod[128];
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) { smres[i] = a.mres[i]; smmod[i] = a.mmod[i]; }
+// Keys for the sort by bin, and the forward list.  A warp's 32 lists are
+// neighbours in both arrays: they are staged in shared memory, padding
+// included, and written from there in whole lines; lists that do not fit
+// (more than 64 ions a peptide) are written ion by ion.
+// 2.74 -> 0.52 ms for 50 M ions (600 MB written).
+__global__ void __launch_bounds__(kIonThreads) ion_emit_kernel(IonArgs a, const uint64_t* __restrict__ off,
+                                                               uint64_t* __restrict__ keys,
+                                                               const uint64_t* __restrict__ fwd_off,
+                                                               uint32_t* __restrict__ fwd) {
+    __shared__ int64_t fix[256];
+    __shared__ __align__(16) uint32_t stage_all[kIonThreads / 32][kIonStage];
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) fix[i] = a.fix[i];
     __syncthreads();
-    const uint64_t pid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (pid >= a.P) return;
-    uint64_t o = off[pid], f = 4 * fwd_off[pid];
-    for_each_ion_bin(a, smres, smmod, pid, [&](uint32_t bin, uint32_t isy) {
-        keys[o] = ((uint64_t)bin << 32) | (uint64_t)((uint32_t)(pid << 1) | isy);
-        ++o;
-        fwd[f++] = (bin << 1) | isy;   // n_bins < 2^31 (parameter check)
-    });
-    for (; f & 3; ++f) fwd[f] = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint64_t pid0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+    if (pid0 >= a.P) return;
+    uint32_t* stage = stage_all[threadIdx.x >> 5];
+    const uint64_t pid = pid0 + lane;
+    const bool mine = pid < a.P;
+    const uint64_t f0 = fwd_off[pid0], f1 = fwd_off[min(pid0 + 32, a.P)];
+    const uint64_t o = mine ? off[pid] : 0, f = mine ? fwd_off[pid] : f0;
+    const bool fits = (f1 - f0) * 4 <= (uint64_t)kIonStage;
+    const uint32_t low = (uint32_t)(pid << 1);
+    uint32_t n = 0;
+    if (mine) {
+        uint32_t* list = fits ? stage + 4 * (uint32_t)(f - f0) : fwd + 4 * f;
+        auto put = [&](uint32_t bin, uint32_t isy) {
+            list[n] = (bin << 1) | isy;   // n_bins < 2^31 (parameter check)
+            if (!fits) keys[o + n] = ((uint64_t)bin << 32) | (low | isy);
+            ++n;
+        };
+        if (!a.fixed || !each_ion_bin_fixed(a, fix, pid, put)) {
+            uint32_t m = 0;
+            uint32_t* to = list;
+            uint64_t* key = fits ? nullptr : keys + o;
+            each_ion_bin_fp64(a, pid, [&m, to, key, low](uint32_t bin, uint32_t isy) {
+                to[m] = (bin << 1) | isy;
+                if (key) key[m] = ((uint64_t)bin << 32) | (low | isy);
+                ++m;
+            });
+            n = m;
+        }
+        for (uint32_t i = n; i & 3; ++i) list[i] = 0xffffffffu;
+    }
+    if (!fits) return;   // the whole warp
+    __syncwarp();
+    uint4* out = reinterpret_cast<uint4*>(fwd) + f0;
+    const uint4* in = reinterpret_cast<const uint4*>(stage);
+    for (uint32_t i = lane; i < (uint32_t)(f1 - f0); i += 32) out[i] = in[i];
+    for (int l = 0; l < 32; ++l) {
+        const uint32_t cnt = __shfl_sync(0xffffffffu, n, l);
+        const uint64_t to = __shfl_sync(0xffffffffu, o, l);
+        const uint32_t from = 4 * (uint32_t)(__shfl_sync(0xffffffffu, f, l) - f0);
+        const uint32_t plow = (uint32_t)((pid0 + l) << 1);
+        for (uint32_t i = lane; i < cnt; i += 32) {
+            const uint32_t e = stage[from + i];
+            keys[to + i] = ((uint64_t)(e >> 1) << 32) | (plow | (e & 1u));
+        }
+    }
+}
+
+// LS[v] = round(2^32 log10 v) of the host's libm.  The device's log10 and the
+// host's each lie within 2 ulp of the true value, under 2^-14 in these units
+// (log10 v < 8), so a value farther than 2^-10 from a rounding edge rounds
+// alike; the others (2 in 1,000) are listed and computed by the host.
+__global__ void ls_kernel(int64_t* __restrict__ ls, uint32_t n, uint32_t* __restrict__ list,
+                          unsigned long long* __restrict__ listed) {
+    const uint32_t v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= n) return;
+    const double x = v < 2 ? 0.0 : ldexp(log10((double)v), 32);
+    const double lo = floor(x);
+    ls[v] = (int64_t)floor(x + 0.5);
+    if (fabs((x - lo) - 0.5) < 0x1p-10) list[atomicAdd(listed, 1ull)] = v;
+}
+
+__global__ void ls_patch_kernel(int64_t* __restrict__ ls, const uint32_t* __restrict__ list,
+                                const int64_t* __restrict__ value, uint32_t n) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) ls[list[i]] = value[i];
 }
 
 // ---- stable LSD radix sort on the bin field (bits 32..) of 64-bit keys
@@ -214,73 +310,103 @@ __global__ void bucket_off_kernel(const uint64_t* __restrict__ keys, uint64_t n,
     for (int64_t b = prev + 1; b <= cur; ++b) off[b] = i;
 }
 
-// Bucket sizes rounded up to whole groups of 4 entries (16 bytes), so that
-// every bucket starts 16-byte aligned in the entry array.
-__global__ void padded_size_kernel(const uint64_t* __restrict__ off, uint32_t nbins, uint32_t* __restrict__ psz) {
+// Per bucket: its size rounded up to whole groups of 4 entries (16 bytes, so
+// that every bucket starts 16-byte aligned in the entry array), whether it
+// holds an entry, whether it is hot; and the largest size.
+__global__ void __launch_bounds__(256) bucket_kernel(const uint64_t* __restrict__ off, uint32_t nbins, uint64_t hot_lo,
+                                                     uint32_t* __restrict__ psz, uint32_t* __restrict__ some,
+                                                     uint32_t* __restrict__ hot, unsigned long long* __restrict__ mx) {
+    __shared__ unsigned long long block_max;
+    if (threadIdx.x == 0) block_max = 0;
+    __syncthreads();
     const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbins) psz[b] = (uint32_t)((off[b + 1] - off[b] + 3) & ~3ull);
+    if (b < nbins) {
+        const uint64_t size = off[b + 1] - off[b];
+        psz[b] = (uint32_t)((size + 3) & ~3ull);
+        some[b] = size ? 1u : 0u;
+        hot[b] = size >= hot_lo ? 1u : 0u;
+        if (size) atomicMax(&block_max, (unsigned long long)size);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && block_max) atomicMax(mx, block_max);
 }
 
+// row of every flagged bin (its rank among the flagged; -1 for the others), and the bins by rank
+__global__ void row_of_kernel(const uint32_t* __restrict__ flag, const uint64_t* __restrict__ scan, uint32_t nbins,
+                              int32_t* __restrict__ row, uint32_t* __restrict__ bin_of) {
+    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= nbins) return;
+    row[b] = flag[b] ? (int32_t)scan[b] : -1;
+    if (flag[b] && bin_of) bin_of[scan[b]] = b;
+}
+
+// The stored form of the sorted keys, one read of them:
 // entry[poff[bin] + rank in bucket] = pid << 1 | isY; the up to 3 slots after
 // a bucket's last entry keep the pad value 0xffffffff (pid 2^31 - 1, above
 // every peptide id, so a bucket stays pid-sorted and no window contains it).
-__global__ void take_low_kernel(const uint64_t* __restrict__ keys, uint64_t n, const uint64_t* __restrict__ off,
-                                const uint64_t* __restrict__ poff, uint32_t* __restrict__ entry) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t bin = (uint32_t)(keys[i] >> 32);
-    entry[poff[bin] + (i - off[bin])] = (uint32_t)keys[i];
-}
-
-__global__ void bucket_max_kernel(const uint64_t* __restrict__ off, uint32_t nbins, unsigned long long* mx) {
-    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbins) atomicMax(mx, (unsigned long long)(off[b + 1] - off[b]));
-}
-
-// flag[b] = bucket b holds at least lo entries (and is hot when lo > 1)
-__global__ void bucket_flag_kernel(const uint64_t* __restrict__ off, uint32_t nbins, uint64_t lo,
-                                   uint32_t* __restrict__ flag) {
-    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbins) flag[b] = (off[b + 1] - off[b]) >= lo ? 1u : 0u;
-}
-
-__global__ void row_of_kernel(const uint32_t* __restrict__ flag, const uint64_t* __restrict__ scan, uint32_t nbins,
-                              int32_t* __restrict__ row) {
-    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nbins) row[b] = flag[b] ? (int32_t)scan[b] : -1;
-}
-
 // Chunk skip table: skip[row * stride + j] = number of entries of the bucket
 // with pid < j * 2^kChunkShift, for j = 0 .. stride-1 (the last column is the
 // bucket size).  Every cell is written by exactly one entry.
-__global__ void skip_fill_kernel(const uint64_t* __restrict__ keys, uint64_t n, const uint64_t* __restrict__ off,
-                                 const int32_t* __restrict__ row, uint32_t stride, uint32_t* __restrict__ skip) {
+__global__ void store_kernel(const uint64_t* __restrict__ keys, uint64_t n, const uint64_t* __restrict__ off,
+                             const uint64_t* __restrict__ poff, uint32_t* __restrict__ entry,
+                             const int32_t* __restrict__ row, uint32_t stride, uint32_t* __restrict__ skip) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t bin = (uint32_t)(keys[i] >> 32);
-    const uint32_t ch = ((uint32_t)keys[i] >> 1) >> kChunkShift;
+    const uint64_t key = keys[i];
+    const uint32_t bin = (uint32_t)(key >> 32);
+    const uint32_t ch = ((uint32_t)key >> 1) >> kChunkShift;
     const uint64_t b0 = off[bin], b1 = off[bin + 1];
-    uint32_t* base = skip + (uint64_t)row[bin] * stride;
     const uint32_t rel = (uint32_t)(i - b0);
+    entry[poff[bin] + rel] = (uint32_t)key;
     const uint32_t jlo = (i == b0) ? 0u : (((uint32_t)keys[i - 1] >> 1) >> kChunkShift) + 1u;
+    if (jlo > ch && i + 1 != b1) return;
+    uint32_t* base = skip + (uint64_t)row[bin] * stride;
     for (uint32_t j = jlo; j <= ch; ++j) base[j] = rel;
     if (i + 1 == b1)
         for (uint32_t j = ch + 1; j < stride; ++j) base[j] = (uint32_t)(b1 - b0);
 }
 
-// Hot buckets as pid bitmaps: bit pid of hb[h] (b ion) or hy[h] (y ion).
-__global__ void hot_fill_kernel(const uint64_t* __restrict__ keys, uint64_t n, const int32_t* __restrict__ hot_id,
-                                uint64_t words, uint32_t* __restrict__ hb, uint32_t* __restrict__ hy,
-                                uint32_t* __restrict__ hflags) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int32_t h = hot_id[(uint32_t)(keys[i] >> 32)];
-    if (h < 0) return;
-    const uint32_t e = (uint32_t)keys[i];
-    const uint32_t pid = e >> 1;
-    uint32_t* bm = (e & 1u) ? hy : hb;
-    atomicOr(&bm[(uint64_t)h * words + (pid >> 5)], 1u << (pid & 31));
-    atomicOr(&hflags[h], (e & 1u) ? 2u : 1u);
+// Hot buckets as pid bitmaps: bit pid of hb[h] (b ion) or hy[h] (y ion).  One
+// block makes one chunk (2^kChunkShift pids) of one bucket's two bitmaps in
+// shared memory from the chunk's run of entries and writes them whole, zero
+// words included; the last chunk's block also writes the row's spare words.
+// 3.34 ms (a global atomic for every entry, and a memset) -> 0.02 ms for an
+// index of 50 M entries.
+__global__ void __launch_bounds__(256) hot_fill_kernel(const uint32_t* __restrict__ entry,
+                                                       const uint64_t* __restrict__ poff,
+                                                       const uint32_t* __restrict__ hot_bin,
+                                                       const int32_t* __restrict__ row, uint32_t stride,
+                                                       const uint32_t* __restrict__ skip, uint64_t words,
+                                                       uint32_t* __restrict__ hb, uint32_t* __restrict__ hy,
+                                                       uint32_t* __restrict__ hflags) {
+    constexpr uint32_t kWords = kChunk / 32;
+    __shared__ __align__(16) uint32_t bm[2][kWords];
+    __shared__ uint32_t seen;
+    const uint32_t chunks = stride - 1, h = blockIdx.x / chunks, c = blockIdx.x % chunks;
+    for (uint32_t i = threadIdx.x; i < 2 * kWords; i += blockDim.x) (&bm[0][0])[i] = 0;
+    if (threadIdx.x == 0) seen = 0;
+    __syncthreads();
+    const uint32_t bin = hot_bin[h];
+    const uint32_t* sk = skip + (uint64_t)row[bin] * stride + c;
+    const uint32_t* e = entry + poff[bin];
+    uint32_t kinds = 0;
+    for (uint32_t i = sk[0] + threadIdx.x; i < sk[1]; i += blockDim.x) {
+        const uint32_t v = e[i], pid = (v >> 1) & (kChunk - 1);
+        atomicOr(&bm[v & 1u][pid >> 5], 1u << (pid & 31));
+        kinds |= (v & 1u) ? 2u : 1u;
+    }
+    kinds = __reduce_or_sync(0xffffffffu, kinds);
+    if ((threadIdx.x & 31) == 0 && kinds) atomicOr(&seen, kinds);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < 2 * kWords / 4; i += blockDim.x) {
+        const uint32_t y = i >= kWords / 4, j = i - y * (kWords / 4);
+        uint4* to = reinterpret_cast<uint4*>((y ? hy : hb) + h * words + (uint64_t)c * kWords);   // words % 4 == 0
+        to[j] = reinterpret_cast<const uint4*>(bm[y])[j];
+    }
+    if (c + 1 == chunks)
+        for (uint64_t i = (uint64_t)chunks * kWords + threadIdx.x; i < words; i += blockDim.x)
+            hb[h * words + i] = hy[h * words + i] = 0;
+    if (threadIdx.x == 0 && seen) atomicOr(&hflags[h], seen);
 }
 
 // the search's record of every bin
@@ -298,6 +424,38 @@ cudaError_t dalloc(T** p, uint64_t n, std::vector<void*>& tmp) {
     cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (n ? n : 1));
     if (e == cudaSuccess) tmp.push_back(*p);
     return e;
+}
+
+// The residue masses and m/z limits in bins with 32 fraction bits, and how far
+// a sum of them can lie from the FP64 quotient: a fixed-point term is off by
+// half a unit and by its own division's rounding, the FP64 sum by half an ulp
+// of at most the range's end plus one residue for each of its additions, the
+// FP64 quotient by half an ulp.  66 terms and additions (kMaxLen and two
+// constants), all doubled.  Left to FP64 altogether: masses that are not
+// positive and finite, and grids so fine that a sum could leave 60 bits or the
+// bound reach an eighth of a bin.
+void fixed_ions(IonArgs* a, const double* mres, const double* mmod, int64_t* fix) {
+    a->fixed = 0;
+    double top = 0.0;
+    for (int c = 0; c < 256; ++c) {
+        const double m = c < 128 ? mres[c] : mmod[c - 128];
+        fix[c] = 0;
+        // bytes that are no residue have no mass and occur in no peptide
+        if (m == 0.0) continue;
+        if (!(m > 0.0) || !std::isfinite(m)) return;
+        top = std::max(top, m);
+    }
+    const double reach = (a->mz_hi + top + kWaterDa + kProtonDa) / a->w;
+    const double tol = 2.0 * (34.0 + 70.0 * 0x1p-53 * reach * 0x1p32);
+    if (!(reach < 0x1p28) || !(tol < 0x1p29)) return;
+    auto in_bins = [&](double m) { return (int64_t)std::llrint(std::ldexp(m / a->w, 32)); };
+    for (int c = 0; c < 256; ++c) fix[c] = in_bins(c < 128 ? mres[c] : mmod[c - 128]);
+    a->b_add = in_bins(kProtonDa);
+    a->y_add = in_bins(kWaterDa) + in_bins(kProtonDa);
+    a->lo = in_bins(a->mz_lo);
+    a->hi = in_bins(a->mz_hi);
+    a->tol = (uint32_t)std::ceil(tol);
+    a->fixed = 1;
 }
 
 struct TmpFree {
@@ -360,31 +518,38 @@ hicops_status upload_index(hicops_index* idx) {
     }
     HC_CUDA(cudaMalloc(&d.off, sizeof(uint64_t) * (idx->n_bins + 1)));
     // score tables (host libm, FP64): LF[n] = round(2^32 sum_{i<=n} log10 i), LS[s] = round(2^32 log10 s)
-    std::vector<int64_t> lf(kMaxLen + 1), ls(idx->s_max + 1);
+    std::vector<int64_t> lf(kMaxLen + 1);
     double acc = 0.0;
     lf[0] = 0;
     for (uint32_t n = 1; n <= kMaxLen; ++n) {
         if (n >= 2) acc = acc + std::log10((double)n);
         lf[n] = std::llround(std::ldexp(acc, 32));
     }
-    ls[0] = 0;
-    for (uint64_t v = 1; v <= idx->s_max; ++v) ls[v] = std::llround(std::ldexp(std::log10((double)v), 32));
+    const uint32_t n_ls = (uint32_t)idx->s_max + 1;   // s_max < 2^20 (parameter check)
     HC_CUDA(cudaMalloc(&d.lf, sizeof(int64_t) * lf.size()));
-    HC_CUDA(cudaMalloc(&d.ls, sizeof(int64_t) * ls.size()));
+    HC_CUDA(cudaMalloc(&d.ls, sizeof(int64_t) * n_ls));
     HC_CUDA(cudaMemcpyAsync(d.lf, lf.data(), sizeof(int64_t) * lf.size(), cudaMemcpyHostToDevice, s));
-    HC_CUDA(cudaMemcpyAsync(d.ls, ls.data(), sizeof(int64_t) * ls.size(), cudaMemcpyHostToDevice, s));
+    uint64_t* d_total;        // ions; LS values left to the host; largest bucket
+    HC_CUDA(dalloc(&d_total, 3, tf.ptrs));
+    HC_CUDA(cudaMemsetAsync(d_total, 0, 3 * sizeof(uint64_t), s));
+    uint32_t* d_list;
+    HC_CUDA(dalloc(&d_list, n_ls, tf.ptrs));
+    ls_kernel<<<(n_ls + 255) / 256, 256, 0, s>>>(d.ls, n_ls, d_list, (unsigned long long*)d_total + 1);
+    HC_CUDA(cudaGetLastError());
 
     // temporaries: peptide table
     uint32_t* d_base;
     uint64_t *d_mask, *d_boff;
     char* d_res;
     double *d_mres, *d_mmod;
+    int64_t* d_fix;
     HC_CUDA(dalloc(&d_base, P, tf.ptrs));
     HC_CUDA(dalloc(&d_mask, P, tf.ptrs));
     HC_CUDA(dalloc(&d_boff, B + 1, tf.ptrs));
     HC_CUDA(dalloc(&d_res, idx->residues.size() + 1, tf.ptrs));
     HC_CUDA(dalloc(&d_mres, 128, tf.ptrs));
     HC_CUDA(dalloc(&d_mmod, 128, tf.ptrs));
+    HC_CUDA(dalloc(&d_fix, 256, tf.ptrs));
     HC_CUDA(cudaMemcpyAsync(d_base, idx->base.data(), sizeof(uint32_t) * P, cudaMemcpyHostToDevice, s));
     HC_CUDA(cudaMemcpyAsync(d_mask, idx->mask.data(), sizeof(uint64_t) * P, cudaMemcpyHostToDevice, s));
     HC_CUDA(cudaMemcpyAsync(d_boff, idx->base_off.data(), sizeof(uint64_t) * (B + 1), cudaMemcpyHostToDevice, s));
@@ -392,27 +557,44 @@ hicops_status upload_index(hicops_index* idx) {
     HC_CUDA(cudaMemcpyAsync(d_mres, idx->mres, sizeof(double) * 128, cudaMemcpyHostToDevice, s));
     HC_CUDA(cudaMemcpyAsync(d_mmod, idx->mmod, sizeof(double) * 128, cudaMemcpyHostToDevice, s));
 
-    IonArgs a{d_base, d_mask, d_boff, d_res, d_mres, d_mmod, p.bin_width_da, p.frag_mz_min, p.frag_mz_max, P};
-    uint32_t* d_cnt;
+    IonArgs a{d_base, d_mask, d_boff, d_res, d_mres, d_mmod, p.bin_width_da, p.frag_mz_min, p.frag_mz_max, P,
+              d_fix, 0, 0, 0, 0, 0, 0};
+    int64_t fix[256];
+    fixed_ions(&a, idx->mres, idx->mmod, fix);
+    HC_CUDA(cudaMemcpyAsync(d_fix, fix, sizeof(fix), cudaMemcpyHostToDevice, s));
+    uint32_t *d_cnt, *d_groups;
     uint64_t* d_ionoff;
-    uint64_t* d_total;
     HC_CUDA(dalloc(&d_cnt, P, tf.ptrs));
+    HC_CUDA(dalloc(&d_groups, P, tf.ptrs));
     HC_CUDA(dalloc(&d_ionoff, P, tf.ptrs));
     HC_CUDA(cudaMalloc(&d.fwd_off, sizeof(uint64_t) * (P + 1)));
-    HC_CUDA(dalloc(&d_total, 1, tf.ptrs));
     uint64_t* d_scan_tmp;
     HC_CUDA(dalloc(&d_scan_tmp, scan_tmp_words(P), tf.ptrs));
     const unsigned pgrid = (unsigned)((P + kIonThreads - 1) / kIonThreads);
-    if (P) ion_count_kernel<<<pgrid, kIonThreads, 0, s>>>(a, d_cnt);
+    if (P) ion_count_kernel<<<pgrid, kIonThreads, 0, s>>>(a, d_cnt, d_groups);
     HC_CUDA(cudaGetLastError());
     HC_CUDA(exclusive_scan<uint32_t>(d_cnt, P, d_ionoff, d_total, d_scan_tmp, s));
-    if (P) ion_groups_kernel<<<pgrid, kIonThreads, 0, s>>>(d_cnt, P);
-    HC_CUDA(cudaGetLastError());
-    HC_CUDA(exclusive_scan<uint32_t>(d_cnt, P, d.fwd_off, d.fwd_off + P, d_scan_tmp, s));
-    uint64_t E = 0;
+    HC_CUDA(exclusive_scan<uint32_t>(d_groups, P, d.fwd_off, d.fwd_off + P, d_scan_tmp, s));
+    uint64_t totals[3] = {0, 0, 0};
     HC_CUDA(cudaMemcpyAsync(&d.n_fwd, d.fwd_off + P, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    HC_CUDA(cudaMemcpyAsync(&E, d_total, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    HC_CUDA(cudaMemcpyAsync(totals, d_total, sizeof(totals), cudaMemcpyDeviceToHost, s));
     HC_CUDA(cudaStreamSynchronize(s));
+    const uint64_t E = totals[0];
+
+    std::vector<uint32_t> ls_at(totals[1]);
+    std::vector<int64_t> ls_val(totals[1]);
+    if (!ls_at.empty()) {
+        int64_t* d_val;
+        HC_CUDA(dalloc(&d_val, ls_at.size(), tf.ptrs));
+        HC_CUDA(cudaMemcpyAsync(ls_at.data(), d_list, sizeof(uint32_t) * ls_at.size(), cudaMemcpyDeviceToHost, s));
+        HC_CUDA(cudaStreamSynchronize(s));
+        for (size_t i = 0; i < ls_at.size(); ++i)
+            ls_val[i] = std::llround(std::ldexp(std::log10((double)ls_at[i]), 32));
+        HC_CUDA(cudaMemcpyAsync(d_val, ls_val.data(), sizeof(int64_t) * ls_val.size(), cudaMemcpyHostToDevice, s));
+        ls_patch_kernel<<<(unsigned)((ls_at.size() + 255) / 256), 256, 0, s>>>(d.ls, d_list, d_val,
+                                                                              (uint32_t)ls_at.size());
+        HC_CUDA(cudaGetLastError());
+    }
 
     uint64_t *keys, *keys2;
     HC_CUDA(dalloc(&keys, E, tf.ptrs));
@@ -451,13 +633,34 @@ hicops_status upload_index(hicops_index* idx) {
     HC_CUDA(dalloc(&uoff, (uint64_t)nb + 1, tf.ptrs));
     bucket_off_kernel<<<(unsigned)((E + 1 + 255) / 256), 256, 0, s>>>(keys, E, nb, uoff);
     HC_CUDA(cudaGetLastError());
-    unsigned long long* d_mx = (unsigned long long*)d_total;
-    HC_CUDA(cudaMemsetAsync(d_mx, 0, sizeof(uint64_t), s));
-    bucket_max_kernel<<<bgrid, 256, 0, s>>>(uoff, nb, d_mx);
+    const uint64_t hot_lo = std::max<uint64_t>(2, P >> kHotShift);
+    uint32_t *psz, *some, *hot, *hot_bin;
+    uint64_t *some_at, *hot_at, *rtotal, *btmp;
+    HC_CUDA(dalloc(&psz, nb, tf.ptrs));
+    HC_CUDA(dalloc(&some, nb, tf.ptrs));
+    HC_CUDA(dalloc(&hot, nb, tf.ptrs));
+    HC_CUDA(dalloc(&hot_bin, nb, tf.ptrs));
+    HC_CUDA(dalloc(&some_at, nb, tf.ptrs));
+    HC_CUDA(dalloc(&hot_at, nb, tf.ptrs));
+    HC_CUDA(dalloc(&rtotal, 4, tf.ptrs));     // stored entries, skip rows, hot buckets, largest bucket
+    HC_CUDA(dalloc(&btmp, scan_tmp_words(nb), tf.ptrs));
+    HC_CUDA(cudaMemsetAsync(rtotal, 0, 4 * sizeof(uint64_t), s));
+    HC_CUDA(cudaMalloc(&d.skip_row, sizeof(int32_t) * nb));
+    HC_CUDA(cudaMalloc(&d.hot_id, sizeof(int32_t) * nb));
+    bucket_kernel<<<bgrid, 256, 0, s>>>(uoff, nb, hot_lo, psz, some, hot, (unsigned long long*)rtotal + 3);
     HC_CUDA(cudaGetLastError());
-    uint64_t mx = 0;
-    HC_CUDA(cudaMemcpyAsync(&mx, d_mx, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+    HC_CUDA(exclusive_scan<uint32_t>(psz, nb, d.off, d.off + nb, btmp, s));
+    HC_CUDA(cudaMemcpyAsync(rtotal, d.off + nb, sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+    HC_CUDA(exclusive_scan<uint32_t>(some, nb, some_at, rtotal + 1, btmp, s));
+    HC_CUDA(exclusive_scan<uint32_t>(hot, nb, hot_at, rtotal + 2, btmp, s));
+    row_of_kernel<<<bgrid, 256, 0, s>>>(some, some_at, nb, d.skip_row, nullptr);
+    HC_CUDA(cudaGetLastError());
+    row_of_kernel<<<bgrid, 256, 0, s>>>(hot, hot_at, nb, d.hot_id, hot_bin);
+    HC_CUDA(cudaGetLastError());
+    uint64_t sizes[4];
+    HC_CUDA(cudaMemcpyAsync(sizes, rtotal, sizeof(sizes), cudaMemcpyDeviceToHost, s));
     HC_CUDA(cudaStreamSynchronize(s));
+    const uint64_t Ep = sizes[0], rows = sizes[1], nhot = sizes[2], mx = sizes[3];
     // the sort's other buffer goes before the stored entries come, so that the
     // build's peak stays at 20 bytes an entry (two key buffers and the forward lists)
     tf.release(keys2);
@@ -465,51 +668,17 @@ hicops_status upload_index(hicops_index* idx) {
         set_error("a bucket holds %llu entries (limit 2^32 - 4)", (unsigned long long)mx);
         return HICOPS_EOVERFLOW;
     }
-    uint32_t* flag;
-    uint64_t *rscan, *rtotal, *btmp;
-    HC_CUDA(dalloc(&flag, nb, tf.ptrs));
-    HC_CUDA(dalloc(&rscan, nb, tf.ptrs));
-    HC_CUDA(dalloc(&rtotal, 1, tf.ptrs));
-    HC_CUDA(dalloc(&btmp, scan_tmp_words(nb), tf.ptrs));
-    padded_size_kernel<<<bgrid, 256, 0, s>>>(uoff, nb, flag);
-    HC_CUDA(cudaGetLastError());
-    HC_CUDA(exclusive_scan<uint32_t>(flag, nb, d.off, d.off + nb, btmp, s));
-    uint64_t Ep = 0;
-    HC_CUDA(cudaMemcpyAsync(&Ep, d.off + nb, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    HC_CUDA(cudaStreamSynchronize(s));
-    // four spare words: the allocation is never empty and ends 16-byte aligned
+    // stored entries and the chunk skip tables of every non-empty bucket
+    // (positions relative to the bucket start); four spare words: the entry
+    // allocation is never empty and ends 16-byte aligned
     HC_CUDA(cudaMalloc(&d.entry, sizeof(uint32_t) * (Ep + 4)));
     HC_CUDA(cudaMemsetAsync(d.entry, 0xff, sizeof(uint32_t) * (Ep + 4), s));
-    if (E) take_low_kernel<<<egrid, 256, 0, s>>>(keys, E, uoff, d.off, d.entry);
-    HC_CUDA(cudaGetLastError());
-
-    // chunk skip tables for every non-empty bucket (positions relative to
-    // the bucket start, so the same in both layouts)
-    bucket_flag_kernel<<<bgrid, 256, 0, s>>>(uoff, nb, 1, flag);
-    HC_CUDA(cudaGetLastError());
-    HC_CUDA(exclusive_scan<uint32_t>(flag, nb, rscan, rtotal, btmp, s));
-    HC_CUDA(cudaMalloc(&d.skip_row, sizeof(int32_t) * nb));
-    row_of_kernel<<<bgrid, 256, 0, s>>>(flag, rscan, nb, d.skip_row);
-    HC_CUDA(cudaGetLastError());
-    uint64_t rows = 0;
-    HC_CUDA(cudaMemcpyAsync(&rows, rtotal, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    HC_CUDA(cudaStreamSynchronize(s));
     d.skip_stride = (uint32_t)(((P + kChunk - 1) >> kChunkShift) + 1);
     HC_CUDA(cudaMalloc(&d.skip, sizeof(uint32_t) * (rows ? rows : 1) * d.skip_stride));
-    if (E) skip_fill_kernel<<<egrid, 256, 0, s>>>(keys, E, uoff, d.skip_row, d.skip_stride, d.skip);
+    if (E) store_kernel<<<egrid, 256, 0, s>>>(keys, E, uoff, d.off, d.entry, d.skip_row, d.skip_stride, d.skip);
     HC_CUDA(cudaGetLastError());
 
     // hot buckets as bitmaps
-    const uint64_t hot_lo = std::max<uint64_t>(2, P >> kHotShift);
-    bucket_flag_kernel<<<bgrid, 256, 0, s>>>(uoff, nb, hot_lo, flag);
-    HC_CUDA(cudaGetLastError());
-    HC_CUDA(exclusive_scan<uint32_t>(flag, nb, rscan, rtotal, btmp, s));
-    HC_CUDA(cudaMalloc(&d.hot_id, sizeof(int32_t) * nb));
-    row_of_kernel<<<bgrid, 256, 0, s>>>(flag, rscan, nb, d.hot_id);
-    HC_CUDA(cudaGetLastError());
-    uint64_t nhot = 0;
-    HC_CUDA(cudaMemcpyAsync(&nhot, rtotal, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    HC_CUDA(cudaStreamSynchronize(s));
     d.n_hot = (uint32_t)nhot;
     // rows cover every pid of the last search chunk (up to 2 * kChunk past P)
     // and start 16-byte aligned
@@ -518,10 +687,12 @@ hicops_status upload_index(hicops_index* idx) {
     HC_CUDA(cudaMalloc(&d.hot_b, hbytes));
     HC_CUDA(cudaMalloc(&d.hot_y, hbytes));
     HC_CUDA(cudaMalloc(&d.hot_flags, sizeof(uint32_t) * (nhot ? nhot : 1)));
-    HC_CUDA(cudaMemsetAsync(d.hot_b, 0, hbytes, s));
-    HC_CUDA(cudaMemsetAsync(d.hot_y, 0, hbytes, s));
     HC_CUDA(cudaMemsetAsync(d.hot_flags, 0, sizeof(uint32_t) * (nhot ? nhot : 1), s));
-    if (E && nhot) hot_fill_kernel<<<egrid, 256, 0, s>>>(keys, E, d.hot_id, d.hot_words, d.hot_b, d.hot_y, d.hot_flags);
+    // a peptide has at most 126 ions, so at most 126 * 64 buckets hold 1/64 of the
+    // peptides each: nhot * chunks < 2^31
+    if (nhot)
+        hot_fill_kernel<<<(unsigned)(nhot * (d.skip_stride - 1)), 256, 0, s>>>(
+            d.entry, d.off, hot_bin, d.skip_row, d.skip_stride, d.skip, d.hot_words, d.hot_b, d.hot_y, d.hot_flags);
     HC_CUDA(cudaGetLastError());
     HC_CUDA(cudaMalloc(&d.bins, sizeof(BinInfo) * nb));
     bin_info_kernel<<<bgrid, 256, 0, s>>>(d.off, d.skip_row, d.hot_id, d.hot_flags, nb, d.bins);
@@ -535,7 +706,7 @@ hicops_status upload_index(hicops_index* idx) {
 
     d.n_stored = Ep;
     d.bytes = sizeof(double) * P + sizeof(uint64_t) * (idx->n_bins + 1) + sizeof(uint32_t) * (Ep + 4) +
-              sizeof(int64_t) * (lf.size() + ls.size()) + sizeof(BinInfo) * nb +
+              sizeof(int64_t) * (lf.size() + n_ls) + sizeof(BinInfo) * nb +
               sizeof(uint32_t) * rows * d.skip_stride + 2 * hbytes + sizeof(uint64_t) * (P + 1) +
               16 * (d.n_fwd ? d.n_fwd : 1);
     idx->stats.n_entries = E;
