@@ -231,17 +231,28 @@ inline void mark(hicops_index* idx, int i, cudaStream_t s, bool on) {
 
 // Query preprocessing of n spectra (R8), then, with a fragment tolerance of
 // t > 0 bins, the widening of every spectrum's bins (R15).  qbin / qiq hold
-// query_bins_cap(p) words per spectrum.
+// query_bins_cap(p) words per spectrum.  Histograms and counts, where given,
+// are set to zero on the way.
 hicops_status prepare_queries(hicops_index* idx, const DevBatch& d, uint32_t n, uint32_t* qbin, uint32_t* qiq,
-                              uint32_t* qn, uint32_t* lo, uint32_t* hi, cudaStream_t s) {
+                              uint32_t* qn, uint32_t* lo, uint32_t* hi, uint32_t* hist, uint32_t* ns,
+                              cudaStream_t s) {
     const hicops_params& p = idx->p;
     const uint32_t stride = query_bins_cap(p);
+    auto not_below = [](double x) {      // the least float >= x
+        const float f = (float)x;
+        return (double)f < x ? std::nextafterf(f, INFINITY) : f;
+    };
+    int e;
+    const double f = std::frexp(1.0 / p.bin_width_da, &e);
+    // (a 1 / w outside the doubles has no such form: every bin by division)
+    const bool finite = std::isfinite(f) && f > 0.0;
     PrepArgs pa{d.peak_off, d.mz, d.inten, d.prec, d.z, d.tol, n, p.top_n_peaks, stride, p.bin_width_da,
-                p.frag_mz_min, p.frag_mz_max, (double)p.intensity_scale, idx->dev.mass, idx->mass.size(),
-                qbin, qiq, qn, lo, hi};
-    prep_warp_kernel<<<(n + kPrepWarps - 1) / kPrepWarps, kPrepWarps * 32, 0, s>>>(pa);
-    prep_kernel<<<n, kPrepThreads, 0, s>>>(pa);   // spectra of more than kPrepWarpPeaks peaks
-    count_launches(2);
+                not_below(p.frag_mz_min), not_below(p.frag_mz_max),
+                finite ? (uint64_t)std::ldexp(f, 64) : 0ull, finite ? e : 4096, p.intensity_scale,
+                idx->dev.mass, idx->mass.size(), qbin, qiq, qn, lo, hi, hist, ns};
+    const uint32_t big = std::min(n, kPrepBigBlocks);
+    prep_kernel<<<big + (n + kPrepWarps - 1) / kPrepWarps, kPrepThreads, 0, s>>>(pa, big);
+    count_launches(1);
     HC_CUDA(cudaGetLastError());
     if (p.tol_bins > 0) {
         ExpandArgs ea{qbin, qiq, qn, n, stride, p.tol_bins, idx->n_bins};
@@ -262,7 +273,7 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     const hicops_search_config cfg = resolved(cfg_in, query_bins_cap(idx->p));
     const uint32_t k = p.top_k;
     mark(idx, 0, s, timing_marks);
-    hicops_status st = prepare_queries(idx, d, n, w.qbin, w.qiq, w.qn, w.lo, w.hi, s);
+    hicops_status st = prepare_queries(idx, d, n, w.qbin, w.qiq, w.qn, w.lo, w.hi, d_hist, d_ns, s);
     if (st != HICOPS_OK) return st;
     mark(idx, 1, s, timing_marks);
     const uint32_t max_seg = w.max_seg;
@@ -285,8 +296,6 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
         count_launches(1);
     }
     HC_CUDA(cudaGetLastError());
-    HC_CUDA(cudaMemsetAsync(d_hist, 0, sizeof(uint32_t) * n * kHistBins, s));
-    HC_CUDA(cudaMemsetAsync(d_ns, 0, sizeof(uint32_t) * n, s));
     SearchArgs sa{w.qbin, w.qiq, w.qn, n, query_bins_cap(p), w.unit, w.seg_off + n, di.bins, di.entry, di.skip,
                   di.skip_stride, di.hot_b, di.hot_y, di.hot_words, di.fwd_off, reinterpret_cast<const uint4*>(di.fwd), di.lf, di.ls,
                   (uint32_t)idx->s_max, p.min_shared, k, cfg.chunk_entries < 16 ? cfg.chunk_entries * 1024u : 0xffffffffu, w.utop, d_hist, d_ns, w.work,
@@ -526,7 +535,7 @@ extern "C" hicops_status hicops_search_work(hicops_index* idx, const hicops_batc
         HC_CUDA(sc.get(&lo, n));
         HC_CUDA(sc.get(&hi, n));
         HC_CUDA(sc.get(&hits, n));
-        st = prepare_queries(idx, d, n, qbin, qiq, qn, lo, hi, s);
+        st = prepare_queries(idx, d, n, qbin, qiq, qn, lo, hi, nullptr, nullptr, s);
         if (st != HICOPS_OK) return st;
         work_kernel<<<n, 256, 0, s>>>(qbin, qn, lo, hi, query_bins_cap(p), idx->dev.off, idx->dev.entry, hits);
         count_launches(1);
