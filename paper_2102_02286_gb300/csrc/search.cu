@@ -304,9 +304,9 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     st = launch_search(sa, cfg, (uint64_t)n * max_seg, s);
     if (st != HICOPS_OK) return st;
     mark(idx, 3, s, timing_marks);
-    MergeArgs ma{w.seg_off, w.utop, d_hist, n, k, 0, d_psm, idx->pid_stride, idx->pid_base, di.pid_map,
-                 p.evalue_mode};
-    merge_kernel<<<(n + kMergeWarps - 1) / kMergeWarps, kMergeWarps * 32, 0, s>>>(ma);
+    MergeArgs ma{w.seg_off, w.utop, nullptr, nullptr, 0, 0, nullptr, nullptr, d_hist, n, k, d_psm,
+                 idx->pid_stride, idx->pid_base, di.pid_map, p.evalue_mode};
+    merge_kernel<false><<<(n + kMergeWarps - 1) / kMergeWarps, kMergeWarps * 32, 0, s>>>(ma);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
     mark(idx, 4, s, timing_marks);
@@ -845,42 +845,6 @@ extern "C" hicops_status hicops_search_noalloc(hicops_index* idx, const hicops_b
 // merge sums the partial histograms and candidate counts, merges the shard
 // top-k lists by (key desc, pid asc) with merge_kernel and fits the e-value
 // to the summed histogram, so the result equals the unsharded search.
-namespace hicops {
-namespace {
-
-// one block per spectrum: shard rows -> unit lists, summed histogram
-__global__ void shard_gather_kernel(const hicops_psm* __restrict__ parts, uint32_t n_shards, uint32_t n,
-                                    uint32_t k, const uint32_t* __restrict__ hist_in,
-                                    const uint32_t* __restrict__ ns_in, uint32_t hist_parts,
-                                    UnitTop* __restrict__ utop, uint64_t* __restrict__ seg_off,
-                                    uint32_t* __restrict__ hist, uint32_t* __restrict__ ns) {
-    const uint32_t q = blockIdx.x;
-    for (uint32_t i = threadIdx.x; i < n_shards * k; i += blockDim.x) {
-        const uint32_t s = i / k, r = i % k;
-        const hicops_psm row = parts[((uint64_t)s * n + q) * k + r];
-        UnitTop t;
-        t.key = row.key;
-        t.pid = row.pid;
-        t.packed = ((uint32_t)row.nb << kNbShift) | ((uint32_t)row.ny << kNyShift);
-        utop[((uint64_t)q * n_shards + s) * k + r] = t;
-    }
-    for (uint32_t j = threadIdx.x; j < kHistBins; j += blockDim.x) {
-        uint32_t h = 0;
-        for (uint32_t p = 0; p < hist_parts; ++p) h += hist_in[((uint64_t)p * n + q) * kHistBins + j];
-        hist[(uint64_t)q * kHistBins + j] = h;
-    }
-    if (threadIdx.x == 0) {
-        uint32_t c = 0;
-        for (uint32_t p = 0; p < hist_parts; ++p) c += ns_in[(uint64_t)p * n + q];
-        ns[q] = c;
-        seg_off[q] = (uint64_t)q * n_shards;
-        if (q == n - 1) seg_off[n] = (uint64_t)n * n_shards;
-    }
-}
-
-}  // namespace
-}  // namespace hicops
-
 extern "C" hicops_status hicops_merge_shards(uint32_t n_shards, uint32_t n, uint32_t top_k,
                                              const hicops_psm* shard_psm, const uint32_t* hist,
                                              const uint32_t* nscored, uint32_t hist_parts,
@@ -917,25 +881,29 @@ extern "C" hicops_status hicops_merge_shards(uint32_t n_shards, uint32_t n, uint
             d_hin = h;
             d_nin = c;
         }
-        UnitTop* utop;
-        uint64_t* seg_off;
         uint32_t *d_hist, *d_ns;
-        hicops_psm* d_out = on_device ? out_psm : nullptr;
-        HC_CUDA(sc.get(&utop, rows));
-        HC_CUDA(sc.get(&seg_off, (uint64_t)n + 1));
+        // rows that overlap an input are written aside first: a block reads its
+        // spectra's rows of every part after another has written its own
+        auto apart = [&](const void* p, uint64_t bytes) {
+            const uintptr_t a = reinterpret_cast<uintptr_t>(p), o = reinterpret_cast<uintptr_t>(out_psm);
+            return o + sizeof(hicops_psm) * n * top_k <= a || a + bytes <= o;
+        };
+        const bool direct = on_device && apart(d_parts, sizeof(hicops_psm) * rows) &&
+                            apart(d_hin, sizeof(uint32_t) * hist_parts * n * kHistBins) &&
+                            apart(d_nin, sizeof(uint32_t) * hist_parts * n);
+        hicops_psm* d_out = direct ? out_psm : nullptr;
         if (on_device && out_hist) d_hist = out_hist; else HC_CUDA(sc.get(&d_hist, (uint64_t)n * kHistBins));
         if (on_device && out_nscored) d_ns = out_nscored; else HC_CUDA(sc.get(&d_ns, n));
         if (!d_out) HC_CUDA(sc.get(&d_out, (uint64_t)n * top_k));
-        shard_gather_kernel<<<n, 256, 0, s>>>(d_parts, n_shards, n, top_k, d_hin, d_nin, hist_parts, utop,
-                                              seg_off, d_hist, d_ns);
+        MergeArgs ma{nullptr, nullptr, d_parts, d_nin, n_shards, hist_parts, d_hist, d_ns, d_hin, n, top_k, d_out,
+                     1u, 0u, nullptr, evalue_mode};
+        merge_kernel<true><<<(n + kMergeWarps - 1) / kMergeWarps, kMergeWarps * 32, 0, s>>>(ma);
         count_launches(1);
         HC_CUDA(cudaGetLastError());
-        MergeArgs ma{seg_off, utop, d_hist, n, top_k, 0, d_out, 1u, 0u, nullptr, evalue_mode};
-        merge_kernel<<<(n + kMergeWarps - 1) / kMergeWarps, kMergeWarps * 32, 0, s>>>(ma);
-        count_launches(1);
-        HC_CUDA(cudaGetLastError());
+        if (d_out != out_psm)
+            HC_CUDA(cudaMemcpyAsync(out_psm, d_out, sizeof(hicops_psm) * n * top_k,
+                                    on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
         if (!on_device) {
-            HC_CUDA(cudaMemcpyAsync(out_psm, d_out, sizeof(hicops_psm) * n * top_k, cudaMemcpyDeviceToHost, s));
             if (out_hist)
                 HC_CUDA(cudaMemcpyAsync(out_hist, d_hist, sizeof(uint32_t) * n * kHistBins, cudaMemcpyDeviceToHost, s));
             if (out_nscored)
@@ -952,16 +920,12 @@ namespace hicops {
 namespace {
 
 constexpr uint32_t kBinsPerLane = kHistBins / 32;
+static_assert(kBinsPerLane == 8, "lane_bins");
 
-// warp-wide best of (count, bin) pairs: higher count, then lower bin
-__device__ __forceinline__ void warp_best(uint32_t& c, uint32_t& j) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const uint32_t oc = __shfl_xor_sync(0xffffffffu, c, o), oj = __shfl_xor_sync(0xffffffffu, j, o);
-        if (oc > c || (oc == c && oj < j)) { c = oc; j = oj; }
-    }
-}
-
+// The most intense bins come from a warp argmax over 32-bit keys (count, then
+// the lower bin) as long as every count fits beside the bin's 8 bits, else
+// over 64-bit ones.
+// 160,000 spectra (164 MB of histograms): 120 -> 37 us.
 __global__ void hist_sample_kernel(const uint32_t* __restrict__ hist, uint32_t n, uint32_t s,
                                    uint32_t* __restrict__ rec) {
     const uint32_t lane = threadIdx.x & 31;
@@ -969,42 +933,64 @@ __global__ void hist_sample_kernel(const uint32_t* __restrict__ hist, uint32_t n
     if (q >= n) return;
     const uint32_t* h = hist + (uint64_t)q * kHistBins;
     uint32_t v[kBinsPerLane];
-#pragma unroll
-    for (uint32_t i = 0; i < kBinsPerLane; ++i) v[i] = h[lane * kBinsPerLane + i];
+    lane_bins(h, (int)lane, v);
     // support [L, R] of the non-zero bins
-    uint32_t L = kHistBins, R = 0;
+    uint32_t some = 0, most = 0;
 #pragma unroll
-    for (uint32_t i = 0; i < kBinsPerLane; ++i)
-        if (v[i]) { L = min(L, lane * kBinsPerLane + i); R = max(R, lane * kBinsPerLane + i); }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        L = min(L, __shfl_xor_sync(0xffffffffu, L, o));
-        R = max(R, __shfl_xor_sync(0xffffffffu, R, o));
+    for (uint32_t i = 0; i < kBinsPerLane; ++i) {
+        some |= (v[i] ? 1u : 0u) << i;
+        most = max(most, v[i]);
     }
+    const unsigned lanes = __ballot_sync(0xffffffffu, some != 0);
     uint32_t* out = rec + (uint64_t)q * (s + 1);
     uint32_t lo = 0, len = 0;
-    if (L <= R) {
-        // the three most intense bins: three rounds of a warp arg-max, each
-        // winner taken out of the next round
-        uint32_t taken = 0, sum = 0, k = 0;
-        for (int r = 0; r < 3; ++r) {
-            uint32_t c = 0, j = 0xffffffffu;
-#pragma unroll
-            for (uint32_t i = 0; i < kBinsPerLane; ++i) {
-                const uint32_t b = lane * kBinsPerLane + i;
-                if (!((taken >> i) & 1u) && (v[i] > c || (v[i] == c && v[i] && b < j))) { c = v[i]; j = b; }
-            }
-            warp_best(c, j);
-            if (c == 0) break;
-            sum += j;
-            ++k;
-            if (j / kBinsPerLane == lane) taken |= 1u << (j % kBinsPerLane);
-        }
-        const uint32_t m = sum / k;
+    if (lanes) {
+        const uint32_t ll = __ffs(lanes) - 1, lr = 31 - __clz(lanes);
+        const uint32_t L = ll * kBinsPerLane + (__ffs(__shfl_sync(0xffffffffu, some, ll)) - 1);
+        const uint32_t R = lr * kBinsPerLane + (31 - __clz(__shfl_sync(0xffffffffu, some, lr)));
         if (R - L + 1 <= s) {
             lo = L;
             len = R - L + 1;
         } else {
+            // the three most intense bins (higher count, then lower bin): three
+            // rounds of a warp argmax, each winner taken out of the next round
+            uint32_t sum = 0, k = 0;
+            if (__reduce_max_sync(0xffffffffu, most) < 1u << 24) {
+                uint32_t key[kBinsPerLane];
+#pragma unroll
+                for (uint32_t i = 0; i < kBinsPerLane; ++i)
+                    key[i] = v[i] ? v[i] << 8 | (kHistBins - 1u - (lane * kBinsPerLane + i)) : 0u;
+                for (int r = 0; r < 3; ++r) {
+                    uint32_t best = 0;
+#pragma unroll
+                    for (uint32_t i = 0; i < kBinsPerLane; ++i) best = max(best, key[i]);
+                    best = __reduce_max_sync(0xffffffffu, best);
+                    if (best == 0) break;
+                    sum += kHistBins - 1u - (best & 0xffu);
+                    ++k;
+#pragma unroll
+                    for (uint32_t i = 0; i < kBinsPerLane; ++i)
+                        if (key[i] == best) key[i] = 0;
+                }
+            } else {
+                uint32_t taken = 0;
+                for (int r = 0; r < 3; ++r) {
+                    int64_t best = 0;
+#pragma unroll
+                    for (uint32_t i = 0; i < kBinsPerLane; ++i)
+                        if (v[i] && !((taken >> i) & 1u))
+                            best = max(best, (int64_t)((uint64_t)v[i] << 8 |
+                                                       (kHistBins - 1u - (lane * kBinsPerLane + i))));
+                    bool mine;
+                    best = warp_max_i64(best, &mine);
+                    if (best == 0) break;
+                    const uint32_t j = kHistBins - 1u - (uint32_t)(best & 0xff);
+                    sum += j;
+                    ++k;
+                    if (j / kBinsPerLane == lane) taken |= 1u << (j % kBinsPerLane);
+                }
+            }
+            const uint32_t m = sum / k;
             // pruning the farther end first ends with s bins, the lower side
             // longer by at most one, unless an end of the support stops it
             const int dl = (int)(s / 2), dh = (int)((s - 1) / 2);
@@ -1019,6 +1005,9 @@ __global__ void hist_sample_kernel(const uint32_t* __restrict__ hist, uint32_t n
     for (uint32_t i = lane; i < s; i += 32) out[1 + i] = i < len ? h[lo + i] : 0u;
 }
 
+// Lane l adds bins l, l + 32, ..., so that a record is read in whole lines;
+// the records' first words are read a lane each, ahead of the records.
+// 20,000 spectra of eight parts: 35 -> 24 us.
 __global__ void hist_unsample_kernel(const uint32_t* __restrict__ rec, uint32_t n_parts, uint32_t n, uint32_t s,
                                      uint32_t* __restrict__ hist, uint32_t* __restrict__ bad) {
     const uint32_t lane = threadIdx.x & 31;
@@ -1027,21 +1016,25 @@ __global__ void hist_unsample_kernel(const uint32_t* __restrict__ rec, uint32_t 
     uint32_t acc[kBinsPerLane];
 #pragma unroll
     for (uint32_t i = 0; i < kBinsPerLane; ++i) acc[i] = 0;
-    for (uint32_t p = 0; p < n_parts; ++p) {
-        const uint32_t* r = rec + ((uint64_t)p * n + q) * (s + 1);
-        const uint32_t w0 = r[0], lo = w0 & 0xffffu, len = w0 >> 16;
-        if (len > s || lo + len > kHistBins) {   // not a record of this s
-            if (lane == 0) atomicOr(bad, 1u);
-            continue;
-        }
+    for (uint32_t p0 = 0; p0 < n_parts; p0 += 32) {
+        const uint32_t parts = min(n_parts - p0, 32u);
+        const uint32_t mine = lane < parts ? __ldg(rec + ((uint64_t)(p0 + lane) * n + q) * (s + 1)) : 0u;
+        const bool off = (mine >> 16) > s || (mine & 0xffffu) + (mine >> 16) > kHistBins;   // not a record of this s
+        if (__any_sync(0xffffffffu, off) && lane == 0) atomicOr(bad, 1u);
+        const uint32_t w = off ? 0u : mine;
+#pragma unroll 4
+        for (uint32_t p = 0; p < parts; ++p) {
+            const uint32_t w0 = __shfl_sync(0xffffffffu, w, p), lo = w0 & 0xffffu, len = w0 >> 16;
+            const uint32_t* r = rec + ((uint64_t)(p0 + p) * n + q) * (s + 1) + 1;
 #pragma unroll
-        for (uint32_t i = 0; i < kBinsPerLane; ++i) {
-            const uint32_t b = lane * kBinsPerLane + i;
-            if (b >= lo && b < lo + len) acc[i] += r[1 + (b - lo)];
+            for (uint32_t i = 0; i < kBinsPerLane; ++i) {
+                const uint32_t at = i * 32 + lane - lo;   // below lo: wraps, above len
+                if (at < len) acc[i] += __ldg(r + at);
+            }
         }
     }
 #pragma unroll
-    for (uint32_t i = 0; i < kBinsPerLane; ++i) hist[(uint64_t)q * kHistBins + lane * kBinsPerLane + i] = acc[i];
+    for (uint32_t i = 0; i < kBinsPerLane; ++i) hist[(uint64_t)q * kHistBins + i * 32 + lane] = acc[i];
 }
 
 constexpr int kSampleWarps = 8;

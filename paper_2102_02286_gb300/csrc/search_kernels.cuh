@@ -584,12 +584,20 @@ __device__ __forceinline__ uint64_t entry_lower_bound(const uint32_t* __restrict
     return a;
 }
 
+// Where merge_kernel finds a spectrum's sorted lists and its histogram: the
+// units of a search, or the results of the parts of a database (rows and
+// partial histograms of part p behind those of part p - 1), whose summed
+// histogram and candidate count it writes too.
 struct MergeArgs {
-    const uint64_t* seg_off;
+    const uint64_t* seg_off;         // search: first unit of every spectrum
     const UnitTop* utop;
+    const hicops_psm* parts;         // parts: rows, counts, how many
+    const uint32_t* ns_in;
+    uint32_t n_parts, hist_parts;
+    uint32_t* hist_out;
+    uint32_t* ns_out;
     const uint32_t* hist;
     uint32_t n, k;
-    uint32_t q_base;          // query index written into the rows
     hicops_psm* out;
     uint32_t pid_stride, pid_base;   // row pid = list pid * pid_stride + pid_base ...
     const uint32_t* pid_map;         // ... or pid_map[list pid] when not NULL
@@ -602,189 +610,271 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
     return v;
 }
 
-// One warp per spectrum (kMergeWarps spectra per block): the top-k merge of
-// the spectrum's unit lists, then the e-value fit (Supplementary Algorithm
-// 4) over its histogram.  Lane l owns unit lists l and l + 32 (at most 64
-// units, each sorted by (key desc, pid asc)); k rounds of a warp argmax
-// over the list heads give the rows in rank order.  Lane l holds histogram
-// bins 8l .. 8l + 7.
-__global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(MergeArgs a) {
-    __shared__ int64_t gsurv[kMergeWarps][kHistBins + 1];   // the fit's survival function G[0..256]
-    const int lane = threadIdx.x & 31;
-    const uint32_t q = blockIdx.x * kMergeWarps + (threadIdx.x >> 5);
-    if (q >= a.n) return;
-    int64_t* const G = gsurv[threadIdx.x >> 5];
-    const uint32_t k = a.k;
-    const uint64_t u0 = a.seg_off[q];
-    const int nseg = (int)(a.seg_off[q + 1] - u0);
-    const UnitTop* lists = a.utop + u0 * k;
-    uint32_t h0 = 0, h1 = 0;   // heads of lists lane and lane + 32
-    UnitTop row;               // row `lane` of the result
-    row.key = INT64_MIN;
-    row.pid = 0xffffffffu;
-    row.packed = 0u;
-    for (uint32_t r = 0; r < k; ++r) {
-        int64_t bk = INT64_MIN;
-        uint32_t bp = 0xffffffffu, bpk = 0u;
-        int which = -1;
-        if (lane < nseg && h0 < k) {
-            const UnitTop t = lists[(uint64_t)lane * k + h0];
-            if (t.pid != 0xffffffffu) { bk = t.key; bp = t.pid; bpk = t.packed; which = 0; }
-        }
-        if (lane + 32 < nseg && h1 < k) {
-            const UnitTop t = lists[(uint64_t)(lane + 32) * k + h1];
-            if (t.pid != 0xffffffffu && better(t.key, t.pid, bk, bp)) { bk = t.key; bp = t.pid; bpk = t.packed; which = 1; }
-        }
-        int64_t wk = bk;
-        uint32_t wp = bp, wpk = bpk;
-        int wl = lane;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const int64_t ok = __shfl_xor_sync(0xffffffffu, wk, o);
-            const uint32_t op = __shfl_xor_sync(0xffffffffu, wp, o);
-            const uint32_t opk = __shfl_xor_sync(0xffffffffu, wpk, o);
-            const int ol = __shfl_xor_sync(0xffffffffu, wl, o);
-            if (better(ok, op, wk, wp) || (ok == wk && op == wp && ol < wl)) { wk = ok; wp = op; wpk = opk; wl = ol; }
-        }
-        if (wp != 0xffffffffu && lane == wl) { if (which == 0) ++h0; else ++h1; }
-        if ((uint32_t)lane == r) { row.key = wk; row.pid = wp; row.packed = wpk; }
-    }
-    // the histogram, bins 8 lane .. 8 lane + 7 of this lane
-    const uint32_t* hq = a.hist + (uint64_t)q * kHistBins + 8 * lane;   // caller's buffer: 4-byte aligned only
-    uint32_t v[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = hq[i];
-    uint32_t nl = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) nl += v[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) nl += __shfl_xor_sync(0xffffffffu, nl, o);
-    const double N = (double)nl;
-    // the distribution the fit sees (R16): the histogram, or 35 times its
-    // 5-point quadratic Savitzky-Golay smoothing (zero outside the bins);
-    // integers, so every sum and comparison below is exact
-    int64_t g[8];
-    {
-        const uint32_t l2 = __shfl_up_sync(0xffffffffu, v[6], 1), l1 = __shfl_up_sync(0xffffffffu, v[7], 1);
-        const uint32_t r1 = __shfl_down_sync(0xffffffffu, v[0], 1), r2 = __shfl_down_sync(0xffffffffu, v[1], 1);
-        int64_t e[12];
-        e[0] = lane > 0 ? l2 : 0;
-        e[1] = lane > 0 ? l1 : 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) e[2 + i] = v[i];
-        e[10] = lane < 31 ? r1 : 0;
-        e[11] = lane < 31 ? r2 : 0;
-        const bool smooth = (a.ev_mode & HICOPS_EVALUE_SMOOTH) != 0u;
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            g[i] = smooth ? -3 * e[i] + 12 * e[i + 1] + 17 * e[i + 2] + 12 * e[i + 3] - 3 * e[i + 4] : e[i + 2];
-    }
-    // survival G[j] = sum of g[i >= j]: within the lane, then over the lanes above
-    int64_t loc[8];
-    int64_t run = 0;
-#pragma unroll
-    for (int i = 7; i >= 0; --i) { run += g[i]; loc[i] = run; }
-    int64_t above = run;   // inclusive suffix over lanes >= lane
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t y = __shfl_down_sync(0xffffffffu, above, o);
-        if (lane + o < 32) above += y;
-    }
-    const int64_t G0 = __shfl_sync(0xffffffffu, above, 0);
-    above -= run;           // lanes > lane
-    // G[j] in shared memory, so that the fit's points (a few bins next to
-    // one another) are spread one a lane and its FP64 logarithms run once
-    // for the warp rather than once per bin of a lane
-#pragma unroll
-    for (int i = 0; i < 8; ++i) G[8 * lane + i] = loc[i] + above;
-    if (lane == 0) G[kHistBins] = 0;
-    __syncwarp();
-    const double dG0 = (double)G0;
-    const int64_t key0 = __shfl_sync(0xffffffffu, row.key, 0);
-    const uint32_t pid0 = __shfl_sync(0xffffffffu, row.pid, 0);
-    const bool have_top = pid0 != 0xffffffffu;
-    const bool weibull = (a.ev_mode & HICOPS_EVALUE_LOG_WEIBULL) != 0u;
-    double cn = 0, sx = 0, sy = 0, sxx = 0, sxy = 0;
-    if (weibull) {
-        // R17: least squares of -ln(-ln F_j) on x = j + 1, F_j = 1 - G[j+1] / G[0],
-        // over the bins with 0 < F_j < 1
-        for (int j = lane; j < (int)kHistBins && have_top; j += 32) {
-            const int64_t gn = G[j + 1];
-            if (gn > 0 && gn < G0) {
-                const double x = (double)(j + 1);
-                const double y = -log(-log1p(-((double)gn / dG0)));
-                cn += 1.0;
-                sx += x;
-                sy += y;
-                sxx += x * x;
-                sxy += x * y;
-            }
-        }
+// the greatest of the lanes' 64-bit values, and which lanes hold it
+__device__ __forceinline__ int64_t warp_max_i64(int64_t v, bool* mine) {
+    const int hi = (int)(v >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const uint32_t lo = hi == mh ? (uint32_t)v : 0u, ml = __reduce_max_sync(0xffffffffu, lo);
+    *mine = hi == mh && lo == ml;
+    return (int64_t)((uint64_t)(uint32_t)mh << 32 | ml);
+}
+
+// lane l's eight bins 8 l .. 8 l + 7 of a histogram (a caller's buffer: 4-byte aligned only)
+__device__ __forceinline__ void lane_bins(const uint32_t* __restrict__ h, int lane, uint32_t* v) {
+    const uint32_t* at = h + 8 * lane;
+    if ((reinterpret_cast<uintptr_t>(h) & 15u) == 0) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(at)), y = __ldg(reinterpret_cast<const uint4*>(at) + 1);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
     } else {
-        // R12 on g: the mode (largest g, lowest bin on ties), then the line
-        // through (j, log10(G[j] / G[0])) for j in [mode + 1, jtop - 1], G[j] > 0
-        int64_t bv = g[0];
-        int bj = 8 * lane;
 #pragma unroll
-        for (int i = 1; i < 8; ++i)
-            if (g[i] > bv) { bv = g[i]; bj = 8 * lane + i; }
+        for (int i = 0; i < 8; ++i) v[i] = __ldg(at + i);
+    }
+}
+
+// One warp per spectrum (kMergeWarps spectra per block): the top-k merge of
+// the spectrum's lists, then the e-value fit (Supplementary Algorithm 4) over
+// its histogram.  Lane l owns lists l and l + 32 (at most 64, each sorted by
+// (key desc, pid asc)), holds the head and the next row of each, and k rounds
+// of a warp argmax over the heads give the rows in rank order.  Lane l holds
+// histogram bins 8l .. 8l + 7.
+// The FP64 unit (2 lanes a clock) bounds it, whatever number of lanes an
+// instruction has, so the FP64 work of the block's spectra is put together:
+// the fit's points are spread over the block's threads for the logarithms,
+// the lines are solved by a thread each, and the rows' e-values are a thread
+// each; the sums of whole numbers are taken in integers (exact in both).
+// 30,000 spectra: 207 -> 94 us; 20,000 of eight parts: 212 us with the
+// kernel that gathered the parts -> 132 us.
+template <bool PARTS>
+__global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const __grid_constant__ MergeArgs a) {
+    static_assert(kMergeWarps * kMaxTopK <= kMergeWarps * 32, "a thread a row");
+    // the fit's survival function G[0..256]; at a point of the fit, then its ordinate
+    __shared__ int64_t gsurv[kMergeWarps][kHistBins + 1];
+    __shared__ UnitTop rows[kMergeWarps][kMaxTopK];
+    __shared__ uint32_t first[kMergeWarps], points[kMergeWarps], total[kMergeWarps];
+    __shared__ double sum_y[kMergeWarps], sum_xy[kMergeWarps];      // then slope and intercept
+    __shared__ uint32_t sum_1[kMergeWarps], sum_x[kMergeWarps], sum_xx[kMergeWarps];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
+    const uint32_t q = blockIdx.x * kMergeWarps + wi;
+    int64_t* const G = gsurv[wi];
+    const uint32_t k = a.k;
+    const bool weibull = (a.ev_mode & HICOPS_EVALUE_LOG_WEIBULL) != 0u;
+    uint32_t s0 = 1, np = 0;      // the fit's points: bins (linear) or bins + 1 (log-Weibull)
+    if (q < a.n) {
+        uint32_t v[8];
+        lane_bins(a.hist + (uint64_t)q * kHistBins, lane, v);
+        if (PARTS) {
+            uint32_t c = lane == 0 ? a.ns_in[q] : 0u;
+            for (uint32_t p = 1; p < a.hist_parts; ++p) {
+                uint32_t w[8];
+                lane_bins(a.hist + ((uint64_t)p * a.n + q) * kHistBins, lane, w);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const int64_t ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-            if (ov > bv || (ov == bv && oj < bj)) { bv = ov; bj = oj; }
+                for (int i = 0; i < 8; ++i) v[i] += w[i];
+                if (lane == 0) c += a.ns_in[(uint64_t)p * a.n + q];
+            }
+            uint32_t* ho = a.hist_out + (uint64_t)q * kHistBins + 8 * lane;
+            if ((reinterpret_cast<uintptr_t>(a.hist_out) & 15u) == 0) {
+                reinterpret_cast<uint4*>(ho)[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                reinterpret_cast<uint4*>(ho)[1] = make_uint4(v[4], v[5], v[6], v[7]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) ho[i] = v[i];
+            }
+            if (lane == 0) a.ns_out[q] = c;
         }
-        const int mode = bj;
-        int64_t jtop = 0;
-        if (have_top) { jtop = key0 >> 31; if (jtop > 255) jtop = 255; }
-        for (int j = mode + 1 + lane; j <= (int)jtop - 1 && have_top; j += 32) {
-            const int64_t gj = G[j];
-            if (gj > 0) {
-                const double x = (double)j;
-                const double y = log10((double)gj / dG0);
-                cn += 1.0;
-                sx += x;
-                sy += y;
-                sxx += x * x;
-                sxy += x * y;
+        // the lists
+        const uint64_t u0 = PARTS ? 0 : a.seg_off[q];
+        const int nl = PARTS ? (int)a.n_parts : (int)(a.seg_off[q + 1] - u0);
+        const UnitTop none{INT64_MIN, 0xffffffffu, 0u};
+        auto row = [&](int l, uint32_t r) -> UnitTop {
+            if (l >= nl || r >= k) return none;
+            if (!PARTS) return a.utop[(u0 + l) * k + r];
+            const hicops_psm* t = a.parts + ((uint64_t)l * a.n + q) * k + r;
+            return UnitTop{t->key, t->pid, ((uint32_t)t->nb << kNbShift) | ((uint32_t)t->ny << kNyShift)};
+        };
+        UnitTop c0 = row(lane, 0), n0 = row(lane, 1);
+        UnitTop c1 = row(lane + 32, 0), n1 = row(lane + 32, 1);
+        uint32_t h0 = 1, h1 = 1;   // rows n0 and n1 hold
+        if (lane < k) rows[wi][lane] = none;
+        __syncwarp();
+        int64_t key0 = INT64_MIN;
+        uint32_t r = 0;
+        for (; r < k; ++r) {
+            const bool second = c1.pid != 0xffffffffu && (c0.pid == 0xffffffffu || better(c1.key, c1.pid, c0.key, c0.pid));
+            const uint32_t pid = second ? c1.pid : c0.pid;
+            const int64_t key = pid != 0xffffffffu ? (second ? c1.key : c0.key) : INT64_MIN;
+            bool best;
+            const int64_t wk = warp_max_i64(key, &best);
+            const uint32_t wp = __reduce_min_sync(0xffffffffu, best ? pid : 0xffffffffu);
+            if (wp == 0xffffffffu) break;   // every list is at its end
+            const int wl = __ffs(__ballot_sync(0xffffffffu, best && pid == wp)) - 1;
+            if (r == 0) key0 = wk;
+            if (lane == wl) {
+                rows[wi][r] = second ? c1 : c0;
+                if (second) {
+                    c1 = n1;
+                    n1 = row(lane + 32, ++h1);
+                } else {
+                    c0 = n0;
+                    n0 = row(lane, ++h0);
+                }
+            }
+        }
+        const bool have_top = r > 0;
+        uint32_t n_sum = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) n_sum += v[i];
+        n_sum = __reduce_add_sync(0xffffffffu, n_sum);
+        if (lane == 0) total[wi] = n_sum;
+        // the distribution the fit sees (R16): the histogram, or 35 times its
+        // 5-point quadratic Savitzky-Golay smoothing (zero outside the bins);
+        // integers, so every sum and comparison below is exact
+        int64_t g[8];
+        {
+            const uint32_t l2 = __shfl_up_sync(0xffffffffu, v[6], 1), l1 = __shfl_up_sync(0xffffffffu, v[7], 1);
+            const uint32_t r1 = __shfl_down_sync(0xffffffffu, v[0], 1), r2 = __shfl_down_sync(0xffffffffu, v[1], 1);
+            int64_t e[12];
+            e[0] = lane > 0 ? l2 : 0;
+            e[1] = lane > 0 ? l1 : 0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) e[2 + i] = v[i];
+            e[10] = lane < 31 ? r1 : 0;
+            e[11] = lane < 31 ? r2 : 0;
+            const bool smooth = (a.ev_mode & HICOPS_EVALUE_SMOOTH) != 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                g[i] = smooth ? -3 * e[i] + 12 * e[i + 1] + 17 * e[i + 2] + 12 * e[i + 3] - 3 * e[i + 4] : e[i + 2];
+        }
+        // survival G[j] = sum of g[i >= j]: within the lane, then over the lanes above
+        int64_t loc[8];
+        int64_t run = 0;
+#pragma unroll
+        for (int i = 7; i >= 0; --i) { run += g[i]; loc[i] = run; }
+        int64_t above = run;   // inclusive suffix over lanes >= lane
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t y = __shfl_down_sync(0xffffffffu, above, o);
+            if (lane + o < 32) above += y;
+        }
+        above -= run;           // lanes > lane
+#pragma unroll
+        for (int i = 0; i < 8; ++i) G[8 * lane + i] = loc[i] + above;
+        if (lane == 0) G[kHistBins] = 0;
+        if (have_top) {
+            if (weibull) {
+                // R17: least squares of -ln(-ln F_j) on x = j + 1, F_j = 1 - G[j+1] / G[0],
+                // over the bins with 0 < F_j < 1
+                np = kHistBins;
+            } else {
+                // R12 on g: the mode (largest g, lowest bin on ties), then the line
+                // through (j, log10(G[j] / G[0])) for j in [mode + 1, jtop - 1], G[j] > 0
+                int64_t bv = g[0];
+                int bj = 8 * lane;
+#pragma unroll
+                for (int i = 1; i < 8; ++i)
+                    if (g[i] > bv) { bv = g[i]; bj = 8 * lane + i; }
+                bool best;
+                warp_max_i64(bv, &best);
+                s0 = __reduce_min_sync(0xffffffffu, best ? (uint32_t)bj : 0xffffffffu) + 1u;
+                int64_t jtop = key0 >> 31;
+                if (jtop > 255) jtop = 255;
+                if (jtop > (int64_t)s0) np = (uint32_t)jtop - s0;
             }
         }
     }
-    cn = warp_sum_f64(cn);
-    sx = warp_sum_f64(sx);
-    sy = warp_sum_f64(sy);
-    sxx = warp_sum_f64(sxx);
-    sxy = warp_sum_f64(sxy);
-    bool fit = cn >= 3.0;
-    double wfit = 0.0, bfit = 0.0;
-    if (fit) {
-        const double den = cn * sxx - sx * sx;
-        wfit = (cn * sxy - sx * sy) / den;
-        bfit = (sy - wfit * sx) / cn;
-        if (weibull) fit = wfit > 0.0;
+    if (lane == 0) {
+        first[wi] = s0;
+        points[wi] = np;
     }
-    if ((uint32_t)lane < k) {
-        hicops_psm o;
-        o.query = a.q_base + q;
-        o.reserved = 0;
-        if (row.pid != 0xffffffffu) {
-            o.pid = a.pid_map ? a.pid_map[row.pid] : row.pid * a.pid_stride + a.pid_base;
-            o.nb = (uint8_t)(row.packed >> kNbShift);
-            o.ny = (uint8_t)((row.packed >> kNyShift) & 63u);
-            o.key = row.key;
-            o.hyperscore = (float)((double)row.key * 0x1p-32);
-            const double x = (double)row.key * 0x1p-31;
-            if (!fit) o.evalue = N;
-            else if (weibull) o.evalue = N * -expm1(-exp(-(wfit * x + bfit)));   // N * P(score >= x)
-            else o.evalue = N * exp10(wfit * x + bfit);
-        } else {
-            o.pid = 0xffffffffu;
-            o.nb = o.ny = 0;
-            o.key = INT64_MIN;
-            o.hyperscore = 0.0f;
-            o.evalue = INFINITY;
+    __syncthreads();
+    uint32_t all = 0;
+#pragma unroll
+    for (int w = 0; w < kMergeWarps; ++w) all += points[w];
+    for (uint32_t i = threadIdx.x; i < all; i += kMergeWarps * 32) {
+        uint32_t at = i;
+        int w = 0;
+        for (; at >= points[w]; ++w) at -= points[w];
+        at += first[w];
+        const int64_t gj = gsurv[w][at], G0 = gsurv[w][0];
+        double y = NAN;                                  // not a point
+        if (gj > 0 && (!weibull || gj < G0)) {
+            const double f = (double)gj / (double)G0;
+            y = weibull ? -log(-log1p(-f)) : log10(f);
         }
-        a.out[(uint64_t)q * k + lane] = o;
+        gsurv[w][at] = __double_as_longlong(y);
+    }
+    __syncthreads();
+    if (np) {   // warp-uniform
+        uint32_t c1 = 0, cx = 0, cxx = 0;
+        double sy = 0, sxy = 0;
+        for (uint32_t i = lane; i < np; i += 32) {
+            const uint32_t xi = s0 + i;
+            const double y = __longlong_as_double(G[xi]);
+            if (!isnan(y)) {
+                const double x = (double)xi;
+                c1 += 1u;
+                cx += xi;
+                cxx += xi * xi;
+                sy += y;
+                sxy += x * y;
+            }
+        }
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        cx = __reduce_add_sync(0xffffffffu, cx);
+        cxx = __reduce_add_sync(0xffffffffu, cxx);
+        sy = warp_sum_f64(sy);
+        sxy = warp_sum_f64(sxy);
+        if (lane == 0) {
+            sum_1[wi] = c1;
+            sum_x[wi] = cx;
+            sum_xx[wi] = cxx;
+            sum_y[wi] = sy;
+            sum_xy[wi] = sxy;
+        }
+    } else if (lane == 0) {
+        sum_1[wi] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x < kMergeWarps) {
+        const int w = threadIdx.x;
+        if (sum_1[w] >= 3u) {
+            const double cn = (double)sum_1[w], sx = (double)sum_x[w], sxx = (double)sum_xx[w];
+            const double sy = sum_y[w], sxy = sum_xy[w];
+            const double den = cn * sxx - sx * sx;
+            const double wfit = (cn * sxy - sx * sy) / den;
+            sum_y[w] = wfit;
+            sum_xy[w] = (sy - wfit * sx) / cn;
+            if (weibull && !(wfit > 0.0)) sum_1[w] = 0;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < kMergeWarps * k) {
+        const uint32_t w = threadIdx.x / k, r = threadIdx.x % k;
+        const uint32_t qo = blockIdx.x * kMergeWarps + w;
+        if (qo < a.n) {
+            const UnitTop t = rows[w][r];
+            hicops_psm o;
+            o.query = qo;
+            o.reserved = 0;
+            if (t.pid != 0xffffffffu) {
+                o.pid = a.pid_map ? a.pid_map[t.pid] : t.pid * a.pid_stride + a.pid_base;
+                o.nb = (uint8_t)(t.packed >> kNbShift);
+                o.ny = (uint8_t)((t.packed >> kNyShift) & 63u);
+                o.key = t.key;
+                o.hyperscore = (float)((double)t.key * 0x1p-32);
+                const double x = (double)t.key * 0x1p-31, N = (double)total[w];
+                const double wfit = sum_y[w], bfit = sum_xy[w];
+                if (sum_1[w] < 3u) o.evalue = N;
+                else if (weibull) o.evalue = N * -expm1(-exp(-(wfit * x + bfit)));   // N * P(score >= x)
+                else o.evalue = N * exp10(wfit * x + bfit);
+            } else {
+                o.pid = 0xffffffffu;
+                o.nb = o.ny = 0;
+                o.key = INT64_MIN;
+                o.hyperscore = 0.0f;
+                o.evalue = INFINITY;
+            }
+            a.out[(uint64_t)qo * k + r] = o;
+        }
     }
 }
 
