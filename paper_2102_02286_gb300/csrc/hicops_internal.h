@@ -57,6 +57,7 @@ struct DeviceIndex {
                                    // bucket padded to a multiple of 4 with 0xffffffff (16-byte groups)
     uint64_t n_stored = 0;         // entries including the pads (off[n_bins])
     int64_t* lf = nullptr;         // [kMaxLen + 1] LF[n] = round(2^32 log10 n!)
+    void* pool = nullptr;          // cudaMemPool_t: scratch of hicops_search calls (upload_index)
     int64_t* ls = nullptr;         // [s_max + 1]   LS[s] = round(2^32 log10 s)
     // chunk skip table of every non-empty bucket: row[bin] (-1 empty) and
     // skip[row * skip_stride + j] = entries with pid < j << kChunkShift

@@ -17,6 +17,7 @@ namespace hicops {
 namespace {
 
 constexpr int kIonThreads = 128;
+constexpr uint64_t kPoolKeep = 128ull << 20;   // 12,000 spectra of 500 peaks; no more for 64 shards than 8 GB
 constexpr int kIonStage = 2048;      // ion bins a warp stages in shared memory (8 KB)
 
 struct IonArgs {
@@ -491,6 +492,7 @@ void free_device_index(hicops_index* idx) {
         cudaFree(d.fwd);
         cudaFree(d.pid_map);
         for (void* e : d.ev) if (e) cudaEventDestroy((cudaEvent_t)e);
+        if (d.pool) cudaMemPoolDestroy((cudaMemPool_t)d.pool);   // (the frees above have waited for its last call)
         if (cur >= 0 && cur != d.device) cudaSetDevice(cur);
     }
     d = DeviceIndex{};
@@ -508,6 +510,19 @@ hicops_status upload_index(hicops_index* idx) {
     cudaStream_t s;
     HC_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
     struct StreamGuard { cudaStream_t s; ~StreamGuard() { cudaStreamSynchronize(s); cudaStreamDestroy(s); } } sg{s};
+
+    // Scratch of the searches: a pool of the index's own, which keeps up to
+    // kPoolKeep bytes over a synchronisation.  The device's default pool keeps
+    // none, and mapping a search's scratch anew costs it 200 us.
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = d.device;
+    cudaMemPool_t pool;
+    HC_CUDA(cudaMemPoolCreate(&pool, &props));
+    d.pool = pool;
+    uint64_t keep = kPoolKeep;
+    HC_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
 
     // persistent parts
     HC_CUDA(cudaMalloc(&d.mass, sizeof(double) * (P ? P : 1)));

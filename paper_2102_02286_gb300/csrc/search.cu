@@ -10,7 +10,7 @@
 //   exclusive scan
 //   search_kernel  filter_2 + score + heap over persistent CTAs;
 //   merge_kernel   per-spectrum top-k merge and the survival-tail e-value.
-// hicops_search allocates its scratch stream-ordered per call; a plan
+// hicops_search takes its scratch stream-ordered from its index's pool; a plan
 // (hicops_plan_*) allocates it once and can replay the sequence as a CUDA
 // graph.
 #include <algorithm>
@@ -39,14 +39,16 @@ struct DevBatch {
     const double* tol;
 };
 
-// stream-ordered scratch; freed on every exit path
+// stream-ordered scratch from a pool (or the device's default one); freed on every exit path
 struct Scratch {
     cudaStream_t s;
+    cudaMemPool_t pool;
     std::vector<void*> ptrs;
-    explicit Scratch(cudaStream_t st) : s(st) {}
+    explicit Scratch(cudaStream_t st, cudaMemPool_t p = nullptr) : s(st), pool(p) {}
     template <class T>
     cudaError_t get(T** p, uint64_t n) {
-        cudaError_t e = cudaMallocAsync((void**)p, sizeof(T) * (n ? n : 1), s);
+        const size_t bytes = sizeof(T) * (n ? n : 1);
+        cudaError_t e = pool ? cudaMallocFromPoolAsync((void**)p, bytes, pool, s) : cudaMallocAsync((void**)p, bytes, s);
         if (e == cudaSuccess) ptrs.push_back(*p);
         return e;
     }
@@ -63,6 +65,34 @@ struct Arena {
         return e;
     }
     ~Arena() { for (void* p : ptrs) cudaFree(p); }
+};
+
+constexpr uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
+
+// alloc_workspace's allocators over caller memory.  Carve hands out
+// consecutive 256-byte aligned pieces of one buffer and fails when they would
+// not fit; Tally only adds up the bytes Carve would hand out.
+struct Carve {
+    unsigned char* base;
+    uint64_t cap, used;
+    template <class T>
+    cudaError_t get(T** p, uint64_t n) {
+        const uint64_t bytes = align256(sizeof(T) * (n ? n : 1));
+        if (used + bytes > cap) return cudaErrorMemoryAllocation;
+        *p = reinterpret_cast<T*>(base + used);
+        used += bytes;
+        return cudaSuccess;
+    }
+};
+
+struct Tally {
+    uint64_t used = 0;
+    template <class T>
+    cudaError_t get(T** p, uint64_t n) {
+        *p = nullptr;
+        used += align256(sizeof(T) * (n ? n : 1));
+        return cudaSuccess;
+    }
 };
 
 // Device scratch of one search of up to cap_n spectra.
@@ -329,9 +359,9 @@ hicops_status check_batch(const hicops_index* idx, const hicops_batch* b) {
     return sm_count();
 }
 
-// Inputs on the device (copied from the host when on_device = 0).
-hicops_status stage_inputs(const hicops_batch* b, Scratch& sc, DevBatch& d) {
-    const cudaStream_t s = sc.s;
+// Inputs on the device: the caller's, or (on_device = 0) pieces to copy them to.
+template <class A>
+hicops_status place_inputs(A& al, const hicops_batch* b, DevBatch& d) {
     if (b->on_device) {
         d = DevBatch{b->peak_off, b->mz, b->intensity, b->prec_mz, b->charge, b->prec_tol_da};
         return HICOPS_OK;
@@ -342,51 +372,30 @@ hicops_status stage_inputs(const hicops_batch* b, Scratch& sc, DevBatch& d) {
     float *mz, *it;
     double *pr, *tl;
     uint8_t* z;
-    HC_CUDA(sc.get(&po, b->n + 1));
-    HC_CUDA(sc.get(&mz, npk));
-    HC_CUDA(sc.get(&it, npk));
-    HC_CUDA(sc.get(&pr, b->n));
-    HC_CUDA(sc.get(&tl, b->n));
-    HC_CUDA(sc.get(&z, b->n));
-    HC_CUDA(cudaMemcpyAsync(po, b->peak_off, sizeof(uint64_t) * (b->n + 1), cudaMemcpyHostToDevice, s));
-    if (npk) {
-        HC_CUDA(cudaMemcpyAsync(mz, b->mz, sizeof(float) * npk, cudaMemcpyHostToDevice, s));
-        HC_CUDA(cudaMemcpyAsync(it, b->intensity, sizeof(float) * npk, cudaMemcpyHostToDevice, s));
-    }
-    HC_CUDA(cudaMemcpyAsync(pr, b->prec_mz, sizeof(double) * b->n, cudaMemcpyHostToDevice, s));
-    HC_CUDA(cudaMemcpyAsync(tl, b->prec_tol_da, sizeof(double) * b->n, cudaMemcpyHostToDevice, s));
-    HC_CUDA(cudaMemcpyAsync(z, b->charge, sizeof(uint8_t) * b->n, cudaMemcpyHostToDevice, s));
+    HC_CUDA(al.get(&po, b->n + 1));
+    HC_CUDA(al.get(&mz, npk));
+    HC_CUDA(al.get(&it, npk));
+    HC_CUDA(al.get(&pr, b->n));
+    HC_CUDA(al.get(&tl, b->n));
+    HC_CUDA(al.get(&z, b->n));
     d = DevBatch{po, mz, it, pr, z, tl};
     return HICOPS_OK;
 }
 
-constexpr uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
-
-// alloc_workspace's allocators over caller memory.  Carve hands out
-// consecutive 256-byte aligned pieces of one buffer and fails when they would
-// not fit; Tally only adds up the bytes Carve would hand out.
-struct Carve {
-    unsigned char* base;
-    uint64_t cap, used;
-    template <class T>
-    cudaError_t get(T** p, uint64_t n) {
-        const uint64_t bytes = align256(sizeof(T) * (n ? n : 1));
-        if (used + bytes > cap) return cudaErrorMemoryAllocation;
-        *p = reinterpret_cast<T*>(base + used);
-        used += bytes;
-        return cudaSuccess;
-    }
-};
-
-struct Tally {
-    uint64_t used = 0;
-    template <class T>
-    cudaError_t get(T** p, uint64_t n) {
-        *p = nullptr;
-        used += align256(sizeof(T) * (n ? n : 1));
-        return cudaSuccess;
-    }
-};
+hicops_status copy_inputs(const hicops_batch* b, const DevBatch& d, cudaStream_t s) {
+    if (b->on_device) return HICOPS_OK;
+    auto copy = [&](const void* to, const void* from, uint64_t bytes) {
+        return bytes ? cudaMemcpyAsync(const_cast<void*>(to), from, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
+    };
+    const uint64_t npk = b->peak_off[b->n];
+    HC_CUDA(copy(d.peak_off, b->peak_off, sizeof(uint64_t) * (b->n + 1)));
+    HC_CUDA(copy(d.mz, b->mz, sizeof(float) * npk));
+    HC_CUDA(copy(d.inten, b->intensity, sizeof(float) * npk));
+    HC_CUDA(copy(d.prec, b->prec_mz, sizeof(double) * b->n));
+    HC_CUDA(copy(d.tol, b->prec_tol_da, sizeof(double) * b->n));
+    HC_CUDA(copy(d.z, b->charge, sizeof(uint8_t) * b->n));
+    return HICOPS_OK;
+}
 
 // The workspace of a search in caller memory: alloc_workspace's pieces
 // without the PSM rows (the caller always gives those), then a histogram and
@@ -488,18 +497,35 @@ extern "C" hicops_status hicops_search(hicops_index* idx, const hicops_batch* b,
     const uint32_t k = p.top_k;
     cudaStream_t s = (cudaStream_t)b->cuda_stream;
     {
-        Scratch sc(s);
+        // one piece of the pool a call, carved into inputs, workspace and outputs
+        const uint32_t max_seg = max_segments(idx->dev.cfg, n);
+        const bool own_hist = !b->on_device || !out_hist, own_ns = !b->on_device || !out_nscored;
         DevBatch d;
-        st = stage_inputs(b, sc, d);
-        if (st != HICOPS_OK) return st;
         Workspace w;
-        st = alloc_workspace(sc, p, n, max_segments(idx->dev.cfg, n), !b->on_device, w);
+        auto pieces = [&](auto& al) -> hicops_status {
+            hicops_status e = place_inputs(al, b, d);
+            if (e != HICOPS_OK) return e;
+            e = alloc_workspace(al, p, n, max_seg, false, w);
+            if (e != HICOPS_OK) return e;
+            if (!b->on_device) HC_CUDA(al.get(&w.psm, (uint64_t)n * k));
+            if (own_hist) HC_CUDA(al.get(&w.hist, (uint64_t)n * kHistBins));
+            if (own_ns) HC_CUDA(al.get(&w.ns, n));
+            return HICOPS_OK;
+        };
+        Tally need;
+        st = pieces(need);
+        if (st != HICOPS_OK) return st;
+        Scratch sc(s, (cudaMemPool_t)idx->dev.pool);
+        unsigned char* base;
+        HC_CUDA(sc.get(&base, need.used));
+        Carve carve{base, need.used, 0};
+        st = pieces(carve);
+        if (st != HICOPS_OK) return st;
+        st = copy_inputs(b, d, s);
         if (st != HICOPS_OK) return st;
         hicops_psm* d_psm = b->on_device ? out_psm : w.psm;
-        uint32_t* d_hist = b->on_device && out_hist ? out_hist : nullptr;
-        uint32_t* d_ns = b->on_device && out_nscored ? out_nscored : nullptr;
-        if (!d_hist) { if (!w.hist) HC_CUDA(sc.get(&w.hist, (uint64_t)n * kHistBins)); d_hist = w.hist; }
-        if (!d_ns) { if (!w.ns) HC_CUDA(sc.get(&w.ns, n)); d_ns = w.ns; }
+        uint32_t* d_hist = own_hist ? w.hist : out_hist;
+        uint32_t* d_ns = own_ns ? w.ns : out_nscored;
         st = enqueue_search(idx, d, n, w, idx->dev.cfg, d_psm, d_hist, d_ns, s, true);
         if (st != HICOPS_OK) return st;
         if (!b->on_device) {
@@ -523,9 +549,10 @@ extern "C" hicops_status hicops_search_work(hicops_index* idx, const hicops_batc
     cudaStream_t s = (cudaStream_t)b->cuda_stream;
     const hicops_params& p = idx->p;
     {
-        Scratch sc(s);
+        Scratch sc(s, (cudaMemPool_t)idx->dev.pool);
         DevBatch d;
-        st = stage_inputs(b, sc, d);
+        st = place_inputs(sc, b, d);
+        if (st == HICOPS_OK) st = copy_inputs(b, d, s);
         if (st != HICOPS_OK) return st;
         uint32_t *qbin, *qiq, *qn, *lo, *hi;
         uint64_t* hits;
