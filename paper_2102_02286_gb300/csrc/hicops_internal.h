@@ -2,6 +2,8 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -85,6 +87,26 @@ struct DeviceIndex {
     hicops_search_config cfg = {0, 0, 0, 0};
 };
 
+// base (unmodified, deduplicated) peptides, in sequence-byte order
+struct BaseSet {
+    std::string residues;             // concatenated letters
+    std::vector<uint64_t> base_off;   // [B + 1]
+};
+
+// A vector whose resize leaves new elements unset, so that the threads that
+// fill it are the first to touch its pages.
+template <class T>
+struct RawAllocator : std::allocator<T> {
+    template <class U>
+    struct rebind { using other = RawAllocator<U>; };
+    template <class U>
+    void construct(U* p) { ::new ((void*)p) U; }
+    template <class U, class... A>
+    void construct(U* p, A&&... a) { ::new ((void*)p) U(std::forward<A>(a)...); }
+};
+template <class T>
+using RawVector = std::vector<T, RawAllocator<T>>;
+
 // Counts every kernel launch of the library.
 void count_launches(uint64_t n);
 
@@ -101,13 +123,12 @@ struct hicops_index {
     std::vector<double> var_delta;
     std::vector<uint32_t> var_max;
 
-    // base (unmodified, deduplicated) peptides, in sequence-byte order
-    std::string residues;          // concatenated letters
-    std::vector<uint64_t> base_off;   // [B + 1]
+    // shared by a database and its parts, not changed once it has any
+    std::shared_ptr<hicops::BaseSet> bases = std::make_shared<hicops::BaseSet>();
     // database entries in pid order
-    std::vector<double> mass;
-    std::vector<uint32_t> base;
-    std::vector<uint64_t> mask;
+    hicops::RawVector<double> mass;
+    hicops::RawVector<uint32_t> base;
+    hicops::RawVector<uint64_t> mask;
 
     // a shard of a database holds its entries pid_base, pid_base + pid_stride, ...:
     // global pid = local pid * pid_stride + pid_base (1 and 0 for a whole database)

@@ -267,20 +267,20 @@ extern "C" hicops_status hicops_digest(const hicops_proteins* prot, const hicops
         bases.resize(w);
     }
     const size_t NB = bases.size();
-    idx->base_off.resize(NB + 1);
-    idx->base_off[0] = 0;
-    for (size_t i = 0; i < NB; ++i) idx->base_off[i + 1] = idx->base_off[i] + bases[i].len;
-    idx->residues.resize(idx->base_off[NB]);
+    idx->bases->base_off.resize(NB + 1);
+    idx->bases->base_off[0] = 0;
+    for (size_t i = 0; i < NB; ++i) idx->bases->base_off[i + 1] = idx->bases->base_off[i] + bases[i].len;
+    idx->bases->residues.resize(idx->bases->base_off[NB]);
     parallel_for(NB, [&](size_t i, unsigned) {
-        memcpy(&idx->residues[idx->base_off[i]], seq + bases[i].pos, bases[i].len);
+        memcpy(&idx->bases->residues[idx->bases->base_off[i]], seq + bases[i].pos, bases[i].len);
     });
 
     // 3. variants: every subset of modifiable positions within the per-rule
     //    caps (and the global cap), masses summed left to right
     std::vector<std::vector<Entry>> ent(T);
     parallel_for(NB, [&](size_t bi, unsigned t) {
-        const char* s = &idx->residues[idx->base_off[bi]];
-        const uint32_t L = (uint32_t)(idx->base_off[bi + 1] - idx->base_off[bi]);
+        const char* s = &idx->bases->residues[idx->bases->base_off[bi]];
+        const uint32_t L = (uint32_t)(idx->bases->base_off[bi + 1] - idx->bases->base_off[bi]);
         // sites in position order, with their rule
         uint32_t site_pos[kMaxLen];
         int site_rule[kMaxLen];
@@ -370,6 +370,9 @@ namespace {
 
 bool is_part(const hicops_index* idx) { return idx->pid_stride != 1 || !idx->pid_map.empty(); }
 
+// entries from which on the threads that take a part's pay for their start
+constexpr size_t kParallelTake = 1u << 17;
+
 // The part of a whole database holding global pids g(0) < g(1) < ... < g(n-1),
 // as a host-only index (hicops_index_upload builds its device part).
 template <class Global>
@@ -383,17 +386,18 @@ hicops_index* make_part(const hicops_index* full, size_t n, Global g) {
     idx->n_var = full->n_var;
     idx->var_delta = full->var_delta;
     idx->var_max = full->var_max;
-    idx->residues = full->residues;
-    idx->base_off = full->base_off;
+    idx->bases = full->bases;
     idx->mass.resize(n);
     idx->base.resize(n);
     idx->mask.resize(n);
-    for (size_t i = 0; i < n; ++i) {
+    auto take = [&](size_t i, unsigned) {
         const size_t k = g(i);
         idx->mass[i] = full->mass[k];
         idx->base[i] = full->base[k];
         idx->mask[i] = full->mask[k];
-    }
+    };
+    if (n < kParallelTake) for (size_t i = 0; i < n; ++i) take(i, 0);
+    else parallel_for(n, take);
     idx->n_bins = full->n_bins;
     idx->s_max = full->s_max;
     idx->stats = hicops_index_stats{};
@@ -460,7 +464,7 @@ extern "C" hicops_status hicops_partition_lbe(const hicops_index* full, uint32_t
         return HICOPS_EINVAL;
     }
     const size_t P = full->mass.size();
-    const size_t NB = full->base_off.size() - 1;
+    const size_t NB = full->bases->base_off.size() - 1;
     std::vector<uint32_t> first(NB, UINT32_MAX);   // each cluster's smallest pid
     for (size_t pid = P; pid-- > 0;) first[full->base[pid]] = (uint32_t)pid;
     struct Key {
@@ -469,7 +473,7 @@ extern "C" hicops_status hicops_partition_lbe(const hicops_index* full, uint32_t
     std::vector<Key> keys(P);
     parallel_for(P, [&](size_t pid, unsigned) {
         const uint32_t b = full->base[pid];
-        const uint32_t L = (uint32_t)(full->base_off[b + 1] - full->base_off[b]);
+        const uint32_t L = (uint32_t)(full->bases->base_off[b + 1] - full->bases->base_off[b]);
         const uint64_t m = full->mask[pid];
         uint32_t a = 2 * L;
         if (m) a = (uint32_t)__builtin_ctzll(m) + (L - 1 - (63 - (uint32_t)__builtin_clzll(m)));
@@ -504,10 +508,10 @@ extern "C" hicops_status hicops_peptide(const hicops_index* idx, uint32_t pid, c
     }
     if (pid >= idx->mass.size()) { set_error("pid out of range"); return HICOPS_EINVAL; }
     const uint32_t b = idx->base[pid];
-    const uint64_t a = idx->base_off[b], e = idx->base_off[b + 1];
+    const uint64_t a = idx->bases->base_off[b], e = idx->bases->base_off[b + 1];
     if (seq && cap) {
         const uint64_t n = std::min<uint64_t>(e - a, cap - 1);
-        memcpy(seq, &idx->residues[a], n);
+        memcpy(seq, &idx->bases->residues[a], n);
         seq[n] = 0;
     }
     if (mass) *mass = idx->mass[pid];
@@ -538,10 +542,10 @@ struct FileOut {
     }
     template <class T>
     void pod(const T& v) { raw(&v, sizeof(T)); }
-    template <class T>
-    void vec(const std::vector<T>& v) {
+    template <class V>
+    void vec(const V& v) {
         pod<uint64_t>(v.size());
-        raw(v.data(), v.size() * sizeof(T));
+        raw(v.data(), v.size() * sizeof(v[0]));
     }
 };
 
@@ -555,13 +559,13 @@ struct FileIn {
     }
     template <class T>
     void pod(T& v) { raw(&v, sizeof(T)); }
-    template <class T>
-    void vec(std::vector<T>& v) {
+    template <class V>
+    void vec(V& v) {
         uint64_t n = 0;
         pod(n);
-        if (!ok || n > left / sizeof(T)) { ok = false; return; }   // never allocate past the file
+        if (!ok || n > left / sizeof(v[0])) { ok = false; return; }   // never allocate past the file
         v.resize(n);
-        raw(v.data(), n * sizeof(T));
+        raw(v.data(), n * sizeof(v[0]));
     }
 };
 
@@ -582,9 +586,9 @@ extern "C" hicops_status hicops_index_save(const hicops_index* idx, const char* 
     o.pod(idx->n_var);
     o.vec(idx->var_delta);
     o.vec(idx->var_max);
-    o.pod<uint64_t>(idx->residues.size());
-    o.raw(idx->residues.data(), idx->residues.size());
-    o.vec(idx->base_off);
+    o.pod<uint64_t>(idx->bases->residues.size());
+    o.raw(idx->bases->residues.data(), idx->bases->residues.size());
+    o.vec(idx->bases->base_off);
     o.vec(idx->mass);
     o.vec(idx->base);
     o.vec(idx->mask);
@@ -631,12 +635,12 @@ extern "C" hicops_status hicops_index_load(const char* path, hicops_index** out)
         uint64_t nres = 0;
         in.pod(nres);
         if (in.ok && nres <= in.left) {
-            idx->residues.resize(nres);
-            in.raw(&idx->residues[0], nres);
+            idx->bases->residues.resize(nres);
+            in.raw(&idx->bases->residues[0], nres);
         } else {
             in.ok = false;
         }
-        in.vec(idx->base_off);
+        in.vec(idx->bases->base_off);
         in.vec(idx->mass);
         in.vec(idx->base);
         in.vec(idx->mask);
@@ -655,21 +659,21 @@ extern "C" hicops_status hicops_index_load(const char* path, hicops_index** out)
     // consistency of what was read: sizes, ranges and orders
     hicops_index& x = *idx;
     const size_t P = x.mass.size();
-    bool good = x.n_var == x.var_delta.size() && x.n_var == x.var_max.size() && !x.base_off.empty() &&
-                x.base_off.front() == 0 && x.base_off.back() == x.residues.size() && x.base.size() == P &&
+    bool good = x.n_var == x.var_delta.size() && x.n_var == x.var_max.size() && !x.bases->base_off.empty() &&
+                x.bases->base_off.front() == 0 && x.bases->base_off.back() == x.bases->residues.size() && x.base.size() == P &&
                 x.mask.size() == P && x.pid_stride >= 1 && (x.pid_map.empty() || x.pid_map.size() == P) &&
                 P < (1ull << 31);
-    for (size_t i = 1; good && i < x.base_off.size(); ++i) good = x.base_off[i] >= x.base_off[i - 1];
+    for (size_t i = 1; good && i < x.bases->base_off.size(); ++i) good = x.bases->base_off[i] >= x.bases->base_off[i - 1];
     for (size_t i = 0; good && i < 128; ++i) good = x.var_type[i] < (int)x.n_var;
     for (size_t i = 0; good && i < P; ++i) {
-        good = x.base[i] + 1 < x.base_off.size() &&
-               x.base_off[x.base[i] + 1] - x.base_off[x.base[i]] <= kMaxLen && (i == 0 || x.mass[i] >= x.mass[i - 1]);
+        good = x.base[i] + 1 < x.bases->base_off.size() &&
+               x.bases->base_off[x.base[i] + 1] - x.bases->base_off[x.base[i]] <= kMaxLen && (i == 0 || x.mass[i] >= x.mass[i - 1]);
     }
     for (size_t i = 1; good && i < x.pid_map.size(); ++i) good = x.pid_map[i] > x.pid_map[i - 1];
     // every residue byte indexes the 128-entry mass tables on the device and
     // must be a letter with a mass (digestion keeps no other)
-    for (size_t i = 0; good && i < x.residues.size(); ++i) {
-        const unsigned char c = (unsigned char)x.residues[i];
+    for (size_t i = 0; good && i < x.bases->residues.size(); ++i) {
+        const unsigned char c = (unsigned char)x.bases->residues[i];
         good = c < 128 && x.mres[c] > 0.0 && std::isfinite(x.mres[c]) && std::isfinite(x.mmod[c]);
     }
     if (!good) { set_error("%s: inconsistent index contents", path); return HICOPS_EINVAL; }

@@ -505,7 +505,7 @@ hicops_status upload_index(hicops_index* idx) {
     HC_CUDA(cudaGetDevice(&d.device));
     const hicops_params& p = idx->p;
     const uint64_t P = idx->mass.size();
-    const uint64_t B = idx->base_off.size() - 1;
+    const uint64_t B = idx->bases->base_off.size() - 1;
     TmpFree tf;   // destroyed after the stream guard has synchronised
     cudaStream_t s;
     HC_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
@@ -561,14 +561,14 @@ hicops_status upload_index(hicops_index* idx) {
     HC_CUDA(dalloc(&d_base, P, tf.ptrs));
     HC_CUDA(dalloc(&d_mask, P, tf.ptrs));
     HC_CUDA(dalloc(&d_boff, B + 1, tf.ptrs));
-    HC_CUDA(dalloc(&d_res, idx->residues.size() + 1, tf.ptrs));
+    HC_CUDA(dalloc(&d_res, idx->bases->residues.size() + 1, tf.ptrs));
     HC_CUDA(dalloc(&d_mres, 128, tf.ptrs));
     HC_CUDA(dalloc(&d_mmod, 128, tf.ptrs));
     HC_CUDA(dalloc(&d_fix, 256, tf.ptrs));
     HC_CUDA(cudaMemcpyAsync(d_base, idx->base.data(), sizeof(uint32_t) * P, cudaMemcpyHostToDevice, s));
     HC_CUDA(cudaMemcpyAsync(d_mask, idx->mask.data(), sizeof(uint64_t) * P, cudaMemcpyHostToDevice, s));
-    HC_CUDA(cudaMemcpyAsync(d_boff, idx->base_off.data(), sizeof(uint64_t) * (B + 1), cudaMemcpyHostToDevice, s));
-    HC_CUDA(cudaMemcpyAsync(d_res, idx->residues.data(), idx->residues.size(), cudaMemcpyHostToDevice, s));
+    HC_CUDA(cudaMemcpyAsync(d_boff, idx->bases->base_off.data(), sizeof(uint64_t) * (B + 1), cudaMemcpyHostToDevice, s));
+    HC_CUDA(cudaMemcpyAsync(d_res, idx->bases->residues.data(), idx->bases->residues.size(), cudaMemcpyHostToDevice, s));
     HC_CUDA(cudaMemcpyAsync(d_mres, idx->mres, sizeof(double) * 128, cudaMemcpyHostToDevice, s));
     HC_CUDA(cudaMemcpyAsync(d_mmod, idx->mmod, sizeof(double) * 128, cudaMemcpyHostToDevice, s));
 
