@@ -1048,6 +1048,8 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
             st.c = st.e;
             st.e = min(st.e + st.m, col_end);
             take_unit();
+            // (a warp's next repeats may go into another's share of the table)
+            if (st.c < col_end && sh.no_room >= 0) __syncthreads();
         }
         if (tid == 0 && !st.taken)   // an empty segment (a window split into more units than it has peptides)
             set_unit((uint64_t)gridDim.x + atomicAdd(a.work, 1ull));
