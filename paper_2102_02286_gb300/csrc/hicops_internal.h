@@ -43,7 +43,7 @@ struct BinInfo {
     uint32_t group;   // the bucket's first 4-entry group
     int32_t row;      // its skip-table row (-1: empty bucket)
     int32_t hot;      // its bitmaps' row (-1: not hot)
-    uint32_t flags;   // hot: bit 0 has b entries, bit 1 has y entries
+    uint32_t flags;   // its 4-entry groups << 2; hot: bit 0 has b entries, bit 1 has y entries
 };
 
 // Thread-local error message (host.cpp).

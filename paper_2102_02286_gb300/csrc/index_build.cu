@@ -417,7 +417,8 @@ __global__ void bin_info_kernel(const uint64_t* __restrict__ off, const int32_t*
     const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nbins) return;
     const int32_t h = hot_id[b];
-    out[b] = BinInfo{(uint32_t)(off[b] >> 2), row[b], h, h >= 0 ? hflags[h] : 0u};
+    const uint32_t groups = (uint32_t)((off[b + 1] - off[b]) >> 2);   // < 2^30 (bucket limit)
+    out[b] = BinInfo{(uint32_t)(off[b] >> 2), row[b], h, groups << 2 | (h >= 0 ? hflags[h] : 0u)};
 }
 
 template <class T>

@@ -95,37 +95,43 @@ struct Tally {
     }
 };
 
-// Device scratch of one search of up to cap_n spectra.
+// Device scratch of one search of up to cap_n spectra in units of at most
+// max_units, at most max_seg of them a spectrum.
 struct Workspace {
     uint32_t cap_n = 0, max_seg = 0;
-    uint32_t *qbin = nullptr, *qiq = nullptr, *qn = nullptr, *lo = nullptr, *hi = nullptr, *nseg = nullptr;
-    uint64_t *seg_off = nullptr, *stmp = nullptr;
+    uint64_t max_units = 0;
+    uint32_t *qbin = nullptr, *qiq = nullptr, *qn = nullptr, *lo = nullptr, *hi = nullptr, *cost = nullptr;
+    uint64_t* seg_off = nullptr;
     UnitTop* utop = nullptr;
     unsigned long long* work = nullptr;
-    uint4* unit = nullptr;       // [cap_n * max_seg] units in the order they are taken
-    uint32_t* ocnt = nullptr;    // [2 * kOrderBuckets] bucket counts and starts
+    uint4* unit = nullptr;       // [max_units] units in the order they are taken
     hicops_psm* psm = nullptr;   // used when the caller gives no device output
     uint32_t* hist = nullptr;
     uint32_t* ns = nullptr;
 };
 
+// How many units a batch can have (PlanArgs).
+struct UnitLimit {
+    uint32_t max_seg, split;
+    uint64_t units;
+};
+
 template <class A>
-hicops_status alloc_workspace(A& al, const hicops_params& p, uint32_t cap_n, uint32_t max_seg, bool outputs,
+hicops_status alloc_workspace(A& al, const hicops_params& p, uint32_t cap_n, const UnitLimit& lim, bool outputs,
                               Workspace& w) {
     w.cap_n = cap_n;
-    w.max_seg = max_seg;
+    w.max_seg = lim.max_seg;
+    w.max_units = lim.units;
     HC_CUDA(al.get(&w.qbin, (uint64_t)cap_n * query_bins_cap(p)));
     HC_CUDA(al.get(&w.qiq, (uint64_t)cap_n * query_bins_cap(p)));
     HC_CUDA(al.get(&w.qn, cap_n));
     HC_CUDA(al.get(&w.lo, cap_n));
     HC_CUDA(al.get(&w.hi, cap_n));
-    HC_CUDA(al.get(&w.nseg, cap_n));
+    HC_CUDA(al.get(&w.cost, cap_n));
     HC_CUDA(al.get(&w.seg_off, (uint64_t)cap_n + 1));
-    HC_CUDA(al.get(&w.stmp, scan_tmp_words(cap_n)));
-    HC_CUDA(al.get(&w.utop, (uint64_t)cap_n * max_seg * p.top_k));
+    HC_CUDA(al.get(&w.utop, lim.units * p.top_k));
     HC_CUDA(al.get(&w.work, 1));
-    HC_CUDA(al.get(&w.unit, (uint64_t)cap_n * max_seg));
-    HC_CUDA(al.get(&w.ocnt, 2 * kOrderBuckets));
+    HC_CUDA(al.get(&w.unit, lim.units));
     if (outputs) {
         HC_CUDA(al.get(&w.psm, (uint64_t)cap_n * p.top_k));
         HC_CUDA(al.get(&w.hist, (uint64_t)cap_n * kHistBins));
@@ -169,14 +175,13 @@ hicops_search_config resolved(const hicops_search_config& c, uint32_t query_bins
     return r;
 }
 
-// Units per spectrum cap: large when the batch cannot fill the GPU.
-uint32_t max_segments(const hicops_search_config& c, uint32_t n) {
-    if (c.seg_pids) return kMaxSegs;
-    const uint32_t want = 8u * (uint32_t)g_sm_count.load(std::memory_order_relaxed);
-    uint32_t m = (want + n - 1) / (n ? n : 1);
-    if (m < 1) m = 1;
-    if (m > (uint32_t)kMaxSegs) m = kMaxSegs;
-    return m;
+// kSplitPerSm pieces an SM to even out the CTAs' shares, by the batch's cost.
+constexpr uint32_t kSplitPerSm = 8;
+
+UnitLimit unit_limit(const hicops_search_config& c, uint64_t n, uint32_t max_seg = kMaxSegs) {
+    const uint32_t split = kSplitPerSm * (uint32_t)g_sm_count.load(std::memory_order_relaxed);
+    const uint64_t most = n * max_seg;
+    return UnitLimit{max_seg, split, c.seg_pids ? most : std::min(most, n + split)};
 }
 
 // The parts of a CTA's shared memory when ctas CTAs share an SM.
@@ -264,8 +269,8 @@ inline void mark(hicops_index* idx, int i, cudaStream_t s, bool on) {
 // query_bins_cap(p) words per spectrum.  Histograms and counts, where given,
 // are set to zero on the way.
 hicops_status prepare_queries(hicops_index* idx, const DevBatch& d, uint32_t n, uint32_t* qbin, uint32_t* qiq,
-                              uint32_t* qn, uint32_t* lo, uint32_t* hi, uint32_t* hist, uint32_t* ns,
-                              cudaStream_t s) {
+                              uint32_t* qn, uint32_t* lo, uint32_t* hi, uint32_t* cost, uint32_t* hist,
+                              uint32_t* ns, cudaStream_t s) {
     const hicops_params& p = idx->p;
     const uint32_t stride = query_bins_cap(p);
     auto not_below = [](double x) {      // the least float >= x
@@ -279,7 +284,9 @@ hicops_status prepare_queries(hicops_index* idx, const DevBatch& d, uint32_t n, 
     PrepArgs pa{d.peak_off, d.mz, d.inten, d.prec, d.z, d.tol, n, p.top_n_peaks, stride, p.bin_width_da,
                 not_below(p.frag_mz_min), not_below(p.frag_mz_max),
                 finite ? (uint64_t)std::ldexp(f, 64) : 0ull, finite ? e : 4096, p.intensity_scale,
-                idx->dev.mass, idx->mass.size(), qbin, qiq, qn, lo, hi, hist, ns};
+                idx->dev.mass, idx->mass.size(), qbin, qiq, qn, lo, hi, idx->dev.bins,
+                idx->n_bins, p.tol_bins, (float)(4.0 / std::max<double>(1.0, (double)idx->mass.size())),
+                p.min_shared > 2 ? p.min_shared - 2 : 0, cost, hist, ns};
     const uint32_t big = std::min(n, kPrepBigBlocks);
     prep_kernel<<<big + (n + kPrepWarps - 1) / kPrepWarps, kPrepThreads, 0, s>>>(pa, big);
     count_launches(1);
@@ -303,35 +310,21 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     const hicops_search_config cfg = resolved(cfg_in, query_bins_cap(idx->p));
     const uint32_t k = p.top_k;
     mark(idx, 0, s, timing_marks);
-    hicops_status st = prepare_queries(idx, d, n, w.qbin, w.qiq, w.qn, w.lo, w.hi, d_hist, d_ns, s);
+    hicops_status st = prepare_queries(idx, d, n, w.qbin, w.qiq, w.qn, w.lo, w.hi, w.cost, d_hist, d_ns, s);
     if (st != HICOPS_OK) return st;
     mark(idx, 1, s, timing_marks);
-    const uint32_t max_seg = w.max_seg;
-    const uint32_t seg_pids = cfg.seg_pids ? cfg.seg_pids : (uint32_t)kMinSegPids;
-    // longest units first; a small batch has too few units per CTA for the
-    // order to matter, and is planned by one kernel
-    if (n >= kOrderMinSpectra) {
-        plan_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, n, max_seg, seg_pids, w.nseg, w.work);
-        count_launches(1);
-        HC_CUDA(cudaGetLastError());
-        HC_CUDA(exclusive_scan<uint32_t>(w.nseg, n, w.seg_off, w.seg_off + n, w.stmp, s));
-        HC_CUDA(cudaMemsetAsync(w.ocnt, 0, sizeof(uint32_t) * kOrderBuckets, s));
-        order_count_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, w.seg_off, n, w.ocnt);
-        order_scan_kernel<<<1, 32, 0, s>>>(w.ocnt);
-        order_scatter_kernel<<<(n + 255) / 256, 256, 0, s>>>(w.qn, w.lo, w.hi, w.seg_off, n, w.ocnt + kOrderBuckets,
-                                                             w.unit);
-        count_launches(3);
-    } else {
-        plan_small_kernel<<<1, kPlanThreads, 0, s>>>(w.qn, w.lo, w.hi, n, max_seg, seg_pids, w.seg_off, w.unit, w.work);
-        count_launches(1);
-    }
+    const uint32_t split = unit_limit(cfg, n).split;
+    const PlanArgs plan{w.lo, w.hi, w.cost, n, w.max_seg, cfg.seg_pids, split,
+                        split / kSplitPerSm * (uint32_t)search_min_ctas((int)cfg.threads), w.seg_off, w.unit, w.work};
+    plan_kernel<<<1, n <= kPlanFew ? kPlanFew : kPlanThreads, 0, s>>>(plan);
+    count_launches(1);
     HC_CUDA(cudaGetLastError());
     SearchArgs sa{w.qbin, w.qiq, w.qn, n, query_bins_cap(p), w.unit, w.seg_off + n, di.bins, di.entry, di.skip,
                   di.skip_stride, di.hot_b, di.hot_y, di.hot_words, di.fwd_off, reinterpret_cast<const uint4*>(di.fwd), di.lf, di.ls,
                   (uint32_t)idx->s_max, p.min_shared, k, cfg.chunk_entries < 16 ? cfg.chunk_entries * 1024u : 0xffffffffu, w.utop, d_hist, d_ns, w.work,
                   SearchLayout{}};
     mark(idx, 2, s, timing_marks);
-    st = launch_search(sa, cfg, (uint64_t)n * max_seg, s);
+    st = launch_search(sa, cfg, std::min(w.max_units, (uint64_t)n * w.max_seg), s);
     if (st != HICOPS_OK) return st;
     mark(idx, 3, s, timing_marks);
     MergeArgs ma{w.seg_off, w.utop, nullptr, nullptr, 0, 0, nullptr, nullptr, d_hist, n, k, d_psm,
@@ -401,8 +394,8 @@ hicops_status copy_inputs(const hicops_batch* b, const DevBatch& d, cudaStream_t
 // without the PSM rows (the caller always gives those), then a histogram and
 // candidate-count block for callers that pass none.
 template <class A>
-hicops_status scratch_workspace(A& al, const hicops_params& p, uint32_t n, uint32_t max_seg, Workspace& w) {
-    hicops_status st = alloc_workspace(al, p, n, max_seg, false, w);
+hicops_status scratch_workspace(A& al, const hicops_params& p, uint32_t n, const UnitLimit& lim, Workspace& w) {
+    hicops_status st = alloc_workspace(al, p, n, lim, false, w);
     if (st != HICOPS_OK) return st;
     HC_CUDA(al.get(&w.hist, (uint64_t)n * kHistBins));
     HC_CUDA(al.get(&w.ns, n));
@@ -415,7 +408,7 @@ uint64_t scratch_bytes(const hicops_index* idx, const hicops_search_config& cfg,
     if (!n) n = 1;
     Tally t;
     Workspace w;
-    scratch_workspace(t, idx->p, n, max_segments(cfg, n), w);
+    scratch_workspace(t, idx->p, n, unit_limit(cfg, n), w);
     return t.used;
 }
 
@@ -442,7 +435,7 @@ hicops_status search_in_scratch(hicops_index* idx, const hicops_batch* b, const 
     }
     Carve cv{static_cast<unsigned char*>(scratch), bytes, 0};
     Workspace w;
-    st = scratch_workspace(cv, idx->p, n, max_segments(cfg, n), w);
+    st = scratch_workspace(cv, idx->p, n, unit_limit(cfg, n), w);
     if (st != HICOPS_OK) return st;
     const DevBatch d{b->peak_off, b->mz, b->intensity, b->prec_mz, b->charge, b->prec_tol_da};
     return enqueue_search(idx, d, n, w, cfg, out_psm, out_hist ? out_hist : w.hist, out_nscored ? out_nscored : w.ns,
@@ -498,14 +491,14 @@ extern "C" hicops_status hicops_search(hicops_index* idx, const hicops_batch* b,
     cudaStream_t s = (cudaStream_t)b->cuda_stream;
     {
         // one piece of the pool a call, carved into inputs, workspace and outputs
-        const uint32_t max_seg = max_segments(idx->dev.cfg, n);
+        const UnitLimit lim = unit_limit(idx->dev.cfg, n);
         const bool own_hist = !b->on_device || !out_hist, own_ns = !b->on_device || !out_nscored;
         DevBatch d;
         Workspace w;
         auto pieces = [&](auto& al) -> hicops_status {
             hicops_status e = place_inputs(al, b, d);
             if (e != HICOPS_OK) return e;
-            e = alloc_workspace(al, p, n, max_seg, false, w);
+            e = alloc_workspace(al, p, n, lim, false, w);
             if (e != HICOPS_OK) return e;
             if (!b->on_device) HC_CUDA(al.get(&w.psm, (uint64_t)n * k));
             if (own_hist) HC_CUDA(al.get(&w.hist, (uint64_t)n * kHistBins));
@@ -562,7 +555,7 @@ extern "C" hicops_status hicops_search_work(hicops_index* idx, const hicops_batc
         HC_CUDA(sc.get(&lo, n));
         HC_CUDA(sc.get(&hi, n));
         HC_CUDA(sc.get(&hits, n));
-        st = prepare_queries(idx, d, n, qbin, qiq, qn, lo, hi, nullptr, nullptr, s);
+        st = prepare_queries(idx, d, n, qbin, qiq, qn, lo, hi, nullptr, nullptr, nullptr, s);
         if (st != HICOPS_OK) return st;
         work_kernel<<<n, 256, 0, s>>>(qbin, qn, lo, hi, query_bins_cap(p), idx->dev.off, idx->dev.entry, hits);
         count_launches(1);
@@ -599,12 +592,14 @@ extern "C" hicops_status hicops_plan_create(hicops_index* idx, uint32_t max_spec
     pl->idx = idx;
     pl->cfg = cfg ? *cfg : idx->dev.cfg;
     st = check_config(pl->cfg);
-    // per-unit top-k lists: up to kMaxSegs units per spectrum within 1 GiB
+    // with pieces of a given size, per-unit top-k lists of up to kMaxSegs units per spectrum within 1 GiB
     const uint64_t per_seg = (uint64_t)max_spectra * idx->p.top_k * sizeof(UnitTop);
     uint64_t segs = (1ull << 30) / per_seg;
-    if (segs > (uint64_t)kMaxSegs) segs = kMaxSegs;
+    if (segs > (uint64_t)kMaxSegs || !pl->cfg.seg_pids) segs = kMaxSegs;
     if (segs < 1) segs = 1;
-    if (st == HICOPS_OK) st = alloc_workspace(pl->arena, idx->p, max_spectra, (uint32_t)segs, true, pl->ws);
+    if (st == HICOPS_OK)
+        st = alloc_workspace(pl->arena, idx->p, max_spectra, unit_limit(pl->cfg, max_spectra, (uint32_t)segs), true,
+                             pl->ws);
     if (st != HICOPS_OK) { delete pl; return st; }
     *out = pl;
     return HICOPS_OK;
@@ -623,9 +618,7 @@ extern "C" hicops_status hicops_plan_search(hicops_plan* pl, const hicops_batch*
     uint32_t* d_hist = out_hist ? out_hist : pl->ws.hist;
     uint32_t* d_ns = out_nscored ? out_nscored : pl->ws.ns;
     DevBatch d{b->peak_off, b->mz, b->intensity, b->prec_mz, b->charge, b->prec_tol_da};
-    Workspace w = pl->ws;
-    const uint32_t want = max_segments(pl->cfg, n);
-    if (want < w.max_seg) w.max_seg = want;
+    const Workspace& w = pl->ws;
     if (!use_graph || s == nullptr)
         return enqueue_search(pl->idx, d, n, w, pl->cfg, out_psm, d_hist, d_ns, s, true);
     const bool same = pl->exec && memcmp(&pl->key_batch, b, sizeof(hicops_batch)) == 0 &&
@@ -757,17 +750,14 @@ constexpr uint32_t kNoAllocSegs = 16;      // work units per spectrum at most
 constexpr int kNoAllocDevices = 64;        // device ordinals served
 
 // Workspace bytes for cap spectra at the largest top_n_peaks and top_k, in
-// alloc_workspace's order (each piece 256-byte aligned), plus room for the
-// scan's temporary words.
+// alloc_workspace's order (each piece 256-byte aligned).
 constexpr uint64_t noalloc_bytes(uint64_t cap) {
     return 2 * align256(4 * cap * kMaxTopN)                      // qbin, qiq
-           + 4 * align256(4 * cap)                               // qn, lo, hi, nseg
+           + 4 * align256(4 * cap)                               // qn, lo, hi, cost
            + align256(8 * (cap + 1))                             // seg_off
-           + 4096                                                // scan temporaries
            + align256(sizeof(UnitTop) * cap * kNoAllocSegs * kMaxTopK)
            + 256                                                 // work counter
            + align256(sizeof(uint4) * cap * kNoAllocSegs)        // units
-           + align256(4 * 2 * kOrderBuckets)                     // its bucket counts
            + align256(sizeof(hicops_psm) * cap * kMaxTopK)       // psm (unused here)
            + align256(4 * cap * kHistBins) + align256(4 * cap);  // hist, n_scored
 }
@@ -854,9 +844,7 @@ extern "C" hicops_status hicops_search_noalloc(hicops_index* idx, const hicops_b
     if (st != HICOPS_OK) return st;
     Carve cv{base, kNoAllocBytes, 0};
     Workspace w;
-    uint32_t segs = max_segments(idx->dev.cfg, n);
-    if (segs > kNoAllocSegs) segs = kNoAllocSegs;
-    st = alloc_workspace(cv, idx->p, n, segs, true, w);
+    st = alloc_workspace(cv, idx->p, n, unit_limit(idx->dev.cfg, n, kNoAllocSegs), true, w);
     if (st != HICOPS_OK) {
         set_error("hicops_search_noalloc: scratch of %llu bytes is too small", (unsigned long long)kNoAllocBytes);
         return HICOPS_ENOMEM;

@@ -34,7 +34,8 @@
 // the log (one bit a peptide in two planes, super-chunks of 13 columns): 30k
 // spectra of 100 peaks at +-500 Da on 13.0 M peptides 15.7 -> 8.3 ms, 6k of 150
 // peaks on 11.7 M peptides 5.2 -> 3.5 ms, 12k of 50-500 peaks at mixed
-// tolerances 4.9 -> 3.1 ms.
+// tolerances 4.9 -> 3.1 ms; with windows cut by cost (plan_kernel) 7.6, 2.6 and
+// 2.9 ms.
 
 constexpr int kMaxHot = 6;                 // bitmap slices (b or y bitmap of a hot bucket) per spectrum
 constexpr int kMaxWarps = 16;              // CTAs of up to 512 threads

@@ -47,6 +47,11 @@ struct PrepArgs {
     uint32_t* qn;       // [n]
     uint32_t* lo;       // [n]
     uint32_t* hi;       // [n]
+    const BinInfo* bins;
+    uint32_t n_bins, tol_bins;
+    float per_peptide;  // of groups in a bucket to its hits a peptide
+    uint32_t slices;    // hot peaks that are bitmap slices at most (min_shared - 2)
+    uint32_t* cost;     // [n] what the spectrum's window costs (Cost), or NULL
     uint32_t* hist;     // [n * kHistBins] set to zero here, or NULL
     uint32_t* ns;       // [n] likewise
 };
@@ -142,16 +147,104 @@ __device__ __forceinline__ void warp_window(const double* __restrict__ mass, uin
     *hi = __shfl_sync(0xffffffffu, a, 16);
 }
 
-// a spectrum's count and window (one whole warp)
-__device__ __forceinline__ void put_window(const PrepArgs& a, uint32_t q, uint32_t keep, double prec, double tol,
-                                           uint32_t z, int lane) {
+// What searching a spectrum's window costs, in units of 64 entries (0 for an
+// empty window), estimated from the sizes of its peaks' buckets: the entries
+// to stream (a share W / P of every bucket, but for the hot peaks that become
+// bitmap slices, the densest), and where there are slices enough that every
+// peptide hit twice is looked at, those peptides, W lambda^2 / 2 of them at
+// lambda hits a peptide and kRepeatCost entries each (a fit to the measured
+// times gives 16 to 22; 40 splits the spectra whose peptides share fragments
+// beyond chance a little more).  Over 5,000 spectra the estimate's correlation
+// with the time is 0.90, of the entries alone 0.84.  It decides where windows
+// are split and in what order the units are taken, never what is found.
+// 1,111 spectra at +-500 Da: search 644 us with even pieces in their order ->
+// 388 us; 5,000 at a tolerance of one bin 3.21 -> 2.46 ms; 37: 51 -> 39 us;
+// 30,000: 7.95 -> 7.59 ms.
+constexpr float kRepeatCost = 40.0f;
+
+struct Cost {
+    static constexpr int kEarly = 4;
+    int2 early[kEarly];                    // the first peaks' hot and flags, on their way
+    float ordinary = 0.0f, hot = 0.0f;     // groups of 4 entries
+    float top = 0.0f, next = 0.0f;         // the densest hot peaks'
+    uint32_t nhot = 0;
+    static __device__ __forceinline__ int2 bucket(const PrepArgs& a, uint32_t bin) {
+        return __ldg(reinterpret_cast<const int2*>(a.bins + bin) + 1);
+    }
+    __device__ __forceinline__ void add(int2 b) {
+        const float g = (float)((uint32_t)b.y >> 2);
+        if (b.x >= 0) {
+            hot += g;
+            ++nhot;
+            next = fmaxf(next, fminf(top, g));
+            top = fmaxf(top, g);
+        } else {
+            ordinary += g;
+        }
+    }
+    // by a whole warp: the lanes' sums and greatest together, then the cost
+    __device__ __forceinline__ uint32_t of_window(const PrepArgs& a, uint32_t W, int lane) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ordinary += __shfl_xor_sync(0xffffffffu, ordinary, o);
+        nhot = __reduce_add_sync(0xffffffffu, nhot);
+        float streamed = 0.0f;
+        if (nhot > a.slices) {   // uniform
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) hot += __shfl_xor_sync(0xffffffffu, hot, o);
+            // (floats that are not negative order as integers)
+            const uint32_t t = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+            const bool mine = __float_as_uint(top) == t;
+            const unsigned holders = __ballot_sync(0xffffffffu, mine);
+            const bool first = mine && (holders & ((1u << lane) - 1u)) == 0;
+            const float t2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(first ? next : top)));
+            if (a.slices) hot -= __uint_as_float(t) + (float)(a.slices - 1u) * t2;
+            streamed = fmaxf(hot, 0.0f);
+        }
+        const float lambda = (ordinary + streamed) * a.per_peptide;
+        const float each = lambda + (nhot >= a.slices ? 0.5f * kRepeatCost * lambda * lambda : 0.0f);
+        return W ? 1u + (uint32_t)fminf(each * (float)W * (1.0f / 64.0f), 4.0e9f) : 0u;
+    }
+};
+
+// A spectrum's count, window and cost, by one whole warp.  Its keep bins are
+// the keys' high words (SHIFT 32) or low words (0).
+template <int SHIFT>
+__device__ __forceinline__ void put_window(const PrepArgs& a, uint32_t q, const uint64_t* keys, int keep, double prec,
+                                           double tol, uint32_t z, int lane) {
     uint32_t lo = 0, hi = 0;
+    Cost c;
     if (keep) {   // warp-uniform
+        if (a.cost) {
+#pragma unroll
+            for (int i = 0; i < Cost::kEarly; ++i) {
+                const int t = lane + 32 * i;
+                c.early[i] = t < keep ? Cost::bucket(a, (uint32_t)(keys[t] >> SHIFT)) : make_int2(-1, 0);
+            }
+        }
         const double Mq = __dmul_rn(__dsub_rn(prec, kProtonDa), (double)z);
         warp_window(a.mass, a.P, __dsub_rn(Mq, tol), __dadd_rn(Mq, tol), lane, &lo, &hi);
+        if (a.cost) {
+#pragma unroll
+            for (int i = 0; i < Cost::kEarly; ++i) c.add(c.early[i]);
+#pragma unroll 4
+            for (int t = lane + 32 * Cost::kEarly; t < keep; t += 32) c.add(Cost::bucket(a, (uint32_t)(keys[t] >> SHIFT)));
+            // the other bins within the fragment tolerance (two peaks' common ones twice)
+            for (int d = 1; d <= (int)a.tol_bins; ++d) {
+#pragma unroll 2
+                for (int t = lane; t < keep; t += 32) {
+                    const uint32_t bin = (uint32_t)(keys[t] >> SHIFT);
+                    if (bin >= (uint32_t)d) c.add(Cost::bucket(a, bin - d));
+                    if (bin + d < a.n_bins) c.add(Cost::bucket(a, bin + d));
+                }
+            }
+        }
+    }
+    if (a.cost) {
+        const uint32_t cost = c.of_window(a, hi - lo, lane);
+        if (lane == 0) a.cost[q] = cost;
     }
     if (lane == 0) {
-        a.qn[q] = keep;
+        a.qn[q] = (uint32_t)keep;
         a.lo[q] = lo;
         a.hi[q] = hi;
     }
@@ -240,7 +333,7 @@ __device__ __noinline__ void prep_block(const PrepArgs& a, uint32_t q, PrepShare
             }
         }
     }
-    if (threadIdx.x < 32) put_window(a, q, (uint32_t)keep, prec, tol, z, threadIdx.x);
+    if (threadIdx.x < 32) put_window<0>(a, q, keys, keep, prec, tol, z, threadIdx.x);
     __syncthreads();     // the keys, before the next spectrum's
 }
 
@@ -367,10 +460,13 @@ __device__ __forceinline__ void prep_warp(const PrepArgs& a, uint32_t q, uint64_
                 a.qbin[at] = (uint32_t)(k >> 32);
                 a.qiq[at] = quantise(__uint_as_float(val), __uint_as_float(top), a.scale);
             }
+            __syncwarp();
+            if (use) keys[out + __popc(msk & lt)] = k;   // (at or before its own place)
             out += __popc(msk);
         }
+        __syncwarp();
     }
-    put_window(a, q, (uint32_t)keep, prec, tol, z, lane);
+    put_window<32>(a, q, keys, keep, prec, tol, z, lane);
 }
 
 // Query preprocessing (R8) and the precursor window.  The first blocks take a
@@ -411,71 +507,6 @@ __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const __grid_constan
     }
 }
 
-// work units of a spectrum: its window split into pieces of >= seg_pids ids
-__device__ __forceinline__ uint32_t units_of(uint32_t qn, uint32_t lo, uint32_t hi, uint32_t max_seg, uint32_t seg_pids) {
-    if (qn == 0 || hi <= lo) return 0;
-    const uint64_t s = ((uint64_t)(hi - lo) + seg_pids - 1) / seg_pids;
-    return s > max_seg ? max_seg : (uint32_t)s;
-}
-
-__global__ void plan_kernel(const uint32_t* __restrict__ qn, const uint32_t* __restrict__ lo,
-                            const uint32_t* __restrict__ hi, uint32_t n, uint32_t max_seg, uint32_t seg_pids,
-                            uint32_t* __restrict__ nseg, unsigned long long* __restrict__ work) {
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q == 0) *work = 0ull;
-    if (q < n) nseg[q] = units_of(qn[q], lo[q], hi[q], max_seg, seg_pids);
-}
-
-// ---- units in the order they are taken: longest first (the persistent CTAs take units in this
-// order, so the short ones fill the end of the launch).  A unit's cost is
-// estimated as its peptide range times the spectrum's retained peaks; units
-// are bucketed by the cost's binary magnitude (a counting sort over 64
-// buckets, descending), block histograms first so that the global atomics
-// stay few.
-constexpr int kOrderBuckets = 64;
-constexpr uint32_t kOrderMinSpectra = 2048;   // smaller batches take their units in spectrum order
-
-__device__ __forceinline__ int order_bucket(const uint32_t* qn, const uint32_t* lo, const uint32_t* hi,
-                                            const uint64_t* seg_off, uint32_t q, uint32_t* ns) {
-    *ns = (uint32_t)(seg_off[q + 1] - seg_off[q]);
-    if (*ns == 0) return 0;
-    const uint64_t W = hi[q] - lo[q];
-    const uint64_t cost = ((W + *ns - 1) / *ns) * (uint64_t)(qn[q] ? qn[q] : 1) + 1;
-    return __clzll((long long)cost);   // 0 for the costliest magnitudes: descending order
-}
-
-__global__ void order_count_kernel(const uint32_t* __restrict__ qn, const uint32_t* __restrict__ lo,
-                                   const uint32_t* __restrict__ hi, const uint64_t* __restrict__ seg_off,
-                                   uint32_t n, uint32_t* __restrict__ cnt) {
-    __shared__ uint32_t bc[kOrderBuckets];
-    for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x) bc[i] = 0;
-    __syncthreads();
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < n) {
-        uint32_t ns;
-        const int b = order_bucket(qn, lo, hi, seg_off, q, &ns);
-        if (ns) atomicAdd(&bc[b], ns);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x)
-        if (bc[i]) atomicAdd(&cnt[i], bc[i]);
-}
-
-// cnt[0..63] counts -> cnt[64..127] exclusive starts (one warp)
-__global__ void order_scan_kernel(uint32_t* __restrict__ cnt) {
-    const int lane = threadIdx.x;
-    const uint32_t a = cnt[lane], b = cnt[32 + lane];
-    uint32_t ia = a, ib = b;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t xa = __shfl_up_sync(0xffffffffu, ia, o), xb = __shfl_up_sync(0xffffffffu, ib, o);
-        if (lane >= o) { ia += xa; ib += xb; }
-    }
-    const uint32_t tot_a = __shfl_sync(0xffffffffu, ia, 31);
-    cnt[kOrderBuckets + lane] = ia - a;
-    cnt[kOrderBuckets + 32 + lane] = tot_a + ib - b;
-}
-
 // A work unit: {spectrum, segment [lo, hi), unit number}.  The window of
 // spectrum q is split evenly into its ns units.
 __device__ __forceinline__ uint4 unit_record(uint32_t q, uint32_t lo, uint32_t hi, uint32_t ns, uint32_t s,
@@ -485,81 +516,156 @@ __device__ __forceinline__ uint4 unit_record(uint32_t q, uint32_t lo, uint32_t h
     return make_uint4(q, (uint32_t)min(a, (uint64_t)hi), (uint32_t)min(a + len, (uint64_t)hi), (uint32_t)(u0 + s));
 }
 
-__global__ void order_scatter_kernel(const uint32_t* __restrict__ qn, const uint32_t* __restrict__ lo,
-                                     const uint32_t* __restrict__ hi, const uint64_t* __restrict__ seg_off,
-                                     uint32_t n, uint32_t* __restrict__ cursor, uint4* __restrict__ unit) {
-    __shared__ uint32_t bc[kOrderBuckets], bb[kOrderBuckets];
-    for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x) bc[i] = 0;
-    __syncthreads();
-    const uint32_t q = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t ns = 0, local = 0;
-    int b = 0;
-    if (q < n) {
-        b = order_bucket(qn, lo, hi, seg_off, q, &ns);
-        if (ns) local = atomicAdd(&bc[b], ns);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x)
-        if (bc[i]) bb[i] = atomicAdd(&cursor[i], bc[i]);
-    __syncthreads();
-    if (ns) {
-        const uint32_t pos = bb[b] + local;
-        const uint64_t u0 = seg_off[q];
-        for (uint32_t s = 0; s < ns; ++s) unit[pos + s] = unit_record(q, lo[q], hi[q], ns, s, u0);
-    }
-}
+// How windows are split.  seg_pids given: into pieces of that many peptides.
+// Else by cost: into pieces of 1 / split of the batch's whole cost, so n
+// spectra have at most n + split units, and the spectra with common fragments,
+// which cost tens of the others, are in as many pieces.  No piece is under
+// kMinSegPids peptides, or under kUnitCost, where a unit's own set-up
+// outweighs its entries, unless the batch has less than that a CTA.
+struct PlanArgs {
+    const uint32_t* lo;
+    const uint32_t* hi;
+    const uint32_t* cost;
+    uint32_t n, max_seg, seg_pids, split, ctas;
+    uint64_t* seg_off;
+    uint4* unit;
+    unsigned long long* work;    // the search's unit counter, set to zero
+};
+constexpr uint32_t kUnitCost = 128, kUnitCostMin = 16;   // 8,192 and 1,024 entries
 
-// The whole planning of a small batch (fewer than kOrderMinSpectra spectra) in
-// one block: the spectra's units, their prefix and the unit records in
-// spectrum order.  Three launches (counts, scan, records) would be more of a
-// small call's time than the work in them.
-constexpr int kPlanThreads = 1024;
-__global__ void __launch_bounds__(kPlanThreads) plan_small_kernel(const uint32_t* __restrict__ qn,
-                                                                  const uint32_t* __restrict__ lo,
-                                                                  const uint32_t* __restrict__ hi, uint32_t n,
-                                                                  uint32_t max_seg, uint32_t seg_pids,
-                                                                  uint64_t* __restrict__ seg_off,
-                                                                  uint4* __restrict__ unit,
-                                                                  unsigned long long* __restrict__ work) {
-    __shared__ uint32_t off[kOrderMinSpectra + 1];   // (64 units a spectrum at most: 32 bits hold them)
-    __shared__ uint32_t wt[kPlanThreads / 32];
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t base = 0;
-    for (uint32_t q0 = 0; q0 < n; q0 += kPlanThreads) {
-        const uint32_t q = q0 + tid;
-        const uint32_t ns = q < n ? units_of(qn[q], lo[q], hi[q], max_seg, seg_pids) : 0u;
-        uint32_t incl = ns;
+// The planning of a batch in one block: the spectra's units, their prefix, and
+// the unit records, costliest first, since the persistent CTAs take them in
+// this order and the cheap ones fill the end of the launch (a counting sort
+// over quarter octaves of the unit's cost).  One block, since a grid's scan and
+// sort take seven launches: bound by latency, 7 us for a few spectra, 17 us for
+// 5,000 (38 us by seven launches), 58 us for 30,000 (38 us).
+constexpr uint32_t kPlanThreads = 1024, kPlanFew = 128;   // up to kPlanFew spectra: as many threads
+constexpr uint32_t kPlanEach = 4;          // consecutive spectra of a thread
+constexpr uint32_t kPlanBuckets = 512;     // a quarter octave of cost, four times (lanes that are alike spread over them)
+__global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constant__ PlanArgs a) {
+    __shared__ __align__(16) uint32_t bucket[kPlanBuckets];
+    __shared__ unsigned long long csum[kPlanThreads / 32];
+    __shared__ uint32_t wsum[kPlanThreads / 32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const uint32_t step = blockDim.x * kPlanEach;
+    uint32_t lo[kPlanEach], hi[kPlanEach], cost[kPlanEach];
+    // (a piece of the workspace is a multiple of 16 bytes: whole vectors, of which those behind n are left)
+    auto fetch = [&](uint32_t q0) {
+        uint4 l{}, h{}, c{};
+        if (q0 < a.n) {
+            l = *reinterpret_cast<const uint4*>(a.lo + q0);
+            h = *reinterpret_cast<const uint4*>(a.hi + q0);
+            c = *reinterpret_cast<const uint4*>(a.cost + q0);
+        }
+        lo[0] = l.x; lo[1] = l.y; lo[2] = l.z; lo[3] = l.w;
+        hi[0] = h.x; hi[1] = h.y; hi[2] = h.z; hi[3] = h.w;
+        cost[0] = c.x;
+        cost[1] = q0 + 1 < a.n ? c.y : 0u;
+        cost[2] = q0 + 2 < a.n ? c.z : 0u;
+        cost[3] = q0 + 3 < a.n ? c.w : 0u;
+    };
+    // the batch's cost
+    fetch(tid * kPlanEach);
+    unsigned long long sum = (unsigned long long)cost[0] + cost[1] + cost[2] + cost[3];
+#pragma unroll 8
+    for (uint32_t q = step + tid; q < a.n; q += blockDim.x) sum += a.cost[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) csum[warp] = sum;
+    for (uint32_t i = tid; i < kPlanBuckets; i += blockDim.x) bucket[i] = 0;
+    if (tid == 0) *a.work = 0ull;
+    __syncthreads();
+    sum = lane < nwarps ? csum[lane] : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    // (a float not above 1 / piece: 1 + floor of a cost's product with it is at
+    // most 1 + cost / piece, so the units keep to n + split)
+    const unsigned long long share = sum / a.split, cta = sum / a.ctas;
+    const unsigned long long least = min(max(cta, (unsigned long long)kUnitCostMin), (unsigned long long)kUnitCost);
+    const float per = __frcp_rd(__ull2float_ru(max(share + 1ull, least)));
+    uint32_t ns[kPlanEach], at[kPlanEach];    // units, their bucket
+    auto cut = [&]() {
+#pragma unroll
+        for (uint32_t i = 0; i < kPlanEach; ++i) {
+            const uint32_t c = cost[i], W = hi[i] - lo[i];
+            uint32_t k = 0;
+            if (c) {
+                if (a.seg_pids) k = W / a.seg_pids + (W % a.seg_pids ? 1u : 0u);
+                else k = min(1u + __float2uint_rz(__fmul_rz(__uint2float_rz(c), per)),
+                             (W + (kMinSegPids - 1)) / kMinSegPids);   // W < 2^31
+                k = min(k, a.max_seg);
+            }
+            ns[i] = k;
+            const int b = (int)(__float_as_uint(__fdividef((float)c, (float)max(k, 1u))) >> 21) - (int)(0x3f800000u >> 21);
+            at[i] = 4u * (kPlanBuckets / 4u - 1u - (uint32_t)min(max(b, 0), (int)kPlanBuckets / 4 - 1)) + (lane & 3u);
+        }
+    };
+    uint64_t base = 0, u0 = 0;      // units of the steps before; this thread's first unit of the last step
+    for (uint32_t q1 = 0; q1 < a.n; q1 += step) {
+        const uint32_t q0 = q1 + tid * kPlanEach;
+        if (q1) fetch(q0);
+        cut();
+        uint32_t mine = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < kPlanEach; ++i) {
+            if (ns[i]) atomicAdd(&bucket[at[i]], ns[i]);
+            mine += ns[i];
+        }
+        uint32_t incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= (uint32_t)o) incl += x;
         }
-        if (lane == 31) wt[warp] = incl;
+        if (q1) __syncthreads();   // wsum has been read
+        if (lane == 31) wsum[warp] = incl;
         __syncthreads();
-        const uint32_t t = wt[lane];
-        uint32_t before = lane < warp ? t : 0u;
-        before = __reduce_add_sync(0xffffffffu, before);
-        const uint32_t total = __reduce_add_sync(0xffffffffu, t);
-        if (q < n) {
-            off[q] = base + before + incl - ns;
-            seg_off[q] = off[q];
+        const uint32_t t = lane < nwarps ? wsum[lane] : 0u;
+        const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u);
+        u0 = base + before + incl - mine;
+        base += __reduce_add_sync(0xffffffffu, t);
+        uint64_t u = u0;
+#pragma unroll
+        for (uint32_t i = 0; i < kPlanEach; ++i) {
+            if (q0 + i < a.n) a.seg_off[q0 + i] = u;
+            u += ns[i];
         }
-        base += total;
-        __syncthreads();   // wt is reused
     }
-    if (tid == 0) {
-        off[n] = base;
-        seg_off[n] = base;
-        *work = 0ull;
+    if (tid == 0) a.seg_off[a.n] = base;
+    // bucket counts to starts (the last barrier is behind every count)
+    if (warp == 0) {
+        uint32_t start = 0;
+#pragma unroll
+        for (uint32_t i = lane; i < kPlanBuckets / 4; i += 32) {
+            const uint4 c = reinterpret_cast<const uint4*>(bucket)[i];
+            const uint32_t mine = c.x + c.y + c.z + c.w;
+            uint32_t incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= (uint32_t)o) incl += x;
+            }
+            const uint32_t f = start + incl - mine;
+            reinterpret_cast<uint4*>(bucket)[i] = make_uint4(f, f + c.x, f + c.x + c.y, f + c.x + c.y + c.z);
+            start += __shfl_sync(0xffffffffu, incl, 31);
+        }
     }
     __syncthreads();
-    for (uint32_t u = tid; u < base; u += kPlanThreads) {
-        uint32_t a = 0, b = n;   // the last spectrum with off <= u: it has units, the next one starts above u
-        while (b - a > 1) {
-            const uint32_t m = (a + b) >> 1;
-            if (off[m] <= u) a = m; else b = m;
+    for (uint32_t q1 = 0; q1 < a.n; q1 += step) {
+        const uint32_t q0 = q1 + tid * kPlanEach;
+        if (a.n > step) {           // else the only step's values are still there
+            fetch(q0);
+            cut();
+            u0 = q0 < a.n ? a.seg_off[q0] : 0;
         }
-        unit[u] = unit_record(a, lo[a], hi[a], off[a + 1] - off[a], u - off[a], off[a]);
+        uint64_t u = u0;
+#pragma unroll
+        for (uint32_t i = 0; i < kPlanEach; ++i) {
+            if (!ns[i]) continue;
+            const uint32_t to = atomicAdd(&bucket[at[i]], ns[i]);
+            for (uint32_t s = 0; s < ns[i]; ++s) a.unit[to + s] = unit_record(q0 + i, lo[i], hi[i], ns[i], s, u);
+            u += ns[i];
+        }
     }
 }
 
