@@ -28,7 +28,7 @@
 // one column, which is then searched with one counter a peptide.
 //
 // What bounds it: the latencies and the issue slots of pass A (one shared
-// atomic and about 16 instructions an entry; DRAM moves 470 KB a spectrum, a
+// atomic and about 16 instructions an entry; DRAM moves 580 KB a spectrum, a
 // third of the time at full rate) and, in spectra with thousands of scored
 // peptides, the drain.  Against the form that logged every entry and replayed
 // the log (one bit a peptide in two planes, super-chunks of 13 columns): 30k
