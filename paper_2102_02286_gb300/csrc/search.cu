@@ -5,9 +5,9 @@
 // One search is a fixed sequence on one stream:
 //   prep_kernel    R sub-task's "minimal computations": filter, bin, merge,
 //                  keep the B most intense peaks, quantise; precursor mass and
-//                  filter_1 (binary search of the mass-sorted database);
-//   plan_kernel +  work units (spectrum, peptide-id segment);
-//   exclusive scan
+//                  filter_1 (a search of the mass-sorted database);
+//   plan_kernel    work units (spectrum, peptide-id segment), cut and ordered
+//                  by estimated cost;
 //   search_kernel  filter_2 + score + heap over persistent CTAs;
 //   merge_kernel   per-spectrum top-k merge and the survival-tail e-value.
 // hicops_search takes its scratch stream-ordered from its index's pool; a plan

@@ -988,7 +988,7 @@ __global__ void __launch_bounds__(kMergeWarps * 32) merge_kernel(const __grid_co
 // (distinct bins in any order) by the union of their windows [b - t, b + t]
 // cut to [0, n_bins), ascending, each bin with the largest iq of the peaks
 // covering it.  One warp per spectrum, in place: the peaks are read into
-// shared memory and sorted by bin first.  Peak i emits the bins of its
+// shared memory and sorted by bin first, unless they ascend already.  Peak i emits the bins of its
 // window above the previous peak's window, so no bin is emitted twice, and
 // only peaks j >= i can cover them.
 constexpr int kExpWarps = 4;
