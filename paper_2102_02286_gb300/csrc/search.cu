@@ -20,6 +20,7 @@
 #include <cmath>
 #include <vector>
 
+#include "pieces.h"
 #include "search_kernels.cuh"
 #include "search_scratch.h"
 
@@ -37,62 +38,6 @@ struct DevBatch {
     const double* prec;
     const uint8_t* z;
     const double* tol;
-};
-
-// stream-ordered scratch from a pool (or the device's default one); freed on every exit path
-struct Scratch {
-    cudaStream_t s;
-    cudaMemPool_t pool;
-    std::vector<void*> ptrs;
-    explicit Scratch(cudaStream_t st, cudaMemPool_t p = nullptr) : s(st), pool(p) {}
-    template <class T>
-    cudaError_t get(T** p, uint64_t n) {
-        const size_t bytes = sizeof(T) * (n ? n : 1);
-        cudaError_t e = pool ? cudaMallocFromPoolAsync((void**)p, bytes, pool, s) : cudaMallocAsync((void**)p, bytes, s);
-        if (e == cudaSuccess) ptrs.push_back(*p);
-        return e;
-    }
-    ~Scratch() { for (void* p : ptrs) cudaFreeAsync(p, s); }
-};
-
-// persistent scratch of a plan
-struct Arena {
-    std::vector<void*> ptrs;
-    template <class T>
-    cudaError_t get(T** p, uint64_t n) {
-        cudaError_t e = cudaMalloc((void**)p, sizeof(T) * (n ? n : 1));
-        if (e == cudaSuccess) ptrs.push_back(*p);
-        return e;
-    }
-    ~Arena() { for (void* p : ptrs) cudaFree(p); }
-};
-
-constexpr uint64_t align256(uint64_t x) { return (x + 255) & ~uint64_t(255); }
-
-// alloc_workspace's allocators over caller memory.  Carve hands out
-// consecutive 256-byte aligned pieces of one buffer and fails when they would
-// not fit; Tally only adds up the bytes Carve would hand out.
-struct Carve {
-    unsigned char* base;
-    uint64_t cap, used;
-    template <class T>
-    cudaError_t get(T** p, uint64_t n) {
-        const uint64_t bytes = align256(sizeof(T) * (n ? n : 1));
-        if (used + bytes > cap) return cudaErrorMemoryAllocation;
-        *p = reinterpret_cast<T*>(base + used);
-        used += bytes;
-        return cudaSuccess;
-    }
-};
-
-struct Tally {
-    uint64_t used = 0;
-    template <class T>
-    cudaError_t get(T** p, uint64_t n) {
-        *p = nullptr;
-        used += align256(sizeof(T) * (n ? n : 1));
-        return cudaSuccess;
-    }
 };
 
 // Device scratch of one search of up to cap_n spectra in units of at most

@@ -549,7 +549,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const uint32_t step = blockDim.x * kPlanEach;
     uint32_t lo[kPlanEach], hi[kPlanEach], cost[kPlanEach];
-    // (a piece of the workspace is a multiple of 16 bytes: whole vectors, of which those behind n are left)
+    // (a piece of the workspace is a whole number of 256 bytes (pieces.h): whole vectors, whose words behind n
+    // are left)
     auto fetch = [&](uint32_t q0) {
         uint4 l{}, h{}, c{};
         if (q0 < a.n) {
