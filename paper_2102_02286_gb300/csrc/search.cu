@@ -48,7 +48,7 @@ struct Workspace {
     uint32_t *qbin = nullptr, *qiq = nullptr, *qn = nullptr, *lo = nullptr, *hi = nullptr, *cost = nullptr;
     uint64_t* seg_off = nullptr;
     UnitTop* utop = nullptr;
-    unsigned long long* work = nullptr;
+    unsigned long long* work = nullptr;   // [3] PlanArgs
     uint4* unit = nullptr;       // [max_units] units in the order they are taken
     hicops_psm* psm = nullptr;   // used when the caller gives no device output
     uint32_t* hist = nullptr;
@@ -75,7 +75,7 @@ hicops_status alloc_workspace(A& al, const hicops_params& p, uint32_t cap_n, con
     HC_CUDA(al.get(&w.cost, cap_n));
     HC_CUDA(al.get(&w.seg_off, (uint64_t)cap_n + 1));
     HC_CUDA(al.get(&w.utop, lim.units * p.top_k));
-    HC_CUDA(al.get(&w.work, 1));
+    HC_CUDA(al.get(&w.work, 3));
     HC_CUDA(al.get(&w.unit, lim.units));
     if (outputs) {
         HC_CUDA(al.get(&w.psm, (uint64_t)cap_n * p.top_k));
@@ -205,6 +205,67 @@ hicops_status launch_search(SearchArgs& sa, const hicops_search_config& c, uint6
     return launch_search_p<256>(sa, ctas, max_units, s);
 }
 
+// Which units are counted peptide by peptide (count_kernel.cuh): those of
+// spectra of at least this many expected hits a peptide.  No spectrum of a grid
+// whose average one has under two thirds of that: a call whose units are
+// all of one kind is spared the other's launch, and search_kernel falls back to
+// counters by itself where a single column's repeats overflow.
+float count_from(const hicops_index* idx) {
+    const hicops_params& p = idx->p;
+    if (p.min_shared < 2) return 0.0f;
+    if (p.min_shared == 2) return kCountShare2;
+    const float share = p.min_shared == 3 ? kCountShare3 : kCountShare;
+    const double ions = (double)idx->stats.n_entries / std::max<double>(1.0, (double)idx->mass.size());
+    const double grid = (p.frag_mz_max - p.frag_mz_min) / p.bin_width_da;
+    return query_bins_cap(p) * ions / grid > share * 2 / 3 ? share : INFINITY;
+}
+
+CountLayout make_count_layout(uint32_t stride, uint32_t k) {
+    const uint32_t maxp = (stride + 31) & ~31u, lists = kCountThreads / 32 * k;
+    CountLayout l{};
+    uint32_t at = kChunk;
+    auto take = [&at](uint32_t n) { const uint32_t o = at; at += (n + 3) & ~3u; return o; };   // 16-byte aligned
+    l.shared = take((sizeof(CountShared) + 3) / 4);
+    l.runs = take(4 * maxp + 8);
+    l.subs = take(2 * kCountThreads / kSub);
+    l.tkey = take(2 * lists);
+    l.base = take(maxp);
+    l.row = take(maxp);
+    l.iq = take(maxp);
+    l.queue = take(kCountQueue / 2);
+    l.tpid = take(lists);
+    l.tpk = take(lists);
+    l.end = at;
+    return l;
+}
+
+template <int PPT>
+hicops_status launch_count_t(const CountArgs& ca, uint32_t ctas, uint64_t max_units, cudaStream_t s) {
+    static std::atomic<bool> ready{false};   // concurrent first calls set the same values
+    if (!ready.load(std::memory_order_acquire)) {
+        HC_CUDA(cudaFuncSetAttribute(count_kernel<PPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(kSmemPerSm - 1024)));
+        HC_CUDA(cudaFuncSetAttribute(count_kernel<PPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     cudaSharedmemCarveoutMaxShared));
+        ready.store(true, std::memory_order_release);
+    }
+    uint64_t grid = (uint64_t)g_sm_count.load(std::memory_order_relaxed) * ctas;
+    if (max_units < grid) grid = max_units ? max_units : 1;
+    count_kernel<PPT><<<(unsigned)grid, kCountThreads, sizeof(uint32_t) * ca.lay.end, s>>>(ca);
+    count_launches(1);
+    HC_CUDA(cudaGetLastError());
+    return HICOPS_OK;
+}
+
+hicops_status launch_count(CountArgs& ca, const hicops_search_config& c, uint64_t max_units, cudaStream_t s) {
+    ca.lay = make_count_layout(ca.stride, ca.k);
+    // (the largest, 1,024 bins and 32 rows, takes 104 KB: two CTAs an SM)
+    uint32_t ctas = std::min<uint32_t>(kCountCtas, kSmemPerSm / (4 * ca.lay.end + 1024));
+    if (c.ctas_per_sm && c.ctas_per_sm < ctas) ctas = c.ctas_per_sm;
+    if (ca.stride <= kCountThreads) return launch_count_t<1>(ca, ctas, max_units, s);
+    return launch_count_t<kMaxTopN / kCountThreads>(ca, ctas, max_units, s);
+}
+
 inline void mark(hicops_index* idx, int i, cudaStream_t s, bool on) {
     if (on && idx->dev.timing) cudaEventRecord((cudaEvent_t)idx->dev.ev[i], s);
 }
@@ -231,7 +292,7 @@ hicops_status prepare_queries(hicops_index* idx, const DevBatch& d, uint32_t n, 
                 finite ? (uint64_t)std::ldexp(f, 64) : 0ull, finite ? e : 4096, p.intensity_scale,
                 idx->dev.mass, idx->mass.size(), qbin, qiq, qn, lo, hi, idx->dev.bins,
                 idx->n_bins, p.tol_bins, (float)(4.0 / std::max<double>(1.0, (double)idx->mass.size())),
-                p.min_shared > 2 ? p.min_shared - 2 : 0, cost, hist, ns};
+                p.min_shared > 2 ? p.min_shared - 2 : 0, count_from(idx), cost, hist, ns};
     const uint32_t big = std::min(n, kPrepBigBlocks);
     prep_kernel<<<big + (n + kPrepWarps - 1) / kPrepWarps, kPrepThreads, 0, s>>>(pa, big);
     count_launches(1);
@@ -258,18 +319,28 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     hicops_status st = prepare_queries(idx, d, n, w.qbin, w.qiq, w.qn, w.lo, w.hi, w.cost, d_hist, d_ns, s);
     if (st != HICOPS_OK) return st;
     mark(idx, 1, s, timing_marks);
+    const float from = count_from(idx);      // counted units: some may be, all are
     const uint32_t split = unit_limit(cfg, n).split;
     const PlanArgs plan{w.lo, w.hi, w.cost, n, w.max_seg, cfg.seg_pids, split,
-                        split / kSplitPerSm * (uint32_t)search_min_ctas((int)cfg.threads), w.seg_off, w.unit, w.work};
+                        split / kSplitPerSm * (uint32_t)search_min_ctas((int)cfg.threads), w.seg_off, w.unit, w.work,
+                        from < INFINITY};
     plan_kernel<<<1, n <= kPlanFew ? kPlanFew : kPlanThreads, 0, s>>>(plan);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
-    SearchArgs sa{w.qbin, w.qiq, w.qn, n, query_bins_cap(p), w.unit, w.seg_off + n, di.bins, di.entry, di.skip,
-                  di.skip_stride, di.hot_b, di.hot_y, di.hot_words, di.fwd_off, reinterpret_cast<const uint4*>(di.fwd), di.lf, di.ls,
+    SearchArgs sa{w.qbin, w.qiq, w.qn, n, query_bins_cap(p), w.unit,
+                  from < INFINITY ? reinterpret_cast<const uint64_t*>(w.work + 1) : w.seg_off + n, di.bins, di.entry,
+                  di.skip, di.skip_stride, di.hot_b, di.hot_y, di.hot_words, di.fwd_off, reinterpret_cast<const uint4*>(di.fwd), di.lf, di.ls,
                   (uint32_t)idx->s_max, p.min_shared, k, cfg.chunk_entries < 16 ? cfg.chunk_entries * 1024u : 0xffffffffu, w.utop, d_hist, d_ns, w.work,
                   SearchLayout{}};
     mark(idx, 2, s, timing_marks);
-    st = launch_search(sa, cfg, std::min(w.max_units, (uint64_t)n * w.max_seg), s);
+    const uint64_t max_units = std::min(w.max_units, (uint64_t)n * w.max_seg);
+    if (from > 0.0f) st = launch_search(sa, cfg, max_units, s);
+    if (st == HICOPS_OK && from < INFINITY) {
+        CountArgs ca{w.qbin, w.qiq, w.qn, query_bins_cap(p), w.unit, w.work + 1, w.seg_off + n, di.bins, di.entry, di.skip,
+                     di.skip_stride, di.lf, di.ls, (uint32_t)idx->s_max, p.min_shared, k, w.utop, d_hist, d_ns, w.work + 2,
+                     CountLayout{}};
+        st = launch_count(ca, cfg, max_units, s);
+    }
     if (st != HICOPS_OK) return st;
     mark(idx, 3, s, timing_marks);
     MergeArgs ma{w.seg_off, w.utop, nullptr, nullptr, 0, 0, nullptr, nullptr, d_hist, n, k, d_psm,

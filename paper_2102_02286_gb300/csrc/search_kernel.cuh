@@ -197,21 +197,25 @@ __device__ __forceinline__ uint32_t match_group(const SearchParts& sp, const uin
     return match_ion(sp, x.x) + match_ion(sp, x.y) + match_ion(sp, x.z) + match_ion(sp, x.w);
 }
 
-// The lanes' scored peptides (nb | ny | S in c): key, histogram, the warp's
-// top-k list (lanes in turn).  Every lane of the warp calls it.
-__device__ __forceinline__ void score_lanes(const SearchArgs& a, SearchShared& sh, const SearchParts& sp, bool ok,
-                                            uint32_t pid, uint32_t c) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = (int)a.k;
-    int64_t* const tkey = sp.tkey + warp * k;
-    uint32_t* const tpid = sp.tpid + warp * k;
-    uint32_t* const tpk = sp.tpk + warp * k;
-    const uint32_t nb = c >> kNbShift, ny = (c >> kNyShift) & 63u;
-    int64_t K = INT64_MIN;
+// The key of a peptide's nb | ny | S.
+template <class Args, class Shared>
+__device__ __forceinline__ int64_t score_key(const Args& a, const Shared& sh, uint32_t c) {
+    uint32_t S = c & kSMask;
+    if (S > a.s_max) S = a.s_max;   // unreachable for a consistent index
+    return sh.lf[c >> kNbShift] + sh.lf[(c >> kNyShift) & 63u] + __ldg(a.ls + S);
+}
+
+// The lanes' scored peptides (nb | ny | S in c, the key K): histogram, the
+// warp's top-k list (lanes in turn).  Every lane of the warp calls it.
+template <class Shared>
+__device__ __forceinline__ void rank_lanes(Shared& sh, int k, int64_t* tkey, uint32_t* tpid, uint32_t* tpk, bool ok,
+                                           uint32_t pid, uint32_t c, int64_t K) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    tkey += warp * k;
+    tpid += warp * k;
+    tpk += warp * k;
     bool pend = false;
-    if (ok && nb + ny >= a.min_shared) {
-        uint32_t S = c & kSMask;
-        if (S > a.s_max) S = a.s_max;   // unreachable for a consistent index
-        K = sh.lf[nb] + sh.lf[ny] + __ldg(a.ls + S);
+    if (ok) {
         const int64_t hb = K >> 31;
         atomicAdd(&sh.hist[hb > 255 ? 255 : (hb < 0 ? 0 : hb)], 1u);
         const int n = sh.wn[warp];
@@ -239,6 +243,14 @@ __device__ __forceinline__ void score_lanes(const SearchArgs& a, SearchShared& s
         }
         __syncwarp();
     }
+}
+
+__device__ __forceinline__ uint32_t hits_of(uint32_t c) { return (c >> kNbShift) + ((c >> kNyShift) & 63u); }
+
+__device__ __forceinline__ void score_lanes(const SearchArgs& a, SearchShared& sh, const SearchParts& sp, bool ok,
+                                            uint32_t pid, uint32_t c) {
+    ok = ok && hits_of(c) >= a.min_shared;
+    rank_lanes(sh, (int)a.k, sp.tkey, sp.tpid, sp.tpk, ok, pid, c, ok ? score_key(a, sh, c) : INT64_MIN);
 }
 
 // A peptide is taken when its hot bits reach what its ordinary hits leave to
@@ -552,6 +564,58 @@ __device__ __forceinline__ uint32_t put_shared(uint32_t at, uint32_t v, uint32_t
     return at;
 }
 
+// The end of unit u of spectrum q: its top-k, where every item of the warps'
+// sorted lists finds its rank among all of them, and its histogram added to the
+// spectrum's.  Every thread calls it, behind a barrier after the last score.
+template <int THREADS, class Args, class Shared>
+__device__ __forceinline__ void unit_out(const Args& a, Shared& sh, const int64_t* tkey, const uint32_t* tpid,
+                                         const uint32_t* tpk, uint32_t q, uint32_t u) {
+    constexpr int nwarps = THREADS / 32;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int k = (int)a.k;
+    for (uint32_t i = tid; i < (uint32_t)(nwarps * k); i += THREADS) {
+        const uint32_t w = i / (uint32_t)k, r = i % (uint32_t)k;
+        if (r >= (uint32_t)sh.wn[w]) continue;
+        UnitTop row;
+        row.key = tkey[i];
+        row.pid = tpid[i];
+        row.packed = tpk[i];
+        uint32_t rank = r;
+        for (uint32_t x = 0; x < (uint32_t)nwarps && rank < (uint32_t)k; ++x) {
+            if (x == w) continue;
+            const uint32_t n = (uint32_t)sh.wn[x];
+            for (uint32_t y = 0; y < n; ++y) {
+                if (!better(tkey[x * k + y], tpid[x * k + y], row.key, row.pid)) break;
+                ++rank;
+            }
+        }
+        if (rank < (uint32_t)k) a.utop[(uint64_t)u * k + rank] = row;
+    }
+    if (tid < k) {
+        int total = 0;
+#pragma unroll
+        for (int w = 0; w < nwarps; ++w) total += sh.wn[w];
+        if (tid >= total) {
+            UnitTop row;
+            row.key = INT64_MIN;
+            row.pid = 0xffffffffu;
+            row.packed = 0u;
+            a.utop[(uint64_t)u * k + tid] = row;
+        }
+    }
+    uint32_t mine = 0;
+    for (int jb = tid; jb < (int)kHistBins; jb += THREADS) {
+        const uint32_t h = sh.hist[jb];
+        if (h) {
+            atomicAdd(&a.hist[(uint64_t)q * kHistBins + jb], h);
+            mine += h;
+            sh.hist[jb] = 0;
+        }
+    }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0 && mine) atomicAdd(&a.nscored[q], mine);
+}
+
 constexpr int search_min_ctas(int threads) { return threads <= 256 ? 3 : threads <= 384 ? 2 : 1; }
 
 template <int THREADS, int PPT>
@@ -637,7 +701,8 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
                 // or none, which costs what streaming 1/8 of the segment's
                 // peptides does: when the rest hold fewer entries, only
                 // min_shared - 2 slices are taken and the rest are streamed
-                // like ordinary peaks, as are those that get no slice at all.
+                // like ordinary peaks, as are those that get no slice at all
+                // (all of them at min_shared 2: a scan would queue every hit).
                 // Which hot peaks get slices does not change any result.
                 const int nhc = sh.nhotc;
                 const uint32_t lo = sh.unit[st.slot].y, hi = sh.unit[st.slot].z;
@@ -661,7 +726,7 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
                         const int w = __ffs(__ballot_sync(0xffffffffu, left && n + 1u == most)) - 1;
                         const int nd = __shfl_sync(0xffffffffu, need, w);
                         // the cap: min_shared - 2 while the rest are few (all of them, not only these 32)
-                        const bool few = nhc <= 32 && rest < (float)(hi - lo) * 0.125f;
+                        const bool few = a.min_shared <= 2u || (nhc <= 32 && rest < (float)(hi - lo) * 0.125f);
                         if (ns + nd > (few ? min(kMaxHot, max((int)a.min_shared - 2, 0)) : kMaxHot)) open = false;
                         if (open) {
                             if (lane == w) {
@@ -769,7 +834,7 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
         // workloads' databases).  When a peptide of one ordinary hit cannot
         // qualify and the window needs several such super-chunks, they are
         // made wider than the plane (deep): peptides that share a bit only
-        // add repeats, about n n / 2 bits.  A repeat whose peptide needs three
+        // add repeats, about n n / 2 bits (at min_shared 2 each would be scored).  A repeat whose peptide needs three
         // ordinary hits or more then has to find its bit in the second plane
         // set (by an earlier repeat of its own, or of one that shares that
         // bit) before it counts, so the table only sees what is left of them,
@@ -801,7 +866,7 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
                 return (uint32_t)fmaxf(1.0f, fminf(w, (float)min(most, ncols)));
             };
             st.m = cols((float)kKeysAim, 0.0f, a.lay.plane_words / (kChunk / 32));
-            if ((uint32_t)sh.nslices + 2u <= a.min_shared && st.m < ncols) {
+            if ((uint32_t)sh.nslices + 2u <= a.min_shared && a.min_shared > 2u && st.m < ncols) {
                 const uint32_t md = cols(kPlane2Aim, 32.0f * (float)a.lay.plane_words, (1u << kOffBits) / kChunk - 1u);
                 if (md > st.m) {
                     st.m = md;
@@ -1060,51 +1125,7 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
             drain_queue(a);
             restore();
         }
-        // the unit's top-k: every item of the warps' sorted lists finds its
-        // rank among all of them
-        const int k = (int)a.k;
-        for (uint32_t i = tid; i < (uint32_t)(nwarps * k); i += THREADS) {
-            const uint32_t w = i / (uint32_t)k, r = i % (uint32_t)k;
-            if (r >= (uint32_t)sh.wn[w]) continue;
-            UnitTop row;
-            row.key = sp.tkey[i];
-            row.pid = sp.tpid[i];
-            row.packed = sp.tpk[i];
-            uint32_t rank = r;
-            for (uint32_t x = 0; x < (uint32_t)nwarps && rank < (uint32_t)k; ++x) {
-                if (x == w) continue;
-                const uint32_t n = (uint32_t)sh.wn[x];
-                for (uint32_t y = 0; y < n; ++y) {
-                    if (!better(sp.tkey[x * k + y], sp.tpid[x * k + y], row.key, row.pid)) break;
-                    ++rank;
-                }
-            }
-            if (rank < (uint32_t)k) a.utop[(uint64_t)sh.unit[st.slot].w * k + rank] = row;
-        }
-        if (tid < k) {
-            int total = 0;
-#pragma unroll
-            for (int w = 0; w < nwarps; ++w) total += sh.wn[w];
-            if (tid >= total) {
-                UnitTop row;
-                row.key = INT64_MIN;
-                row.pid = 0xffffffffu;
-                row.packed = 0u;
-                a.utop[(uint64_t)sh.unit[st.slot].w * k + tid] = row;
-            }
-        }
-        // histogram of this unit into the spectrum's histogram
-        uint32_t mine = 0;
-        for (int jb = tid; jb < (int)kHistBins; jb += THREADS) {
-            const uint32_t h = sh.hist[jb];
-            if (h) {
-                atomicAdd(&a.hist[(uint64_t)sh.unit[st.slot].x * kHistBins + jb], h);
-                mine += h;
-                sh.hist[jb] = 0;
-            }
-        }
-        mine = __reduce_add_sync(0xffffffffu, mine);
-        if (lane == 0 && mine) atomicAdd(&a.nscored[sh.unit[st.slot].x], mine);
+        unit_out<THREADS>(a, sh, sp.tkey, sp.tpid, sp.tpk, sh.unit[st.slot].x, sh.unit[st.slot].w);
         for (uint32_t i = tid; i < kHeads / 2; i += THREADS) sp.head[i] = 0u;
     }
 }

@@ -51,7 +51,8 @@ struct PrepArgs {
     uint32_t n_bins, tol_bins;
     float per_peptide;  // of groups in a bucket to its hits a peptide
     uint32_t slices;    // hot peaks that are bitmap slices at most (min_shared - 2)
-    uint32_t* cost;     // [n] what the spectrum's window costs (Cost), or NULL
+    float count_from;   // hits a peptide from which on the spectrum's units are counted (count_kernel.cuh)
+    uint32_t* cost;     // [n] what the spectrum's window costs (Cost), and kCounted, or NULL
     uint32_t* hist;     // [n * kHistBins] set to zero here, or NULL
     uint32_t* ns;       // [n] likewise
 };
@@ -160,7 +161,11 @@ __device__ __forceinline__ void warp_window(const double* __restrict__ mass, uin
 // 1,111 spectra at +-500 Da: search 644 us with even pieces in their order ->
 // 388 us; 5,000 at a tolerance of one bin 3.21 -> 2.46 ms; 37: 51 -> 39 us;
 // 30,000: 7.95 -> 7.59 ms.
+// Where a spectrum's units are counted instead (kCounted), the same entries and
+// a look at every counter, which costs what kCounterCost entries do.
 constexpr float kRepeatCost = 40.0f;
+constexpr float kCounterCost = 1.3f;
+constexpr uint32_t kCounted = 0x80000000u;
 
 struct Cost {
     static constexpr int kEarly = 4;
@@ -201,8 +206,10 @@ struct Cost {
             streamed = fmaxf(hot, 0.0f);
         }
         const float lambda = (ordinary + streamed) * a.per_peptide;
-        const float each = lambda + (nhot >= a.slices ? 0.5f * kRepeatCost * lambda * lambda : 0.0f);
-        return W ? 1u + (uint32_t)fminf(each * (float)W * (1.0f / 64.0f), 4.0e9f) : 0u;
+        const bool counted = lambda >= a.count_from;
+        const float each = lambda + (counted ? kCounterCost
+                                     : nhot >= a.slices ? 0.5f * kRepeatCost * lambda * lambda : 0.0f);
+        return W ? (counted ? kCounted : 0u) + 1u + (uint32_t)fminf(each * (float)W * (1.0f / 64.0f), 2.0e9f) : 0u;
     }
 };
 
@@ -529,7 +536,9 @@ struct PlanArgs {
     uint32_t n, max_seg, seg_pids, split, ctas;
     uint64_t* seg_off;
     uint4* unit;
-    unsigned long long* work;    // the search's unit counter, set to zero
+    unsigned long long* work;    // the unit counters of the search (0) and of the count (2), set to zero; where
+                                 // the counted units start (1)
+    uint32_t counts;             // there may be counted units: they come behind the others
 };
 constexpr uint32_t kUnitCost = 128, kUnitCostMin = 16;   // 8,192 and 1,024 entries
 
@@ -543,11 +552,12 @@ constexpr uint32_t kPlanThreads = 1024, kPlanFew = 128;   // up to kPlanFew spec
 constexpr uint32_t kPlanEach = 4;          // consecutive spectra of a thread
 constexpr uint32_t kPlanBuckets = 512;     // a quarter octave of cost, four times (lanes that are alike spread over them)
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constant__ PlanArgs a) {
-    __shared__ __align__(16) uint32_t bucket[kPlanBuckets];
+    __shared__ __align__(16) uint32_t bucket[2 * kPlanBuckets];     // of the units, then of the counted ones
     __shared__ unsigned long long csum[kPlanThreads / 32];
     __shared__ uint32_t wsum[kPlanThreads / 32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const uint32_t step = blockDim.x * kPlanEach;
+    const uint32_t halves = a.counts ? 2u : 1u;
     uint32_t lo[kPlanEach], hi[kPlanEach], cost[kPlanEach];
     // (a piece of the workspace is a whole number of 256 bytes (pieces.h): whole vectors, whose words behind n
     // are left)
@@ -567,14 +577,15 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     };
     // the batch's cost
     fetch(tid * kPlanEach);
-    unsigned long long sum = (unsigned long long)cost[0] + cost[1] + cost[2] + cost[3];
+    auto bare = [](uint32_t c) { return (unsigned long long)(c & ~kCounted); };
+    unsigned long long sum = bare(cost[0]) + bare(cost[1]) + bare(cost[2]) + bare(cost[3]);
 #pragma unroll 8
-    for (uint32_t q = step + tid; q < a.n; q += blockDim.x) sum += a.cost[q];
+    for (uint32_t q = step + tid; q < a.n; q += blockDim.x) sum += bare(a.cost[q]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) csum[warp] = sum;
-    for (uint32_t i = tid; i < kPlanBuckets; i += blockDim.x) bucket[i] = 0;
-    if (tid == 0) *a.work = 0ull;
+    for (uint32_t i = tid; i < halves * kPlanBuckets; i += blockDim.x) bucket[i] = 0;
+    if (tid == 0) a.work[0] = a.work[2] = 0ull;
     __syncthreads();
     sum = lane < nwarps ? csum[lane] : 0ull;
 #pragma unroll
@@ -588,7 +599,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     auto cut = [&]() {
 #pragma unroll
         for (uint32_t i = 0; i < kPlanEach; ++i) {
-            const uint32_t c = cost[i], W = hi[i] - lo[i];
+            const uint32_t c = cost[i] & ~kCounted, W = hi[i] - lo[i];
             uint32_t k = 0;
             if (c) {
                 if (a.seg_pids) k = W / a.seg_pids + (W % a.seg_pids ? 1u : 0u);
@@ -598,7 +609,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
             }
             ns[i] = k;
             const int b = (int)(__float_as_uint(__fdividef((float)c, (float)max(k, 1u))) >> 21) - (int)(0x3f800000u >> 21);
-            at[i] = 4u * (kPlanBuckets / 4u - 1u - (uint32_t)min(max(b, 0), (int)kPlanBuckets / 4 - 1)) + (lane & 3u);
+            at[i] = 4u * (kPlanBuckets / 4u - 1u - (uint32_t)min(max(b, 0), (int)kPlanBuckets / 4 - 1)) + (lane & 3u) +
+                    (cost[i] & kCounted ? kPlanBuckets : 0u);
         }
     };
     uint64_t base = 0, u0 = 0;      // units of the steps before; this thread's first unit of the last step
@@ -636,8 +648,9 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     // bucket counts to starts (the last barrier is behind every count)
     if (warp == 0) {
         uint32_t start = 0;
-#pragma unroll
-        for (uint32_t i = lane; i < kPlanBuckets / 4; i += 32) {
+#pragma unroll 4
+        for (uint32_t i = lane; i < halves * kPlanBuckets / 4; i += 32) {
+            if (i == kPlanBuckets / 4) a.work[1] = start;
             const uint4 c = reinterpret_cast<const uint4*>(bucket)[i];
             const uint32_t mine = c.x + c.y + c.z + c.w;
             uint32_t incl = mine;
@@ -679,6 +692,7 @@ struct SearchLayout {
 };
 
 #include "search_kernel.cuh"
+#include "count_kernel.cuh"
 
 // lower bound of pid key (pid << 1) in entry[a, b)
 __device__ __forceinline__ uint64_t entry_lower_bound(const uint32_t* __restrict__ entry, uint64_t a, uint64_t b,
