@@ -53,6 +53,7 @@ void set_error(const char* fmt, ...);
 struct DeviceIndex {
     bool ready = false;
     int device = -1;
+    uint32_t sms = 0;              // SMs of the device
     double* mass = nullptr;        // [P] neutral mass, pid order
     uint64_t* off = nullptr;       // [n_bins + 1] bucket offsets (multiples of 4)
     uint32_t* entry = nullptr;     // [n_stored + 4] pid << 1 | isY, pid ascending in a bucket; each
@@ -106,6 +107,10 @@ struct RawAllocator : std::allocator<T> {
 };
 template <class T>
 using RawVector = std::vector<T, RawAllocator<T>>;
+
+// Learns what searches need of the index's device, which is current, and opts their
+// kernels into its shared memory (search.cu; part of an upload).
+hicops_status search_setup(hicops_index* idx);
 
 // Counts every kernel launch of the library.
 void count_launches(uint64_t n);

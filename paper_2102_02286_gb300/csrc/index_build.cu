@@ -504,6 +504,8 @@ hicops_status upload_index(hicops_index* idx) {
     auto t0 = std::chrono::steady_clock::now();
     DeviceIndex& d = idx->dev;
     HC_CUDA(cudaGetDevice(&d.device));
+    const hicops_status ready = search_setup(idx);
+    if (ready != HICOPS_OK) return ready;
     const hicops_params& p = idx->p;
     const uint64_t P = idx->mass.size();
     const uint64_t B = idx->bases->base_off.size() - 1;

@@ -85,18 +85,6 @@ hicops_status alloc_workspace(A& al, const hicops_params& p, uint32_t cap_n, con
     return HICOPS_OK;
 }
 
-std::atomic<int> g_sm_count{0};   // set on first use; every thread computes the same value
-
-hicops_status sm_count() {
-    if (!g_sm_count.load(std::memory_order_relaxed)) {
-        int dev, c = 0;
-        HC_CUDA(cudaGetDevice(&dev));
-        HC_CUDA(cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev));
-        g_sm_count.store(c, std::memory_order_relaxed);
-    }
-    return HICOPS_OK;
-}
-
 hicops_status check_config(const hicops_search_config& c) {
     if (c.threads != 0 && c.threads != 256 && c.threads != 384 && c.threads != 512) {
         set_error("threads must be 256, 384 or 512");
@@ -123,8 +111,8 @@ hicops_search_config resolved(const hicops_search_config& c, uint32_t query_bins
 // kSplitPerSm pieces an SM to even out the CTAs' shares, by the batch's cost.
 constexpr uint32_t kSplitPerSm = 8;
 
-UnitLimit unit_limit(const hicops_search_config& c, uint64_t n, uint32_t max_seg = kMaxSegs) {
-    const uint32_t split = kSplitPerSm * (uint32_t)g_sm_count.load(std::memory_order_relaxed);
+UnitLimit unit_limit(const hicops_index* idx, const hicops_search_config& c, uint64_t n, uint32_t max_seg = kMaxSegs) {
+    const uint32_t split = kSplitPerSm * idx->dev.sms;
     const uint64_t most = n * max_seg;
     return UnitLimit{max_seg, split, c.seg_pids ? most : std::min(most, n + split)};
 }
@@ -163,35 +151,38 @@ SearchLayout make_layout(uint32_t stride, uint32_t k, uint32_t threads, uint32_t
     return l;
 }
 
+// A kernel's dynamic shared memory is opted into per function and device: for
+// all of them when an index is uploaded to its device.
+template <class Kernel>
+cudaError_t allow_shared(Kernel* k) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemPerSm - 1024));
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
+
 template <int THREADS, int PPT>
-hicops_status launch_search_t(const SearchArgs& sa, uint32_t ctas, uint64_t max_units, cudaStream_t s) {
-    static std::atomic<bool> ready{false};   // concurrent first calls set the same values
-    const size_t smem = sizeof(uint32_t) * sa.lay.end;
-    if (!ready.load(std::memory_order_acquire)) {
-        HC_CUDA(cudaFuncSetAttribute(search_kernel<THREADS, PPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kSmemPerSm - 1024)));
-        HC_CUDA(cudaFuncSetAttribute(search_kernel<THREADS, PPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared));
-        ready.store(true, std::memory_order_release);
-    }
-    // no more CTAs than work units can exist
-    uint64_t grid = (uint64_t)g_sm_count.load(std::memory_order_relaxed) * ctas;
-    if (max_units < grid) grid = max_units ? max_units : 1;
-    search_kernel<THREADS, PPT><<<(unsigned)grid, THREADS, smem, s>>>(sa);
+hicops_status launch_search_t(const SearchArgs& sa, uint64_t grid, cudaStream_t s) {
+    search_kernel<THREADS, PPT><<<(unsigned)grid, THREADS, sizeof(uint32_t) * sa.lay.end, s>>>(sa);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
     return HICOPS_OK;
 }
 
-// PPT: ordinary peaks a thread owns at most
-template <int THREADS>
-hicops_status launch_search_p(const SearchArgs& sa, uint32_t ctas, uint64_t max_units, cudaStream_t s) {
-    if (sa.stride <= THREADS) return launch_search_t<THREADS, 1>(sa, ctas, max_units, s);
-    if (sa.stride <= 2 * THREADS) return launch_search_t<THREADS, 2>(sa, ctas, max_units, s);
-    return launch_search_t<THREADS, 4>(sa, ctas, max_units, s);
+// no more CTAs than work units can exist
+uint64_t grid_of(const hicops_index* idx, uint32_t ctas, uint64_t max_units) {
+    return std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)idx->dev.sms * ctas, max_units));
 }
 
-hicops_status launch_search(SearchArgs& sa, const hicops_search_config& c, uint64_t max_units, cudaStream_t s) {
+// PPT: ordinary peaks a thread owns at most
+template <int THREADS>
+hicops_status launch_search_p(const SearchArgs& sa, uint64_t grid, cudaStream_t s) {
+    if (sa.stride <= THREADS) return launch_search_t<THREADS, 1>(sa, grid, s);
+    if (sa.stride <= 2 * THREADS) return launch_search_t<THREADS, 2>(sa, grid, s);
+    return launch_search_t<THREADS, 4>(sa, grid, s);
+}
+
+hicops_status launch_search(const hicops_index* idx, SearchArgs& sa, const hicops_search_config& c, uint64_t max_units,
+                            cudaStream_t s) {
     uint32_t ctas = (uint32_t)search_min_ctas((int)c.threads);
     if (c.ctas_per_sm && c.ctas_per_sm < ctas) ctas = c.ctas_per_sm;
     // many query bins or long top-k lists leave little for the plane: fewer
@@ -200,9 +191,10 @@ hicops_status launch_search(SearchArgs& sa, const hicops_search_config& c, uint6
         sa.lay = make_layout(sa.stride, sa.k, c.threads, ctas);
         if (ctas == 1 || sa.lay.plane_words >= kMinPlaneWords) break;
     }
-    if (c.threads == 512) return launch_search_p<512>(sa, ctas, max_units, s);
-    if (c.threads == 384) return launch_search_p<384>(sa, ctas, max_units, s);
-    return launch_search_p<256>(sa, ctas, max_units, s);
+    const uint64_t grid = grid_of(idx, ctas, max_units);
+    if (c.threads == 512) return launch_search_p<512>(sa, grid, s);
+    if (c.threads == 384) return launch_search_p<384>(sa, grid, s);
+    return launch_search_p<256>(sa, grid, s);
 }
 
 // Which units are counted peptide by peptide (count_kernel.cuh): those of
@@ -240,30 +232,22 @@ CountLayout make_count_layout(uint32_t stride, uint32_t k) {
 }
 
 template <int PPT>
-hicops_status launch_count_t(const CountArgs& ca, uint32_t ctas, uint64_t max_units, cudaStream_t s) {
-    static std::atomic<bool> ready{false};   // concurrent first calls set the same values
-    if (!ready.load(std::memory_order_acquire)) {
-        HC_CUDA(cudaFuncSetAttribute(count_kernel<PPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(kSmemPerSm - 1024)));
-        HC_CUDA(cudaFuncSetAttribute(count_kernel<PPT>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared));
-        ready.store(true, std::memory_order_release);
-    }
-    uint64_t grid = (uint64_t)g_sm_count.load(std::memory_order_relaxed) * ctas;
-    if (max_units < grid) grid = max_units ? max_units : 1;
+hicops_status launch_count_t(const CountArgs& ca, uint64_t grid, cudaStream_t s) {
     count_kernel<PPT><<<(unsigned)grid, kCountThreads, sizeof(uint32_t) * ca.lay.end, s>>>(ca);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
     return HICOPS_OK;
 }
 
-hicops_status launch_count(CountArgs& ca, const hicops_search_config& c, uint64_t max_units, cudaStream_t s) {
+hicops_status launch_count(const hicops_index* idx, CountArgs& ca, const hicops_search_config& c, uint64_t max_units,
+                           cudaStream_t s) {
     ca.lay = make_count_layout(ca.stride, ca.k);
     // (the largest, 1,024 bins and 32 rows, takes 104 KB: two CTAs an SM)
     uint32_t ctas = std::min<uint32_t>(kCountCtas, kSmemPerSm / (4 * ca.lay.end + 1024));
     if (c.ctas_per_sm && c.ctas_per_sm < ctas) ctas = c.ctas_per_sm;
-    if (ca.stride <= kCountThreads) return launch_count_t<1>(ca, ctas, max_units, s);
-    return launch_count_t<kMaxTopN / kCountThreads>(ca, ctas, max_units, s);
+    const uint64_t grid = grid_of(idx, ctas, max_units);
+    if (ca.stride <= kCountThreads) return launch_count_t<1>(ca, grid, s);
+    return launch_count_t<kMaxTopN / kCountThreads>(ca, grid, s);
 }
 
 inline void mark(hicops_index* idx, int i, cudaStream_t s, bool on) {
@@ -320,7 +304,7 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     if (st != HICOPS_OK) return st;
     mark(idx, 1, s, timing_marks);
     const float from = count_from(idx);      // counted units: some may be, all are
-    const uint32_t split = unit_limit(cfg, n).split;
+    const uint32_t split = unit_limit(idx, cfg, n).split;
     const PlanArgs plan{w.lo, w.hi, w.cost, n, w.max_seg, cfg.seg_pids, split,
                         split / kSplitPerSm * (uint32_t)search_min_ctas((int)cfg.threads), w.seg_off, w.unit, w.work,
                         from < INFINITY};
@@ -334,12 +318,12 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
                   SearchLayout{}};
     mark(idx, 2, s, timing_marks);
     const uint64_t max_units = std::min(w.max_units, (uint64_t)n * w.max_seg);
-    if (from > 0.0f) st = launch_search(sa, cfg, max_units, s);
+    if (from > 0.0f) st = launch_search(idx, sa, cfg, max_units, s);
     if (st == HICOPS_OK && from < INFINITY) {
         CountArgs ca{w.qbin, w.qiq, w.qn, query_bins_cap(p), w.unit, w.work + 1, w.seg_off + n, di.bins, di.entry, di.skip,
                      di.skip_stride, di.lf, di.ls, (uint32_t)idx->s_max, p.min_shared, k, w.utop, d_hist, d_ns, w.work + 2,
                      CountLayout{}};
-        st = launch_count(ca, cfg, max_units, s);
+        st = launch_count(idx, ca, cfg, max_units, s);
     }
     if (st != HICOPS_OK) return st;
     mark(idx, 3, s, timing_marks);
@@ -365,7 +349,7 @@ hicops_status check_batch(const hicops_index* idx, const hicops_batch* b) {
         set_error("current device %d is not the index's device %d", dev, idx->dev.device);
         return HICOPS_EINVAL;
     }
-    return sm_count();
+    return HICOPS_OK;
 }
 
 // Inputs on the device: the caller's, or (on_device = 0) pieces to copy them to.
@@ -420,11 +404,29 @@ hicops_status scratch_workspace(A& al, const hicops_params& p, uint32_t n, const
 
 }  // namespace
 
+hicops_status search_setup(hicops_index* idx) {
+    int sms = 0;
+    HC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, idx->dev.device));
+    idx->dev.sms = (uint32_t)sms;
+    HC_CUDA((allow_shared(search_kernel<256, 1>)));
+    HC_CUDA((allow_shared(search_kernel<256, 2>)));
+    HC_CUDA((allow_shared(search_kernel<256, 4>)));
+    HC_CUDA((allow_shared(search_kernel<384, 1>)));
+    HC_CUDA((allow_shared(search_kernel<384, 2>)));
+    HC_CUDA((allow_shared(search_kernel<384, 4>)));
+    HC_CUDA((allow_shared(search_kernel<512, 1>)));
+    HC_CUDA((allow_shared(search_kernel<512, 2>)));
+    HC_CUDA((allow_shared(search_kernel<512, 4>)));
+    HC_CUDA((allow_shared(count_kernel<1>)));
+    HC_CUDA((allow_shared(count_kernel<kMaxTopN / kCountThreads>)));
+    return HICOPS_OK;
+}
+
 uint64_t scratch_bytes(const hicops_index* idx, const hicops_search_config& cfg, uint32_t n) {
     if (!n) n = 1;
     Tally t;
     Workspace w;
-    scratch_workspace(t, idx->p, n, unit_limit(cfg, n), w);
+    scratch_workspace(t, idx->p, n, unit_limit(idx, cfg, n), w);
     return t.used;
 }
 
@@ -451,7 +453,7 @@ hicops_status search_in_scratch(hicops_index* idx, const hicops_batch* b, const 
     }
     Carve cv{static_cast<unsigned char*>(scratch), bytes, 0};
     Workspace w;
-    st = scratch_workspace(cv, idx->p, n, unit_limit(cfg, n), w);
+    st = scratch_workspace(cv, idx->p, n, unit_limit(idx, cfg, n), w);
     if (st != HICOPS_OK) return st;
     const DevBatch d{b->peak_off, b->mz, b->intensity, b->prec_mz, b->charge, b->prec_tol_da};
     return enqueue_search(idx, d, n, w, cfg, out_psm, out_hist ? out_hist : w.hist, out_nscored ? out_nscored : w.ns,
@@ -465,8 +467,6 @@ using namespace hicops;
 extern "C" hicops_status hicops_search_scratch_bytes(const hicops_index* idx, uint32_t n, uint64_t* out_bytes) {
     if (!idx || !out_bytes) { set_error("NULL argument"); return HICOPS_EINVAL; }
     if (!idx->dev.ready) { set_error("index has no device part (call hicops_index_upload)"); return HICOPS_EINVAL; }
-    hicops_status st = sm_count();
-    if (st != HICOPS_OK) return st;
     *out_bytes = scratch_bytes(idx, idx->dev.cfg, n);
     return HICOPS_OK;
 }
@@ -507,7 +507,7 @@ extern "C" hicops_status hicops_search(hicops_index* idx, const hicops_batch* b,
     cudaStream_t s = (cudaStream_t)b->cuda_stream;
     {
         // one piece of the pool a call, carved into inputs, workspace and outputs
-        const UnitLimit lim = unit_limit(idx->dev.cfg, n);
+        const UnitLimit lim = unit_limit(idx, idx->dev.cfg, n);
         const bool own_hist = !b->on_device || !out_hist, own_ns = !b->on_device || !out_nscored;
         DevBatch d;
         Workspace w;
@@ -601,20 +601,18 @@ extern "C" hicops_status hicops_plan_create(hicops_index* idx, uint32_t max_spec
     *out = nullptr;
     if (!idx->dev.ready) { set_error("index not uploaded"); return HICOPS_EINVAL; }
     HC_CUDA(cudaSetDevice(idx->dev.device));
-    hicops_status st = sm_count();
-    if (st != HICOPS_OK) return st;
     hicops_plan* pl = new (std::nothrow) hicops_plan();
     if (!pl) { set_error("out of host memory"); return HICOPS_ENOMEM; }
     pl->idx = idx;
     pl->cfg = cfg ? *cfg : idx->dev.cfg;
-    st = check_config(pl->cfg);
+    hicops_status st = check_config(pl->cfg);
     // with pieces of a given size, per-unit top-k lists of up to kMaxSegs units per spectrum within 1 GiB
     const uint64_t per_seg = (uint64_t)max_spectra * idx->p.top_k * sizeof(UnitTop);
     uint64_t segs = (1ull << 30) / per_seg;
     if (segs > (uint64_t)kMaxSegs || !pl->cfg.seg_pids) segs = kMaxSegs;
     if (segs < 1) segs = 1;
     if (st == HICOPS_OK)
-        st = alloc_workspace(pl->arena, idx->p, max_spectra, unit_limit(pl->cfg, max_spectra, (uint32_t)segs), true,
+        st = alloc_workspace(pl->arena, idx->p, max_spectra, unit_limit(idx, pl->cfg, max_spectra, (uint32_t)segs), true,
                              pl->ws);
     if (st != HICOPS_OK) { delete pl; return st; }
     *out = pl;
@@ -642,7 +640,7 @@ extern "C" hicops_status hicops_plan_search(hicops_plan* pl, const hicops_batch*
     if (!same) {
         if (pl->exec) { cudaGraphExecDestroy(pl->exec); pl->exec = nullptr; }
         if (pl->graph) { cudaGraphDestroy(pl->graph); pl->graph = nullptr; }
-        // first-use set-up of the kernel attributes happens outside capture
+        // (a kernel's first use loads it, outside capture)
         st = enqueue_search(pl->idx, d, n, w, pl->cfg, out_psm, d_hist, d_ns, s, false);
         if (st != HICOPS_OK) return st;
         const uint64_t before = g_launches.load();
@@ -860,7 +858,7 @@ extern "C" hicops_status hicops_search_noalloc(hicops_index* idx, const hicops_b
     if (st != HICOPS_OK) return st;
     Carve cv{base, kNoAllocBytes, 0};
     Workspace w;
-    st = alloc_workspace(cv, idx->p, n, unit_limit(idx->dev.cfg, n, kNoAllocSegs), true, w);
+    st = alloc_workspace(cv, idx->p, n, unit_limit(idx, idx->dev.cfg, n, kNoAllocSegs), true, w);
     if (st != HICOPS_OK) {
         set_error("hicops_search_noalloc: scratch of %llu bytes is too small", (unsigned long long)kNoAllocBytes);
         return HICOPS_ENOMEM;

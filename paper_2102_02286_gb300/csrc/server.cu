@@ -327,9 +327,6 @@ extern "C" hicops_status hicops_server_create(hicops_index* idx, const hicops_se
         return HICOPS_EINVAL;
     }
     HC_CUDA(cudaSetDevice(idx->dev.device));
-    uint64_t probe = 0;
-    hicops_status st = hicops_search_scratch_bytes(idx, 1, &probe);   // also learns the SM count
-    if (st != HICOPS_OK) return st;
     std::unique_ptr<hicops_server, void (*)(hicops_server*)> srv(new hicops_server(), free_server);
     srv->idx = idx;
     srv->device = idx->dev.device;
