@@ -510,8 +510,9 @@ void hicops_plan_destroy(hicops_plan* plan);
  * submission and queued.  The server's device memory is one pool of
  * memory_budget bytes, allocated at creation.  A scheduler thread packs the
  * oldest waiting requests into one launch while that launch's block (its
- * spectra, the search's scratch as hicops_search_scratch_bytes counts it,
- * its PSM rows, histograms and counts) fits the pool's largest free range,
+ * spectra, its PSM rows, histograms and counts, and the search's scratch: what
+ * hicops_search_scratch_bytes counts, less the histograms and counts there)
+ * fits the pool's largest free range,
  * and launches it on an idle stream; when the oldest request does not fit,
  * it waits until launches in flight return their blocks.  Requests that
  * arrive while others run are thus admitted as memory and streams free up,

@@ -391,12 +391,13 @@ hicops_status copy_inputs(const hicops_batch* b, const DevBatch& d, cudaStream_t
 }
 
 // The workspace of a search in caller memory: alloc_workspace's pieces
-// without the PSM rows (the caller always gives those), then a histogram and
-// candidate-count block for callers that pass none.
+// without the PSM rows (the caller always gives those), then, for callers that
+// may pass none, a histogram and candidate-count block (outputs).
 template <class A>
-hicops_status scratch_workspace(A& al, const hicops_params& p, uint32_t n, const UnitLimit& lim, Workspace& w) {
+hicops_status scratch_workspace(A& al, const hicops_params& p, uint32_t n, const UnitLimit& lim, bool outputs,
+                                Workspace& w) {
     hicops_status st = alloc_workspace(al, p, n, lim, false, w);
-    if (st != HICOPS_OK) return st;
+    if (st != HICOPS_OK || !outputs) return st;
     HC_CUDA(al.get(&w.hist, (uint64_t)n * kHistBins));
     HC_CUDA(al.get(&w.ns, n));
     return HICOPS_OK;
@@ -422,16 +423,16 @@ hicops_status search_setup(hicops_index* idx) {
     return HICOPS_OK;
 }
 
-uint64_t scratch_bytes(const hicops_index* idx, const hicops_search_config& cfg, uint32_t n) {
+uint64_t scratch_bytes(const hicops_index* idx, const hicops_search_config& cfg, uint32_t n, bool outputs) {
     if (!n) n = 1;
     Tally t;
     Workspace w;
-    scratch_workspace(t, idx->p, n, unit_limit(idx, cfg, n), w);
+    scratch_workspace(t, idx->p, n, unit_limit(idx, cfg, n), outputs, w);
     return t.used;
 }
 
 hicops_status search_in_scratch(hicops_index* idx, const hicops_batch* b, const hicops_search_config& cfg,
-                                void* scratch, uint64_t bytes, hicops_psm* out_psm, uint32_t* out_hist,
+                                void* scratch, uint64_t bytes, bool outputs, hicops_psm* out_psm, uint32_t* out_hist,
                                 uint32_t* out_nscored) {
     hicops_status st = check_batch(idx, b);
     if (st != HICOPS_OK) return st;
@@ -439,13 +440,14 @@ hicops_status search_in_scratch(hicops_index* idx, const hicops_batch* b, const 
         set_error("a search in caller scratch takes device pointers (on_device = 1) and a device out_psm");
         return HICOPS_EINVAL;
     }
+    if (!outputs && (!out_hist || !out_nscored)) { set_error("NULL argument"); return HICOPS_EINVAL; }
     if (!scratch || (reinterpret_cast<uintptr_t>(scratch) & 255u)) {
         set_error("scratch must be a 256-byte aligned device pointer");
         return HICOPS_EINVAL;
     }
     const uint32_t n = b->n;
     if (n == 0) return HICOPS_OK;
-    const uint64_t need = scratch_bytes(idx, cfg, n);
+    const uint64_t need = scratch_bytes(idx, cfg, n, outputs);
     if (bytes < need) {
         set_error("scratch of %llu bytes; a search of %u spectra needs %llu", (unsigned long long)bytes, n,
                   (unsigned long long)need);
@@ -453,7 +455,7 @@ hicops_status search_in_scratch(hicops_index* idx, const hicops_batch* b, const 
     }
     Carve cv{static_cast<unsigned char*>(scratch), bytes, 0};
     Workspace w;
-    st = scratch_workspace(cv, idx->p, n, unit_limit(idx, cfg, n), w);
+    st = scratch_workspace(cv, idx->p, n, unit_limit(idx, cfg, n), outputs, w);
     if (st != HICOPS_OK) return st;
     const DevBatch d{b->peak_off, b->mz, b->intensity, b->prec_mz, b->charge, b->prec_tol_da};
     return enqueue_search(idx, d, n, w, cfg, out_psm, out_hist ? out_hist : w.hist, out_nscored ? out_nscored : w.ns,
@@ -467,7 +469,7 @@ using namespace hicops;
 extern "C" hicops_status hicops_search_scratch_bytes(const hicops_index* idx, uint32_t n, uint64_t* out_bytes) {
     if (!idx || !out_bytes) { set_error("NULL argument"); return HICOPS_EINVAL; }
     if (!idx->dev.ready) { set_error("index has no device part (call hicops_index_upload)"); return HICOPS_EINVAL; }
-    *out_bytes = scratch_bytes(idx, idx->dev.cfg, n);
+    *out_bytes = scratch_bytes(idx, idx->dev.cfg, n, true);
     return HICOPS_OK;
 }
 
@@ -475,7 +477,7 @@ extern "C" hicops_status hicops_search_scratch(hicops_index* idx, const hicops_b
                                                uint64_t bytes, hicops_psm* out_psm, uint32_t* out_hist,
                                                uint32_t* out_nscored) {
     if (!idx) { set_error("NULL argument"); return HICOPS_EINVAL; }
-    return search_in_scratch(idx, b, idx->dev.cfg, scratch, bytes, out_psm, out_hist, out_nscored);
+    return search_in_scratch(idx, b, idx->dev.cfg, scratch, bytes, true, out_psm, out_hist, out_nscored);
 }
 
 struct hicops_plan {

@@ -120,7 +120,7 @@ namespace {
 uint64_t launch_bytes(const hicops_server* srv, uint32_t n, uint64_t npk) {
     return piece(8ull * (n + 1)) + 2 * piece(4 * npk) + 2 * piece(8ull * n) + piece(n) +
            piece(sizeof(hicops_psm) * (uint64_t)n * srv->k) + piece(4ull * n * hicops::kHistBins) + piece(4ull * n) +
-           hicops::scratch_bytes(srv->idx, srv->cfg, n);
+           hicops::scratch_bytes(srv->idx, srv->cfg, n, false);
 }
 
 hicops_status launch(hicops_server* srv, Lane& ln) {
@@ -177,7 +177,7 @@ hicops_status launch(hicops_server* srv, Lane& ln) {
     HC_CUDA(cudaMemcpyAsync(d_z, ln.h_z.p, n, cudaMemcpyHostToDevice, s));
     hicops_batch b{n, 1, d_off, d_mz, d_in, d_prec, d_z, d_tol, s};
     hicops_status st =
-        hicops::search_in_scratch(srv->idx, &b, srv->cfg, at, ln.bytes - used, d_psm, d_hist, d_ns);
+        hicops::search_in_scratch(srv->idx, &b, srv->cfg, at, ln.bytes - used, false, d_psm, d_hist, d_ns);
     if (st != HICOPS_OK) return st;
     HC_CUDA(cudaMemcpyAsync(ln.h_psm.p, d_psm, sizeof(hicops_psm) * n * srv->k, cudaMemcpyDeviceToHost, s));
     HC_CUDA(cudaMemcpyAsync(ln.h_hist.p, d_hist, sizeof(uint32_t) * n * hicops::kHistBins, cudaMemcpyDeviceToHost,

@@ -1,6 +1,7 @@
-"""Indexes on two devices in one process (host check: the library's objects against
-tests/fake_runtime.cpp): each device's search kernels are opted into its shared
-memory, and grids follow each device's number of SMs."""
+"""Host checks of the library's objects against a runtime of two devices that runs
+no kernels (tests/fake_runtime.cpp).  Indexes on two devices in one process: each
+device's search kernels are opted into its shared memory, and grids follow its
+number of SMs.  The server: requests that fill the pool exactly are taken."""
 import glob
 import os
 import shutil
@@ -13,7 +14,8 @@ from paper_2102_02286_gb300 import build as pkg_build
 ROOT = os.path.abspath(os.path.join(os.path.dirname(__file__), ".."))
 
 
-def test_searches_on_two_devices(tmp_path):
+@pytest.mark.parametrize("check", ["two_devices", "server_blocks"])
+def test_host_side(tmp_path, check):
     cxx = shutil.which("g++")
     if cxx is None:
         pytest.skip("no g++")
@@ -23,6 +25,6 @@ def test_searches_on_two_devices(tmp_path):
     exe = str(tmp_path / "fake_runtime")
     subprocess.run([cxx, "-O1", "-std=c++17", "-pthread", "-I", pkg_build.INCLUDE,
                     os.path.join(ROOT, "tests", "fake_runtime.cpp"), *objects, "-o", exe], check=True)
-    out = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    out = subprocess.run([exe, check], capture_output=True, text=True, timeout=60)
     assert out.returncode == 0, out.stdout + out.stderr
     assert out.stdout.strip() == "ok"
