@@ -14,6 +14,7 @@
 #include <memory>
 #include <functional>
 #include <numeric>
+#include <system_error>
 #include <thread>
 
 #include "hicops_internal.h"
@@ -87,21 +88,29 @@ unsigned n_threads() {
     return t ? std::min(t, 64u) : 4u;
 }
 
+// f(i, t) for every i below n, t the number of the thread that calls it (below
+// n_threads()).  The calling thread is one of them, and where the host gives no
+// more threads it does what they would.
 template <class F>
 void parallel_for(size_t n, F&& f) {
     const unsigned T = n_threads();
     std::atomic<size_t> next{0};
     const size_t grain = std::max<size_t>(1, n / (T * 16));
+    auto work = [&](unsigned t) {
+        for (;;) {
+            size_t a = next.fetch_add(grain);
+            if (a >= n) break;
+            size_t b = std::min(n, a + grain);
+            for (size_t i = a; i < b; ++i) f(i, t);
+        }
+    };
     std::vector<std::thread> th;
-    for (unsigned t = 0; t < T; ++t)
-        th.emplace_back([&, t] {
-            for (;;) {
-                size_t a = next.fetch_add(grain);
-                if (a >= n) break;
-                size_t b = std::min(n, a + grain);
-                for (size_t i = a; i < b; ++i) f(i, t);
-            }
-        });
+    th.reserve(T);
+    try {
+        while (th.size() + 1 < T) th.emplace_back(work, (unsigned)th.size());
+    } catch (const std::system_error&) {
+    }
+    work((unsigned)th.size());
     for (auto& x : th) x.join();
 }
 
