@@ -177,8 +177,12 @@ uint64_t grid_of(const hicops_index* idx, uint32_t ctas, uint64_t max_units) {
 template <int THREADS>
 hicops_status launch_search_p(const SearchArgs& sa, uint64_t grid, cudaStream_t s) {
     if (sa.stride <= THREADS) return launch_search_t<THREADS, 1>(sa, grid, s);
-    if (sa.stride <= 2 * THREADS) return launch_search_t<THREADS, 2>(sa, grid, s);
-    return launch_search_t<THREADS, 4>(sa, grid, s);
+    if constexpr (2 * THREADS >= kMaxTopN) {
+        return launch_search_t<THREADS, 2>(sa, grid, s);
+    } else {
+        if (sa.stride <= 2 * THREADS) return launch_search_t<THREADS, 2>(sa, grid, s);
+        return launch_search_t<THREADS, 4>(sa, grid, s);
+    }
 }
 
 hicops_status launch_search(const hicops_index* idx, SearchArgs& sa, const hicops_search_config& c, uint64_t max_units,
@@ -311,7 +315,7 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     plan_kernel<<<1, n <= kPlanFew ? kPlanFew : kPlanThreads, 0, s>>>(plan);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
-    SearchArgs sa{w.qbin, w.qiq, w.qn, n, query_bins_cap(p), w.unit,
+    SearchArgs sa{w.qbin, w.qiq, w.qn, query_bins_cap(p), w.unit,
                   from < INFINITY ? reinterpret_cast<const uint64_t*>(w.work + 1) : w.seg_off + n, di.bins, di.entry,
                   di.skip, di.skip_stride, di.hot_b, di.hot_y, di.hot_words, di.fwd_off, reinterpret_cast<const uint4*>(di.fwd), di.lf, di.ls,
                   (uint32_t)idx->s_max, p.min_shared, k, cfg.chunk_entries < 16 ? cfg.chunk_entries * 1024u : 0xffffffffu, w.utop, d_hist, d_ns, w.work,
@@ -417,7 +421,6 @@ hicops_status search_setup(hicops_index* idx) {
     HC_CUDA((allow_shared(search_kernel<384, 4>)));
     HC_CUDA((allow_shared(search_kernel<512, 1>)));
     HC_CUDA((allow_shared(search_kernel<512, 2>)));
-    HC_CUDA((allow_shared(search_kernel<512, 4>)));
     HC_CUDA((allow_shared(count_kernel<1>)));
     HC_CUDA((allow_shared(count_kernel<kMaxTopN / kCountThreads>)));
     return HICOPS_OK;

@@ -60,7 +60,6 @@ struct SearchArgs {
     const uint32_t* qbin;
     const uint32_t* qiq;
     const uint32_t* qn;
-    uint32_t n;
     uint32_t stride;            // qbin / qiq words per spectrum
     const uint4* unit;          // [units] the units in the order they are taken
     const uint64_t* n_units;    // their number
