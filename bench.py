@@ -171,9 +171,10 @@ def search_traffic_record():
 
 def search_source_hash() -> str:
     """sha256 over the sources that decide the search kernel's memory traffic:
-    the kernel itself, the index layout and its constants."""
+    the kernel itself, the planning and the cost that cut its units, the host
+    code that sizes its shared memory, the index layout and its constants."""
     h = hashlib.sha256()
-    for name in ("search_kernel.cuh", "hicops_internal.h", "index_build.cu"):
+    for name in ("search_kernel.cuh", "search_kernels.cuh", "search.cu", "hicops_internal.h", "index_build.cu"):
         with open(os.path.join(ROOT, "paper_2102_02286_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()
