@@ -466,10 +466,13 @@ hicops_status hicops_index_copy_csr(const hicops_index* index, uint64_t* off, ui
  * 384 or 512 (default 256 for up to 160 query bins a spectrum, else 384).
  * chunk_entries: index entries a CTA aims to read per pass over a range of
  * peptide ids, in units of 1024, 1..16 (default 16, which sets no such limit);
- * the range is sized from the spectrum's entry density.  ctas_per_sm: resident CTAs per
- * SM (0 = as many as fit).  seg_pids: a spectrum's precursor window is split
- * into work units of at least this many peptide ids (0 = split only when the
- * batch is too small to fill the GPU).  Results do not depend on the shape. */
+ * the range is sized from the spectrum's entry density.  Neither concerns the
+ * spectra whose peptides are counted one by one (min_shared 1 and 2, coarse
+ * grids).  ctas_per_sm: resident CTAs per SM (0 = as many as fit).  seg_pids: a
+ * spectrum's precursor window is cut into even work units of at most this many
+ * peptide ids, but into no more than 64 units (16 in hicops_search_noalloc);
+ * 0 = into pieces of like estimated cost, small enough to even out the CTAs'
+ * shares of the batch.  Results do not depend on the shape. */
 typedef struct hicops_search_config {
     uint32_t threads;
     uint32_t chunk_entries;
@@ -582,7 +585,7 @@ void hicops_server_destroy(hicops_server* srv);
  * HICOPS_EINVAL (not uploaded, timing not enabled), HICOPS_ECUDA. */
 typedef struct hicops_timing {
     float prep_ms;      /* preprocessing + precursor window */
-    float plan_ms;      /* work-unit planning (segments, scan) */
+    float plan_ms;      /* work-unit planning (segments and their order) */
     float search_ms;    /* shared-peak accumulation, scoring, top-k, histogram */
     float merge_ms;     /* top-k merge + e-value */
     float total_ms;     /* first to last kernel of the call */

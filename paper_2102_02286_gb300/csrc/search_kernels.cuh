@@ -12,7 +12,7 @@ namespace hicops {
 namespace {
 
 constexpr int kPrepThreads = 256;
-constexpr int kPrepWarps = kPrepThreads / 32;   // spectra per block of prep_kernel's first blocks
+constexpr int kPrepWarps = kPrepThreads / 32;   // spectra per block of prep_kernel's last blocks
 constexpr int kPrepWarpPeaks = 512;        // spectra with at most this many raw peaks: one warp each
 constexpr uint32_t kPrepBigBlocks = 608;   // blocks for the others, at most (4 an SM)
 constexpr int kMinSegPids = (int)kChunk;  // smallest segment of a split window
@@ -477,9 +477,9 @@ __device__ __forceinline__ void prep_warp(const PrepArgs& a, uint32_t q, uint64_
     put_window<32>(a, q, keys, keep, prec, tol, z, lane);
 }
 
-// Query preprocessing (R8) and the precursor window.  The first blocks take a
-// spectrum a warp, the others (big_blocks) a spectrum of more than
-// kPrepWarpPeaks raw peaks a block, found by all threads at once.
+// Query preprocessing (R8) and the precursor window.  The first big_blocks
+// blocks take the spectra of more than kPrepWarpPeaks raw peaks, one a block,
+// found by all threads at once; the others a spectrum a warp.
 __global__ void __launch_bounds__(kPrepThreads) prep_kernel(const __grid_constant__ PrepArgs a, uint32_t big_blocks) {
     __shared__ PrepShared sh;
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
