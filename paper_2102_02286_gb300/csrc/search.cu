@@ -8,7 +8,9 @@
 //                  filter_1 (a search of the mass-sorted database);
 //   plan_kernel    work units (spectrum, peptide-id segment), cut and ordered
 //                  by estimated cost;
-//   search_kernel  filter_2 + score + heap over persistent CTAs;
+//   search_kernel  filter_2 + score + heap over persistent CTAs, and
+//   count_kernel   the same for units in which many peptides qualify (only
+//                  where parameters or grid can make such units);
 //   merge_kernel   per-spectrum top-k merge and the survival-tail e-value.
 // hicops_search takes its scratch stream-ordered from its index's pool; a plan
 // (hicops_plan_*) allocates it once and can replay the sequence as a CUDA

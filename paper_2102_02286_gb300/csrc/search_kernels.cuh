@@ -1,6 +1,7 @@
 // Device kernels of the search path (included by search.cu only):
 // preprocessing + precursor window, unit planning, the shared-peak search
-// kernel (search_kernel.cuh), the top-k merge + e-value, and the work count.
+// kernels (search_kernel.cuh, count_kernel.cuh), the top-k merge + e-value, and
+// the work count.
 #pragma once
 
 #include <cfloat>
@@ -546,7 +547,7 @@ constexpr uint32_t kUnitCost = 128, kUnitCostMin = 16;   // 8,192 and 1,024 entr
 // The planning of a batch in one block: the spectra's units, their prefix, and
 // the unit records, costliest first, since the persistent CTAs take them in
 // this order and the cheap ones fill the end of the launch (a counting sort
-// over quarter octaves of the unit's cost).  One block, since a grid's scan and
+// over quarter octaves of the unit's cost), and the counted ones behind.  One block, since a grid's scan and
 // sort take seven launches: bound by latency, 7 us for a few spectra, 17 us for
 // 5,000 (38 us by seven launches), 58 us for 30,000 (38 us).
 constexpr uint32_t kPlanThreads = 1024, kPlanFew = 128;   // up to kPlanFew spectra: as many threads
