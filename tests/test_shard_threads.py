@@ -34,7 +34,9 @@ def test_parts_without_more_threads():
     pkg_build.build()
 
     def stacks():                            # of 128 MB, which no cache of ended threads keeps
-        resource.setrlimit(resource.RLIMIT_STACK, (128 << 20, resource.getrlimit(resource.RLIMIT_STACK)[1]))
+        hard = resource.getrlimit(resource.RLIMIT_STACK)[1]
+        soft = 128 << 20 if hard == resource.RLIM_INFINITY else min(128 << 20, hard)
+        resource.setrlimit(resource.RLIMIT_STACK, (soft, hard))
 
     r = subprocess.run([sys.executable, "-c", CHILD, ROOT], capture_output=True, text=True, timeout=300, preexec_fn=stacks)
     assert r.returncode == 0, (r.returncode, r.stdout, r.stderr[-2000:])
