@@ -13,22 +13,30 @@
 // units behind the others.
 //
 // A column's counters are 64 KB: three CTAs an SM of 256 threads (of 384 threads
-// the same; two of 512: 2.4 against 2.1 ms).  What bounds it: the latencies of a
-// column's passes, about 3 us where few entries lie in it, and the issue of both
-// passes.  13.0 M peptides, 500 spectra of 100 peaks at +-500 Da, scored from an
-// entry log / from forward lists / here: min_shared 1 7.5 / 53 / 4.5 ms, 2 2.2 /
-// 6.4 / 2.1 ms; 50 spectra on a grid of 1 Da, min_shared 4, 2.3 / 12.8 / 0.9 ms.
+// the same; two of 512: 2.4 against 2.1 ms).  Where there are units of both
+// kinds, its CTAs start as search_kernel's leave their SMs, so that one's last
+// units run beside the other's first (500 spectra at min_shared 2: 2.1 -> 1.8 ms).
+// What bounds it: the latencies of a column's passes, about 3 us where few
+// entries lie in it, and the issue of both passes.  13.0 M peptides, 500 spectra
+// of 100 peaks at +-500 Da, scored from an entry log / from forward lists / here:
+// min_shared 1 7.5 / 53 / 4.4 ms, 2 2.2 / 6.4 / 1.8 ms; 50 spectra on a grid of
+// 1 Da, min_shared 4, 2.3 / 12.8 / 0.9 ms.
 
-// Expected hits a peptide from which on a spectrum's units are counted.  With
-// min_shared 2, from 0 / 0.02 / 0.05 / 0.08 on: 500 spectra of 100 peaks 1.9 /
-// 2.1 / 2.7 / 3.1 ms, 2,000 of 10 peaks 3.0 / 1.0 / 0.8 / 0.9 ms.  Above it from
-// where a column's repeats come near the table's size, or with min_shared 3 the
-// peptides to score do.  200 spectra of 100 peaks from forward lists / counted:
-// on a grid of 0.1 Da (0.16 hits) min_shared 3 3.2 / 1.3 ms, 4 1.27 / 1.19, 6
-// 0.63 / 1.13; of 0.2 Da (0.32) min_shared 4 6.3 / 2.6 ms.
-constexpr float kCountShare2 = 0.02f;
-constexpr float kCountShare3 = 0.13f;
-constexpr float kCountShare = 0.30f;
+// Expected hits a peptide from which on a spectrum's units are counted.
+// min_shared 2, from 0.02 / 0.04 / 0.05 / 0.08 on: 500 spectra of 100 peaks 1.89 /
+// 1.79 / 1.74 / 2.20 ms, of 20 peaks 0.52 / 0.55 / 0.76 / 0.79, 2,000 of 10 peaks
+// 0.94 / 0.79 / 0.75 / 0.73.  min_shared 3, from 0.13 / 0.17 / 0.21 / 0.27 on: 300 of
+// 275 peaks on a grid of 0.02 Da 1.57 / 1.32 / 1.50 / 1.48, 200 of 100 peaks on 0.1 Da
+// 1.31 / 1.49 / 1.59 / 1.79.  Above, from 0.20 / 0.25 / 0.30 on, 200 of 100 peaks: 0.1 Da
+// and min_shared 6 0.87 / 0.64 / 0.64, 0.2 Da and 4 1.44 / 1.44 / 1.67, 6 1.26 / 1.26 /
+// 2.25.
+constexpr float kCountShare2 = 0.04f;
+constexpr float kCountShare3 = 0.19f;
+constexpr float kCountShare = 0.25f;
+// With min_shared 3 and above it, only indexes whose average spectrum has this
+// many are looked at (count_from): the call is spared a launch for the others.
+constexpr float kCountGrid3 = 0.09f;
+constexpr float kCountGrid = 0.18f;
 constexpr uint32_t kLook = 32;             // counters a lane looks at together
 
 struct CountLayout {
@@ -354,4 +362,6 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) count_kernel(const 
         unit_out<THREADS>(a, sh, tkey, tpid, tpk, u.x, u.w);
         if (tid == 0) set_unit(t_next);
     }
+    // the search that this kernel may have started beside has ended before this one does
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -204,18 +204,18 @@ hicops_status launch_search(const hicops_index* idx, SearchArgs& sa, const hicop
 }
 
 // Which units are counted peptide by peptide (count_kernel.cuh): those of
-// spectra of at least this many expected hits a peptide.  No spectrum of a grid
-// whose average one has under two thirds of that: a call whose units are
-// all of one kind is spared the other's launch, and search_kernel falls back to
-// counters by itself where a single column's repeats overflow.
+// spectra of at least this many expected hits a peptide.  None on a grid whose
+// average spectrum has far fewer; search_kernel falls back to counters by itself
+// where a single column's repeats overflow.
 float count_from(const hicops_index* idx) {
     const hicops_params& p = idx->p;
     if (p.min_shared < 2) return 0.0f;
     if (p.min_shared == 2) return kCountShare2;
-    const float share = p.min_shared == 3 ? kCountShare3 : kCountShare;
     const double ions = (double)idx->stats.n_entries / std::max<double>(1.0, (double)idx->mass.size());
     const double grid = (p.frag_mz_max - p.frag_mz_min) / p.bin_width_da;
-    return query_bins_cap(p) * ions / grid > share * 2 / 3 ? share : INFINITY;
+    const double average = query_bins_cap(p) * ions / grid;
+    if (p.min_shared == 3) return average > kCountGrid3 ? kCountShare3 : INFINITY;
+    return average > kCountGrid ? kCountShare : INFINITY;
 }
 
 CountLayout make_count_layout(uint32_t stride, uint32_t k) {
@@ -237,23 +237,34 @@ CountLayout make_count_layout(uint32_t stride, uint32_t k) {
     return l;
 }
 
+// Behind a search_kernel its CTAs start as that one's leave their SMs (both only
+// read what the planner wrote, and the count ends behind the search).
 template <int PPT>
-hicops_status launch_count_t(const CountArgs& ca, uint64_t grid, cudaStream_t s) {
-    count_kernel<PPT><<<(unsigned)grid, kCountThreads, sizeof(uint32_t) * ca.lay.end, s>>>(ca);
+hicops_status launch_count_t(const CountArgs& ca, uint64_t grid, bool behind, cudaStream_t s) {
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3(kCountThreads);
+    c.dynamicSmemBytes = sizeof(uint32_t) * ca.lay.end;
+    c.stream = s;
+    c.attrs = &early;
+    c.numAttrs = behind ? 1 : 0;
+    HC_CUDA(cudaLaunchKernelEx(&c, count_kernel<PPT>, ca));
     count_launches(1);
-    HC_CUDA(cudaGetLastError());
     return HICOPS_OK;
 }
 
 hicops_status launch_count(const hicops_index* idx, CountArgs& ca, const hicops_search_config& c, uint64_t max_units,
-                           cudaStream_t s) {
+                           bool behind, cudaStream_t s) {
     ca.lay = make_count_layout(ca.stride, ca.k);
     // (the largest, 1,024 bins and 32 rows, takes 104 KB: two CTAs an SM)
     uint32_t ctas = std::min<uint32_t>(kCountCtas, kSmemPerSm / (4 * ca.lay.end + 1024));
     if (c.ctas_per_sm && c.ctas_per_sm < ctas) ctas = c.ctas_per_sm;
     const uint64_t grid = grid_of(idx, ctas, max_units);
-    if (ca.stride <= kCountThreads) return launch_count_t<1>(ca, grid, s);
-    return launch_count_t<kMaxTopN / kCountThreads>(ca, grid, s);
+    if (ca.stride <= kCountThreads) return launch_count_t<1>(ca, grid, behind, s);
+    return launch_count_t<kMaxTopN / kCountThreads>(ca, grid, behind, s);
 }
 
 inline void mark(hicops_index* idx, int i, cudaStream_t s, bool on) {
@@ -329,7 +340,7 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
         CountArgs ca{w.qbin, w.qiq, w.qn, query_bins_cap(p), w.unit, w.work + 1, w.seg_off + n, di.bins, di.entry, di.skip,
                      di.skip_stride, di.lf, di.ls, (uint32_t)idx->s_max, p.min_shared, k, w.utop, d_hist, d_ns, w.work + 2,
                      CountLayout{}};
-        st = launch_count(idx, ca, cfg, max_units, s);
+        st = launch_count(idx, ca, cfg, max_units, from > 0.0f, s);
     }
     if (st != HICOPS_OK) return st;
     mark(idx, 3, s, timing_marks);

@@ -626,6 +626,8 @@ __global__ void __launch_bounds__(THREADS, search_min_ctas(THREADS)) search_kern
     const SearchParts sp = search_parts(a.lay);
     uint32_t* const plane = sp.plane;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // (a count_kernel behind this one may start where CTAs of this one have ended)
+    asm volatile("griddepcontrol.launch_dependents;");
     for (uint32_t i = tid; i < a.lay.plane_words; i += THREADS) plane[i] = 0u;
     for (uint32_t i = tid; i < kSlots; i += THREADS) sp.tab[i] = 0u;
     for (uint32_t i = tid; i < kPlane2Words; i += THREADS) sp.plane2[i] = 0u;

@@ -88,6 +88,15 @@ int __cudaLaunchKernel(const void* f, Dim3 grid, Dim3, void**, size_t smem, void
     if (grid.x > g_grid[g_device]) g_grid[g_device] = grid.x;
     return 0;
 }
+struct LaunchConfig {
+    Dim3 grid, block;
+    size_t smem;
+    void *stream, *attrs;
+    unsigned n_attrs;
+};
+int cudaLaunchKernelExC(const LaunchConfig* c, const void* f, void** args) {
+    return __cudaLaunchKernel(f, c->grid, c->block, args, c->smem, c->stream);
+}
 void** __cudaRegisterFatBinary(void*) { static void* handle; return &handle; }
 void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}

@@ -53,3 +53,17 @@ def test_counted_units(oracle_lib, name):
         assert hc.kernel_launches() - before == launches
         assert_parity(got, ref, label=f"{name}, pieces of {seg}")
     assert int(ref.n_scored.sum()) > 0
+    # the same launches captured and replayed, one after another on a stream
+    idx.set_config(None)
+    plan, stream = idx.plan(spec.n), torch.cuda.Stream()
+    batch, out = hc.DeviceBatch.from_spectra(spec), hc.DeviceResult.alloc(spec.n, w.params.top_k)
+    torch.cuda.synchronize()
+    for graph in (False, True, True, True):
+        out.psm.zero_()
+        out.hist.zero_()
+        torch.cuda.synchronize()
+        for _ in range(3):
+            plan.search(batch, out, stream, graph=graph)
+        torch.cuda.synchronize()
+        assert_parity(out.to_host(spec.n, w.params.top_k), ref, label=f"{name}, plan, graph {graph}")
+    plan.close()
