@@ -323,9 +323,10 @@ hicops_status enqueue_search(hicops_index* idx, const DevBatch& d, uint32_t n, c
     const float from = count_from(idx);      // counted units: some may be, all are
     const uint32_t split = unit_limit(idx, cfg, n).split;
     const PlanArgs plan{w.lo, w.hi, w.cost, n, w.max_seg, cfg.seg_pids, split,
-                        split / kSplitPerSm * (uint32_t)search_min_ctas((int)cfg.threads), w.seg_off, w.unit, w.work,
-                        from < INFINITY};
-    plan_kernel<<<1, n <= kPlanFew ? kPlanFew : kPlanThreads, 0, s>>>(plan);
+                        split / kSplitPerSm * (uint32_t)search_min_ctas((int)cfg.threads), w.seg_off, w.unit, w.work};
+    const uint32_t threads = n <= kPlanFew ? kPlanFew : kPlanThreads;
+    if (from < INFINITY) plan_kernel<true><<<1, threads, 0, s>>>(plan);
+    else plan_kernel<false><<<1, threads, 0, s>>>(plan);
     count_launches(1);
     HC_CUDA(cudaGetLastError());
     SearchArgs sa{w.qbin, w.qiq, w.qn, query_bins_cap(p), w.unit,

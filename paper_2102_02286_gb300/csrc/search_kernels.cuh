@@ -540,7 +540,6 @@ struct PlanArgs {
     uint4* unit;
     unsigned long long* work;    // the unit counters of the search (0) and of the count (2), set to zero; where
                                  // the counted units start (1)
-    uint32_t counts;             // there may be counted units: they come behind the others
 };
 constexpr uint32_t kUnitCost = 128, kUnitCostMin = 16;   // 8,192 and 1,024 entries
 
@@ -553,13 +552,15 @@ constexpr uint32_t kUnitCost = 128, kUnitCostMin = 16;   // 8,192 and 1,024 entr
 constexpr uint32_t kPlanThreads = 1024, kPlanFew = 128;   // up to kPlanFew spectra: as many threads
 constexpr uint32_t kPlanEach = 4;          // consecutive spectra of a thread
 constexpr uint32_t kPlanBuckets = 512;     // a quarter octave of cost, four times (lanes that are alike spread over them)
+// COUNTS: there may be counted units.
+template <bool COUNTS>
 __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constant__ PlanArgs a) {
-    __shared__ __align__(16) uint32_t bucket[2 * kPlanBuckets];     // of the units, then of the counted ones
+    constexpr uint32_t kBuckets = (COUNTS ? 2u : 1u) * kPlanBuckets;     // of the units, then of the counted ones
+    __shared__ __align__(16) uint32_t bucket[kBuckets];
     __shared__ unsigned long long csum[kPlanThreads / 32];
     __shared__ uint32_t wsum[kPlanThreads / 32];
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const uint32_t step = blockDim.x * kPlanEach;
-    const uint32_t halves = a.counts ? 2u : 1u;
     uint32_t lo[kPlanEach], hi[kPlanEach], cost[kPlanEach];
     // (a piece of the workspace is a whole number of 256 bytes (pieces.h): whole vectors, whose words behind n
     // are left)
@@ -579,15 +580,16 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     };
     // the batch's cost
     fetch(tid * kPlanEach);
-    auto bare = [](uint32_t c) { return (unsigned long long)(c & ~kCounted); };
-    unsigned long long sum = bare(cost[0]) + bare(cost[1]) + bare(cost[2]) + bare(cost[3]);
+    auto bare = [](uint32_t c) { return COUNTS ? c & ~kCounted : c; };
+    unsigned long long sum = (unsigned long long)bare(cost[0]) + bare(cost[1]) + bare(cost[2]) + bare(cost[3]);
 #pragma unroll 8
     for (uint32_t q = step + tid; q < a.n; q += blockDim.x) sum += bare(a.cost[q]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (lane == 0) csum[warp] = sum;
-    for (uint32_t i = tid; i < halves * kPlanBuckets; i += blockDim.x) bucket[i] = 0;
-    if (tid == 0) a.work[0] = a.work[2] = 0ull;
+    for (uint32_t i = tid; i < kBuckets; i += blockDim.x) bucket[i] = 0;
+    if (tid == 0) a.work[0] = 0ull;
+    if (COUNTS && tid == 0) a.work[2] = 0ull;
     __syncthreads();
     sum = lane < nwarps ? csum[lane] : 0ull;
 #pragma unroll
@@ -601,7 +603,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     auto cut = [&]() {
 #pragma unroll
         for (uint32_t i = 0; i < kPlanEach; ++i) {
-            const uint32_t c = cost[i] & ~kCounted, W = hi[i] - lo[i];
+            const uint32_t c = bare(cost[i]), W = hi[i] - lo[i];
             uint32_t k = 0;
             if (c) {
                 if (a.seg_pids) k = W / a.seg_pids + (W % a.seg_pids ? 1u : 0u);
@@ -611,8 +613,8 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
             }
             ns[i] = k;
             const int b = (int)(__float_as_uint(__fdividef((float)c, (float)max(k, 1u))) >> 21) - (int)(0x3f800000u >> 21);
-            at[i] = 4u * (kPlanBuckets / 4u - 1u - (uint32_t)min(max(b, 0), (int)kPlanBuckets / 4 - 1)) + (lane & 3u) +
-                    (cost[i] & kCounted ? kPlanBuckets : 0u);
+            at[i] = 4u * (kPlanBuckets / 4u - 1u - (uint32_t)min(max(b, 0), (int)kPlanBuckets / 4 - 1)) + (lane & 3u);
+            if (COUNTS && (cost[i] & kCounted)) at[i] += kPlanBuckets;
         }
     };
     uint64_t base = 0, u0 = 0;      // units of the steps before; this thread's first unit of the last step
@@ -650,9 +652,9 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(const __grid_constan
     // bucket counts to starts (the last barrier is behind every count)
     if (warp == 0) {
         uint32_t start = 0;
-#pragma unroll 4
-        for (uint32_t i = lane; i < halves * kPlanBuckets / 4; i += 32) {
-            if (i == kPlanBuckets / 4) a.work[1] = start;
+#pragma unroll
+        for (uint32_t i = lane; i < kBuckets / 4; i += 32) {
+            if (COUNTS && i == kPlanBuckets / 4) a.work[1] = start;
             const uint4 c = reinterpret_cast<const uint4*>(bucket)[i];
             const uint32_t mine = c.x + c.y + c.z + c.w;
             uint32_t incl = mine;
